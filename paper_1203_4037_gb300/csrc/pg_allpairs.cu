@@ -185,7 +185,7 @@ __global__ void __launch_bounds__(kNT, MinBlocks<NP, TABLE, DF>::value) k_allpai
     const long long G = gridDim.x;
     const long long b = blockIdx.x;
     const long long u0 = b * a.W / G, u1 = (b + 1) * a.W / G;
-    if (u0 >= u1) return;
+    if (u0 >= u1 || (TABLE && a.skip && *a.skip)) return;
 
     if (tid == 0) {
         mbar_init(&bar[0], 1);
@@ -562,7 +562,14 @@ __global__ void k_combine(CombineArgs c)
     long long t = p / c.Bi;
     int li = (int)(p % c.Bi);
     double ax = 0, ay = 0, az = 0, ph = 0;
-    if (c.njsub > 0) {
+    if (c.start && *c.near) {
+        for (long long b = plan_first(c.start, c.near_grid, t * c.nch);
+             b < c.near_grid && c.start[b] < (t + 1) * c.nch; ++b) {
+            if (c.start[b + 1] <= c.start[b]) continue;
+            const double4 v = c.part[(size_t)(t + b) * c.Bi + li];
+            ax += v.x; ay += v.y; az += v.z; ph += v.w;
+        }
+    } else if (c.njsub > 0) {
         long long bf = stream_k_owner(t * c.njsub, c.grid, c.W);
         long long bl = stream_k_owner((t + 1) * c.njsub - 1, c.grid, c.W);
         for (long long s = 0; s <= bl - bf; ++s) {
@@ -628,7 +635,7 @@ __global__ void __launch_bounds__(kWideThreads) k_combine_wide(CombineArgs c)
 cudaError_t launch_combine(const CombineArgs &c, cudaStream_t st)
 {
     if (c.ni <= 0) return cudaSuccess;
-    if (c.smax_slots >= 32)
+    if (c.smax_slots >= 32 && !c.start)
         k_combine_wide<<<(unsigned)c.ni, kWideThreads, 0, st>>>(c);
     else
         k_combine<<<(unsigned)((c.ni + 255) / 256), 256, 0, st>>>(c);

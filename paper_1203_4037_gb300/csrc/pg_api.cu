@@ -73,6 +73,10 @@ struct pg_ctx {
 
     // tiles and ordering
     DevBuf xt, ctr;
+    // table on compact tiles: half extents of the tiles, FP32 j records, the
+    // tiles' costs and density flags, and the CTAs' first units
+    DevBuf t_ext, j_f32, t_cost, t_dense, t_start;
+    bool tiled_ext = false;       // the current tiles have their extents
     SortScratch sort{};
     DevBuf skeys0, skeys1, svals0, svals1, shist, ssums, sbbox;
     unsigned *perm = nullptr;     // tile order -> i index (nullptr: identity)
@@ -505,7 +509,7 @@ void pg_destroy(pg_ctx *c)
                       &c->c_wrapped, &c->c_xs, &c->c_xo, &c->c_perm, &c->c_start, &c->c_jcount,
                       &c->c_icount, &c->c_ioff,
                       &c->c_items_raw, &c->c_items, &c->c_pairs, &c->n_part, &c->bw_wj,
-                      &c->bw_wt, &c->bw_dv, &c->tickets};
+                      &c->bw_wt, &c->bw_dv, &c->tickets, &c->t_ext, &c->j_f32, &c->t_cost, &c->t_dense, &c->t_start};
     for (DevBuf *b : bufs) free_dev(*b);
     for (DevBuf &b : c->tb) free_dev(b);
     for (DevBuf *b : {&c->pm_rec, &c->pm_x, &c->pm_m, &c->pm_acc, &c->pm_pot}) free_dev(*b);
@@ -1232,6 +1236,13 @@ bool tiled_df(const pg_ctx *c, long long ni, long long nj)
     return c->mode == PG_TABLE || !tiles_sorted(c, ni) || nj > 8 * ni;
 }
 
+// The tabulated force is exactly 0 from r_cut on, so compact (sorted) tiles
+// evaluate only the j within r_cut of their box (pg_near.cu).
+// Clocks of one kept record against a warp's run, for the split: per i-pair
+// of a thread in the forward kernel, and in the backward kernel.
+constexpr float kNearPairCost = 215.0f, kNearBackCost = 670.0f;
+bool tiled_cull(const pg_ctx *c, long long ni) { return c->mode == PG_TABLE && tiles_sorted(c, ni); }
+
 // the narrow path's i chunks are the caller's i-particles in the caller's
 // order, as spread as they come: double-float unless single is asked for
 bool narrow_df(const pg_ctx *c) { return c->diff_mode != PG_DIFF_SINGLE; }
@@ -1251,7 +1262,9 @@ int plan_allpairs(pg_ctx *c, Plan &p)
 {
     p.ni = c->ni;
     p.nj = nj_of(c);
-    p.np = c->np ? c->np : auto_np(p.ni);
+    // near-pair runs: smaller tiles keep fewer j (65536 Plummer, r_cut = 0.1:
+    // np 1, 2, 4 take 0.45, 0.42, 0.49 ms; 262144: 2.88, 2.71, 3.27)
+    p.np = c->np ? c->np : tiled_cull(c, p.ni) ? 2 : auto_np(p.ni);
     p.Bi = allpairs_bi(p.np);
     p.ntiles = (int)((p.ni + p.Bi - 1) / p.Bi);
     p.njsub = (int)((p.nj + kTJ - 1) / kTJ);
@@ -1279,6 +1292,8 @@ int enqueue_tiles(pg_ctx *c, const Plan &p)
     if ((rc = ensure(c, c->xt, (size_t)std::max<long long>(n, 1) * sizeof(double4))) ||
         (rc = ensure(c, c->ctr, (size_t)std::max(p.ntiles, 1) * sizeof(double4))))
         return rc;
+    const bool ext = tiled_cull(c, n);
+    if (ext && (rc = ensure(c, c->t_ext, (size_t)std::max(p.ntiles, 1) * sizeof(float4)))) return rc;
     bool do_sort = tiles_sorted(c, n);
     c->perm = nullptr;
     if (do_sort && n > 1) {
@@ -1300,9 +1315,10 @@ int enqueue_tiles(pg_ctx *c, const Plan &p)
         c->last_launches += 3 + 5 * 4;
     }
     PG_CUDA(c, launch_tile_prep((const double4 *)c->xi.p, c->perm, n, p.Bi, (double4 *)c->xt.p,
-                                (double4 *)c->ctr.p, c->stream));
+                                (double4 *)c->ctr.p, c->stream, ext ? (float4 *)c->t_ext.p : nullptr));
     c->last_launches += 1;
     c->tiled_np = p.np;
+    c->tiled_ext = ext;
     return PG_OK;
 }
 
@@ -1383,18 +1399,77 @@ int enqueue_small(pg_ctx *c, const Plan &p, int nchunk, int jchunk, double *acc,
     return PG_OK;
 }
 
+// j records per unit: long units hide their latency, but a CTA should get a
+// dozen of them for the split to balance
+int near_unit(int ntiles, long long nj, int grid)
+{
+    int unit = kNearJ;
+    while (unit > kNearJ / 4 && (long long)ntiles * ((nj + unit - 1) / unit) < 12LL * grid) unit /= 2;
+    return unit;
+}
+
+// the table's near-pair runs (pg_near.cu): the FP32 j records, the tiles'
+// extents (in t_ext already) and the split of the units by cost
+int near_args(pg_ctx *c, NearArgs &a, const double4 *xt, const double4 *jrec, long long ni, long long nj, int Bi,
+              int run, float pair_cost, int grid)
+{
+    int rc;
+    const int ntiles = (int)((ni + Bi - 1) / Bi);
+    a.unit = near_unit(ntiles, nj, grid);
+    if ((rc = ensure(c, c->j_f32, (size_t)nj * sizeof(float4))) ||
+        (rc = ensure(c, c->t_cost, (size_t)ntiles * sizeof(unsigned))) || (rc = ensure(c, c->t_dense, ntiles)) ||
+        (rc = ensure(c, c->t_start, (size_t)(grid + 2) * sizeof(long long))) ||
+        (rc = ensure(c, c->part, ((size_t)ntiles + grid) * Bi * sizeof(double4))))
+        return rc;
+    PG_CUDA(c, launch_pack_f32(jrec, nj, (float4 *)c->j_f32.p, c->stream));
+    a.xi = xt;
+    a.ctr = (const double4 *)c->ctr.p;
+    a.ext = (const float4 *)c->t_ext.p;
+    a.jrec = jrec;
+    a.jf = (const float4 *)c->j_f32.p;
+    a.ni = ni;
+    a.nj = nj;
+    a.ntiles = ntiles;
+    a.nch = (int)((nj + a.unit - 1) / a.unit);
+    a.sstride = near_stride(a.nch);
+    a.start = (const long long *)c->t_start.p;
+    a.dense = (const unsigned char *)c->t_dense.p;
+    int *near = (int *)((long long *)c->t_start.p + grid + 1);
+    a.near = near;
+    a.r_cut = (float)c->r_cut;
+    a.tab = table_dev(c);
+    a.part = (double4 *)c->part.p;
+    a.status = (int *)c->status.p;
+    PG_CUDA(c, launch_near_plan(a, Bi, run, pair_cost, 1500.0f, grid, (unsigned *)c->t_cost.p,
+                                (unsigned char *)c->t_dense.p, (long long *)c->t_start.p, near, c->stream));
+    c->last_launches += 3;
+    return PG_OK;
+}
+
 int enqueue_allpairs(pg_ctx *c, const Plan &p, double *acc, double *pot)
 {
     int rc;
     bool table = c->mode == PG_TABLE;
     int nchunk = 0, jchunk = 0;
     if (use_small(c, p, nchunk, jchunk)) return enqueue_small(c, p, nchunk, jchunk, acc, pot);
-    if (p.ni > 0 && (c->i_dirty || c->use_graph || c->tiled_np != p.np)) {
+    const bool cull = tiled_cull(c, p.ni);
+    if (p.ni > 0 && (c->i_dirty || c->use_graph || c->tiled_np != p.np || (cull && !c->tiled_ext))) {
         if ((rc = enqueue_tiles(c, p))) return rc;
         c->i_dirty = false;
     }
     if (p.ni == 0) return PG_OK;
+    const bool ext = use_ext(c);
+    const bool near = cull && p.nj > 0;
+    NearArgs na{};
+    int ngrid = 0;
     if ((rc = ensure(c, c->part, (size_t)p.ntiles * p.slots * p.Bi * sizeof(double4)))) return rc;
+    if (near) {
+        const int occ = near_max_blocks_per_sm(p.np, tab_units(c), ext, p.df);
+        ngrid = c->sms * (c->ctas_per_sm > 0 ? std::min(c->ctas_per_sm, occ) : occ);
+        if ((rc = near_args(c, na, (const double4 *)c->xt.p, (const double4 *)c->jrec.p, p.ni, p.nj, p.Bi, 64 * p.np,
+                            kNearPairCost * p.np, ngrid)))
+            return rc;
+    }
     AllPairsArgs a{};
     a.xi = (const double4 *)c->xt.p;
     a.ctr = (const double4 *)c->ctr.p;
@@ -1405,6 +1480,7 @@ int enqueue_allpairs(pg_ctx *c, const Plan &p, double *acc, double *pot)
             return rc;
         a.jhl = (const float4 *)c->g_jhl.p;
     }
+    a.skip = na.near;
     a.ni = p.ni;
     a.nj = p.nj;
     a.ntiles = p.ntiles;
@@ -1415,19 +1491,22 @@ int enqueue_allpairs(pg_ctx *c, const Plan &p, double *acc, double *pot)
     if (table) a.tab = table_dev(c);
     a.part = (double4 *)c->part.p;
     a.status = (int *)c->status.p;
-    const bool ext = use_ext(c);
     size_t smem = allpairs_smem(p.np, table, tab_units(c), ext, p.df);
     c->last_np = p.np;
     c->last_df = p.df;
     if (p.grid > 0) {
         if (c->timing) PG_CUDA(c, record_timing(c, c->tk0));
+        if (near) {
+            PG_CUDA(c, launch_near(na, ngrid, p.np, ext, p.df, near_smem(p.np, tab_units(c), ext, p.df), c->stream));
+            c->last_launches += 1;
+        }
         PG_CUDA(c, launch_allpairs(a, p.grid, p.np, table, ext, c->packed != 0, p.df, smem, c->stream));
         if (c->timing) PG_CUDA(c, record_timing(c, c->tk1));
         c->timed = c->timing;
         c->last_launches += 1;
     }
     CombineArgs cb{};
-    cb.part = a.part;
+    cb.part = (const double4 *)c->part.p;
     cb.perm = c->perm;
     cb.jrec = a.jrec;
     cb.ni = p.ni;
@@ -1436,6 +1515,10 @@ int enqueue_allpairs(pg_ctx *c, const Plan &p, double *acc, double *pot)
     cb.smax_slots = p.slots;
     cb.grid = std::max(p.grid, 1);
     cb.W = std::max<long long>(p.W, 1);
+    cb.start = na.start;
+    cb.near = na.near;
+    cb.nch = na.nch;
+    cb.near_grid = ngrid;
     cb.self = c->self;
     cb.self_off = c->self_off;
     combine_ext(c, cb);
@@ -2520,8 +2603,10 @@ int pg_backward_dev(pg_ctx *c, const double *w, double *dx, double *dm, float *d
         c->last_launches += 3 + 5 * 4;
     }
     c->i_dirty = true;      // the tile buffers now hold the backward's order
+    const bool cull = table && n >= 16384;
+    if (cull && (rc = ensure(c, c->t_ext, ntiles * sizeof(float4)))) return rc;
     PG_CUDA(c, launch_tile_prep((const double4 *)c->jrec.p, c->perm, n, Bi, (double4 *)c->xt.p,
-                                (double4 *)c->ctr.p, c->stream));
+                                (double4 *)c->ctr.p, c->stream, cull ? (float4 *)c->t_ext.p : nullptr));
     PG_CUDA(c, launch_pack_w(w, c->perm, n, (double4 *)c->bw_wj.p, (double4 *)c->bw_wt.p, c->stream));
     if (table && dv) PG_CUDA(c, cudaMemsetAsync(c->bw_dv.p, 0, c->ntab * sizeof(double), c->stream));
     BackwardArgs a{};
@@ -2544,13 +2629,33 @@ int pg_backward_dev(pg_ctx *c, const double *w, double *dx, double *dm, float *d
     a.dv = (table && dv) ? (double *)c->bw_dv.p : nullptr;
     a.perm = c->perm;
     a.status = (int *)c->status.p;
+    NearArgs na{};
+    NearCombine nc;
+    if (cull) {
+        const int nocc = near_backward_max_blocks_per_sm(c->ntab);
+        const int ngrid = c->sms * (c->ctas_per_sm > 0 ? std::min(c->ctas_per_sm, nocc) : nocc);
+        if ((rc = near_args(c, na, a.xi, a.jx, n, n, Bi, Bi / 4, kNearBackCost, ngrid))) return rc;
+        a.skip = na.near;
+        nc.start = na.start;
+        nc.near = na.near;
+        nc.nch = na.nch;
+        nc.grid = ngrid;
+        na.wi = a.wv;
+        na.jw = a.jwv;
+        na.dv = a.dv;
+        a.part = na.part;
+    }
     if (c->timing) PG_CUDA(c, record_timing(c, c->tk0));
+    if (cull) {
+        PG_CUDA(c, launch_near_backward(na, nc.grid, near_backward_smem(c->ntab), c->stream));
+        c->last_launches += 1;
+    }
     PG_CUDA(c, launch_backward(a, grid, table, backward_smem(table, c->ntab), c->stream));
     if (c->timing) PG_CUDA(c, record_timing(c, c->tk1));
     c->timed = c->timing;
     double inv = table ? 1.0 / c->scale : 1.0;
     PG_CUDA(c, launch_backward_combine(a.part, c->perm, n, njsub, slots, grid, W, inv, dx, dm,
-                                       c->stream));
+                                       c->stream, nc));
     if (table && dv) PG_CUDA(c, launch_dv_out((const double *)c->bw_dv.p, c->ntab, inv, dv, c->stream));
     c->last_launches += 5;
     c->last_pairs = n * n;

@@ -24,7 +24,7 @@
 
 namespace pg {
 
-constexpr int kKI = 4;                      // i per thread
+constexpr int kKI = kBwKI;                  // i per thread
 constexpr float kFltMinNormal = 1.17549435e-38f;   // smallest normal FP32
 constexpr int kBiB = kNT * kKI;
 
@@ -62,7 +62,7 @@ __global__ void __launch_bounds__(kNT) k_backward_table(BackwardArgs a)
     const int tid = threadIdx.x;
     const long long G = gridDim.x, b = blockIdx.x;
     const long long u0 = b * a.W / G, u1 = (b + 1) * a.W / G;
-    if (u0 >= u1) return;
+    if (u0 >= u1 || (a.skip && *a.skip)) return;
 
     if (tid == 0) {
         mbar_init(&bar[0], 1);
@@ -545,14 +545,22 @@ cudaError_t launch_pack_w(const double *w, const unsigned *perm, long long n, do
 
 __global__ void k_bw_combine(const double4 *__restrict__ part, const unsigned *__restrict__ perm,
                              long long n, int njsub, int slots, int grid, long long W, double mscale,
-                             double *__restrict__ dx, double *__restrict__ dm)
+                             double *__restrict__ dx, double *__restrict__ dm, NearCombine near)
 {
     long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (p >= n) return;
     long long t = p / kBiB;
     int li = (int)(p % kBiB);
     double gx = 0, gy = 0, gz = 0, gm = 0;
-    if (njsub > 0) {
+    if (near.start && *near.near) {
+        const long long *start = near.start;
+        for (long long b = plan_first(start, near.grid, t * near.nch);
+             b < near.grid && start[b] < (t + 1) * near.nch; ++b) {
+            if (start[b + 1] <= start[b]) continue;
+            const double4 v = part[(size_t)(t + b) * kBiB + li];
+            gx += v.x; gy += v.y; gz += v.z; gm += v.w;
+        }
+    } else if (njsub > 0) {
         long long bf = sk_owner(t * njsub, grid, W), bl = sk_owner((t + 1) * njsub - 1, grid, W);
         for (long long s = 0; s <= bl - bf; ++s) {
             double4 v = part[((size_t)t * slots + (size_t)s) * kBiB + li];
@@ -568,12 +576,12 @@ __global__ void k_bw_combine(const double4 *__restrict__ part, const unsigned *_
 
 cudaError_t launch_backward_combine(const double4 *part, const unsigned *perm, long long n, int njsub,
                                     int slots, int grid, long long W, double mscale, double *dx,
-                                    double *dm, cudaStream_t st)
+                                    double *dm, cudaStream_t st, const NearCombine &near)
 {
     if (n <= 0) return cudaSuccess;
     k_bw_combine<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(part, perm, n, njsub, slots,
                                                               grid > 0 ? grid : 1, W > 0 ? W : 1,
-                                                              mscale, dx, dm);
+                                                              mscale, dx, dm, near);
     return cudaGetLastError();
 }
 

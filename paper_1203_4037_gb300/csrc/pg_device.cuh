@@ -197,6 +197,19 @@ __device__ __forceinline__ void bulk_g2s(void *dst, const void *src, unsigned by
         ::"r"(smem_u32(dst)), "l"(src), "r"(bytes), "r"(smem_u32(bar)) : "memory");
 }
 
+// ---------------------------------------------------------------- planned splits
+// the CTA of a culled run that holds unit u or starts last before it
+__device__ __forceinline__ long long plan_first(const long long *start, int grid, long long u)
+{
+    int lo = 0, hi = grid - 1;
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (start[mid] <= u) lo = mid;
+        else hi = mid - 1;
+    }
+    return lo;
+}
+
 // ---------------------------------------------------------------- misc
 __device__ __forceinline__ double4 ldg_d4(const double4 *p)
 {

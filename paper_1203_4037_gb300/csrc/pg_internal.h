@@ -50,6 +50,7 @@ struct AllPairsArgs {
     TableDev tab;
     double4 *part;         // partial sums [ntiles][smax_slots][Bi]
     int *status;
+    const int *skip = nullptr;     // set: a nonzero word here means another kernel does this run
 };
 
 // combine partials into the outputs (fixed slot order) and scatter
@@ -71,6 +72,9 @@ struct CombineArgs {
     double accscale;       // table: r_cut / sqrt(s_max - 2); Newton: 1
     double *acc;           // out: (ni, 3)
     double *pot;           // out: (ni), may be null
+    const long long *start = nullptr;   // a near-pair run's split (NearArgs), used where *near is nonzero
+    const int *near = nullptr;
+    int nch = 0, near_grid = 0;
     const int *fail_nan = nullptr;   // set: a nonzero word here (a force kernel's failure
                                      // status) makes every output NaN
 };
@@ -168,6 +172,7 @@ struct BackwardArgs {
     double *dv;            // knot-gradient accumulators (FP64, 2^(E+F)), may be null
     const unsigned *perm;  // tile order -> particle index (nullptr: identity): the own pair
     int *status;
+    const int *skip = nullptr;     // set: a nonzero word here means another kernel does this run
 };
 
 // Run a kernel's one-time set-up f (a function attribute) once on each
@@ -252,9 +257,62 @@ int pm_solve(PmState *s, const float *rho, const double4 *tgt, long long nt, dou
              int *launches, std::string &err);
 
 
-// gather i into tile order and compute tile centres
+// gather i into tile order and compute tile centres, and with ext set the
+// half extents of each tile's box
 cudaError_t launch_tile_prep(const double4 *xi, const unsigned *perm, long long n, int Bi,
-                             double4 *xi_tiled, double4 *ctr, cudaStream_t st);
+                             double4 *xi_tiled, double4 *ctr, cudaStream_t st, float4 *ext = nullptr);
+// ---------------------------------------------------------------- near pairs
+// The tabulated force on compact (sorted) i-tiles, pg_near.cu: g is exactly 0
+// from r_cut on, so each tile evaluates only the j within r_cut of its box.
+constexpr int kNearJ = 1024;           // j records tested per unit, at most
+struct NearArgs {
+    const double4 *xi;     // i positions (backward: and masses) in tile order
+    const double4 *wi;     // backward: loss weights in tile order
+    const double4 *ctr;    // FP64 centre of each i-tile
+    const float4 *ext;     // half extents of each tile's box, rounded up; infinite with a
+                           // non-finite particle
+    const double4 *jrec;   // j records (x, y, z, m)
+    const double4 *jw;     // backward: loss weights in j order
+    const float4 *jf;      // j records rounded to FP32
+    long long ni, nj;
+    int unit;              // j records per unit: kNearJ, or kNearJ / 2 or / 4 when that leaves few units
+    int ntiles, nch;       // i-tiles; units per tile, ceil(nj / unit)
+    int sstride;           // units of a tile are visited in steps of this (coprime to nch)
+    const long long *start;    // first unit of each CTA, grid + 1 (launch_near_plan)
+    const unsigned char *dense;    // tiles whose warps keep most of what the tile keeps
+    const int *near;       // zero: most pairs are near, the all-pairs kernel does this run
+    float r_cut;
+    TableDev tab;
+    double4 *part;         // CTA b's sums of tile t at part[(t + b) Bi ...]
+    double *dv;            // backward: knot-gradient accumulators, may be null
+    int *status;
+};
+// i-particles per thread of the table's backward kernels
+constexpr int kBwKI = 4;
+size_t near_smem(int np, int ntab, bool ext, bool df);            // ntab in float2 units
+int near_max_blocks_per_sm(int np, int ntab, bool ext, bool df);
+cudaError_t launch_near(const NearArgs &a, int grid, int np, bool ext, bool df, size_t smem, cudaStream_t st);
+size_t near_backward_smem(int ntab);
+int near_backward_max_blocks_per_sm(int ntab);
+cudaError_t launch_near_backward(const NearArgs &a, int grid, size_t smem, cudaStream_t st);
+// The split of the units over the CTAs. How many j a tile keeps differs by
+// two orders of magnitude between the core of a cluster and a tile whose box
+// spans it, so equal unit counts leave the worst CTA with many times the mean
+// work. Each tile's cost per unit is estimated from a sample of the j records
+// against the boxes of its warps' runs (run i each); the plan cuts the total
+// cost into grid equal ranges of consecutive units. pair_cost: clocks of one
+// record against one run, unit_cost: clocks of a unit that keeps nothing.
+// Fills cost (ntiles words), dense (ntiles bytes), start (grid + 1) and near:
+// 1 where the tiles' mean kept share (of each tile's worst warp) is below
+// kNearShare, else 0, and the all-pairs kernel runs instead (65536 Plummer:
+// at a share of 0.85 the near kernel took 3.1 ms, the all-pairs kernel 2.8).
+constexpr float kNearShare = 0.5f;
+cudaError_t launch_near_plan(const NearArgs &a, int Bi, int run, float pair_cost, float unit_cost, int grid,
+                             unsigned *cost, unsigned char *dense, long long *start, int *near, cudaStream_t st);
+// a step through nch units that spreads neighbours (coprime to nch)
+int near_stride(int nch);
+// records rounded to FP32
+cudaError_t launch_pack_f32(const double4 *rec, long long n, float4 *out, cudaStream_t st);
 
 // df: double-float differencing (i-tiles that are not compact; packed
 // arithmetic whatever `packed` says)
@@ -481,9 +539,15 @@ int backward_bi();
 int backward_max_blocks_per_sm(bool table, int ntab);
 cudaError_t launch_pack_w(const double *w, const unsigned *perm, long long n, double4 *wj,
                           double4 *wt, cudaStream_t st);
+// a near-pair run's split, as the combine reads it (start nullptr: none)
+struct NearCombine {
+    const long long *start = nullptr;
+    const int *near = nullptr;
+    int nch = 0, grid = 0;
+};
 cudaError_t launch_backward_combine(const double4 *part, const unsigned *perm, long long n,
                                     int njsub, int slots, int grid, long long W, double mscale,
-                                    double *dx, double *dm, cudaStream_t st);
+                                    double *dx, double *dm, cudaStream_t st, const NearCombine &near = NearCombine());
 cudaError_t launch_dv_out(const double *acc, int n, double scale, float *dv, cudaStream_t st);
 
 }  // namespace pg

@@ -403,16 +403,18 @@ cudaError_t launch_morton_sort(const double4 *xi, long long n, SortScratch &s, u
 // take the midpoint of the tile's bounding box as its FP64 centre.
 __global__ void k_tile_prep(const double4 *__restrict__ xi, const unsigned *__restrict__ perm,
                             long long n, int Bi, double4 *__restrict__ xt,
-                            double4 *__restrict__ ctr)
+                            double4 *__restrict__ ctr, float4 *__restrict__ ext)
 {
     __shared__ double red[6][32];
     long long t = blockIdx.x;
+    bool odd = false;          // a non-finite coordinate
     double lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
     for (int k = threadIdx.x; k < Bi; k += blockDim.x) {
         long long p = t * Bi + k;
         if (p >= n) break;
         double4 v = xi[perm ? (long long)perm[p] : p];
         xt[p] = v;
+        odd |= !(isfinite(v.x) && isfinite(v.y) && isfinite(v.z));
         lo[0] = fmin(lo[0], v.x); lo[1] = fmin(lo[1], v.y); lo[2] = fmin(lo[2], v.z);
         hi[0] = fmax(hi[0], v.x); hi[1] = fmax(hi[1], v.y); hi[2] = fmax(hi[2], v.z);
     }
@@ -424,7 +426,7 @@ __global__ void k_tile_prep(const double4 *__restrict__ xi, const unsigned *__re
     int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (lane == 0)
         for (int c = 0; c < 3; ++c) { red[c][w] = lo[c]; red[3 + c][w] = hi[c]; }
-    __syncthreads();
+    odd = __syncthreads_or(odd);
     if (threadIdx.x == 0) {
         int nw = blockDim.x >> 5;
         for (int q = 1; q < nw; ++q)
@@ -436,15 +438,37 @@ __global__ void k_tile_prep(const double4 *__restrict__ xi, const unsigned *__re
         double c1 = 0.5 * (red[1][0] + red[4][0]);
         double c2 = 0.5 * (red[2][0] + red[5][0]);
         ctr[t] = make_double4(c0, c1, c2, 0.0);
+        if (ext) {
+            // from the centre as stored, rounded up past the FP64 and FP32 roundings
+            auto half = [&](int c, double m) {
+                return odd ? INFINITY : (float)(fmax(red[3 + c][0] - m, m - red[c][0]) * (1.0 + 1e-6));
+            };
+            ext[t] = make_float4(half(0, c0), half(1, c1), half(2, c2), 0.0f);
+        }
     }
 }
 
 cudaError_t launch_tile_prep(const double4 *xi, const unsigned *perm, long long n, int Bi,
-                             double4 *xi_tiled, double4 *ctr, cudaStream_t st)
+                             double4 *xi_tiled, double4 *ctr, cudaStream_t st, float4 *ext)
 {
     long long nt = (n + Bi - 1) / Bi;
     if (nt <= 0) return cudaSuccess;
-    k_tile_prep<<<(unsigned)nt, 256, 0, st>>>(xi, perm, n, Bi, xi_tiled, ctr);
+    k_tile_prep<<<(unsigned)nt, 256, 0, st>>>(xi, perm, n, Bi, xi_tiled, ctr, ext);
+    return cudaGetLastError();
+}
+
+__global__ void k_pack_f32(const double4 *__restrict__ rec, long long n, float4 *__restrict__ out)
+{
+    const long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    if (k >= n) return;
+    const double4 v = rec[k];
+    out[k] = make_float4((float)v.x, (float)v.y, (float)v.z, (float)v.w);
+}
+
+cudaError_t launch_pack_f32(const double4 *rec, long long n, float4 *out, cudaStream_t st)
+{
+    if (n <= 0) return cudaSuccess;
+    k_pack_f32<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(rec, n, out);
     return cudaGetLastError();
 }
 
