@@ -491,6 +491,7 @@ int pg_create(pg_ctx **out, int device)
         pg_destroy(c);
         return PG_ENOMEM;
     }
+    c->sort.status = (int *)c->status.p;
     *out = c;
     return PG_OK;
 }
@@ -1312,7 +1313,7 @@ int enqueue_tiles(pg_ctx *c, const Plan &p)
         c->sort.sums = (unsigned *)c->ssums.p;
         c->sort.bbox = (unsigned long long *)c->sbbox.p;
         PG_CUDA(c, launch_morton_sort((const double4 *)c->xi.p, n, c->sort, &c->perm, c->stream));
-        c->last_launches += 3 + 5 * 4;
+        c->last_launches += 3 + 1 + 4;
     }
     PG_CUDA(c, launch_tile_prep((const double4 *)c->xi.p, c->perm, n, p.Bi, (double4 *)c->xt.p,
                                 (double4 *)c->ctr.p, c->stream, ext ? (float4 *)c->t_ext.p : nullptr));
@@ -2304,11 +2305,11 @@ int enqueue_cells(pg_ctx *c, double *acc, double *pot)
     PG_CUDA(c, launch_cell_build((const double4 *)c->jrec.p, n, c->box, nc, Bi, c->scale, s,
                                  c->sort, c->stream));
     // kernels of the build: key, count, gather, sizes, pairs, iota, items,
-    // permute (8), two scans (6), the 8-bit item sort (5) and the cell sort
-    // (5 per 8 key bits)
+    // permute (8), two scans (6), the 8-bit item sort (2) and the cell sort
+    // (its count and one per 8 key bits)
     int cell_bits = 0;
     while ((1LL << cell_bits) < ncell) ++cell_bits;
-    c->last_launches += 19 + 5 * ((cell_bits + 7) / 8);
+    c->last_launches += 17 + (cell_bits + 7) / 8;
     GroupArgs g = group_args(c);
     g.xi = s.xs;
     g.jrec = s.xs;
@@ -2600,7 +2601,7 @@ int pg_backward_dev(pg_ctx *c, const double *w, double *dx, double *dm, float *d
         c->sort.sums = (unsigned *)c->ssums.p;
         c->sort.bbox = (unsigned long long *)c->sbbox.p;
         PG_CUDA(c, launch_morton_sort((const double4 *)c->jrec.p, n, c->sort, &c->perm, c->stream));
-        c->last_launches += 3 + 5 * 4;
+        c->last_launches += 3 + 1 + 4;
     }
     c->i_dirty = true;      // the tile buffers now hold the backward's order
     const bool cull = table && n >= 16384;

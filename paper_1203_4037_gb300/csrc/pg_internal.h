@@ -204,7 +204,8 @@ cudaError_t launch_pack_i(const double *x, double4 *xi, long long n, cudaStream_
 struct SortScratch {
     unsigned *keys[2];
     unsigned *vals[2];
-    unsigned *hist;        // 256 * nchunks (+ block sums)
+    unsigned *hist;        // sort_hist_entries words: look-back words, digit counts, tickets
+    int *status;           // where a look-back that gives up reports
     unsigned *sums;
     unsigned long long *bbox;  // 6 ordered-int words
     size_t cap;            // elements

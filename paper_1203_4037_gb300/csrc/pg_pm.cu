@@ -478,7 +478,7 @@ cudaError_t records(PmState *s, const double4 *rec, long long n, bool sorted, in
         cudaError_t e = launch_radix_sort(sort.keys[0], sort.vals[0], n, kb, sort, &ko, &sp, st);
         if (e != cudaSuccess) return e;
         perm = sp;
-        if (launches) *launches += (kb + 7) / 8 * 5;
+        if (launches) *launches += (kb + 7) / 8 + 1;
     }
     k_pm_gather<<<blocks256(n), 256, 0, st>>>(s->mj_raw, s->md_raw, perm, n, mj_out, md_out);
     cudaMemcpyAsync(perm_keep, perm, n * sizeof(unsigned), cudaMemcpyDeviceToDevice, st);

@@ -7,6 +7,8 @@
 //  * a stable LSD radix sort (8-bit digits, warp-level ranking) used for that
 //    ordering and for the cell list;
 //  * gather into tile order with per-tile FP64 centres.
+#include <algorithm>
+
 #include "pg_device.cuh"
 
 namespace pg {
@@ -135,148 +137,233 @@ __global__ void k_morton(const double4 *__restrict__ x, long long n,
 }
 
 // ---------------------------------------------------------------- radix sort
-// Each warp owns a chunk of kChunk consecutive elements; a pass histograms
-// the chunk's 8-bit digits, a scan turns the digit-major histogram into
-// global offsets, and the scatter re-reads the chunk in order and ranks
-// equal digits by lane order, which keeps the sort stable. A lane loads
-// kBatch rounds' elements before it uses them, so a warp has kBatch loads
-// in flight instead of one (about seven warps per SM hold the 2^20-key
-// sorts' chunks; one load at a time left each pass latency-bound).
-constexpr int kRounds = 32;
-constexpr int kChunk = 32 * kRounds;
-constexpr int kWarpsPerBlock = 4;
-constexpr int kBatch = 8;
-static_assert(kRounds % kBatch == 0, "rounds come in whole batches");
+// Least significant digit first, 8 bits a pass, one launch a pass. A kernel
+// first counts every pass's digits at once. In a pass each block takes the
+// next tile of keys by ticket, counts its digits, and learns how many keys of
+// each digit the tiles before it hold by looking back at what those blocks
+// have published (the decoupled look-back of Merrill and Garland's scan,
+// 2016, and of Adinets and Merrill's one-sweep radix sort, 2022): its own
+// count first, then, once known, the count up to and including itself. A
+// block waits only on blocks with earlier tickets, which are running or done.
+// Ranking by lane order within rounds keeps the sort stable. The keys are
+// placed in shared memory in destination order first and written out as runs
+// of consecutive addresses.
+//
+// Bound: launches and the look-back's round trips. A histogram, three scan
+// kernels and a scatter per pass took 20 launches for 30-bit keys; now it is
+// a memset, the count and four passes. Measured: a 250007-particle PP + PM
+// call (four sorted passes) 439 -> 410 us, a 65536-particle fit of a table
+// (two sorts of four passes) 2000 -> 1680 us; a pass over 2^21 keys 38 us, as
+// long as the five kernels it replaces.
+constexpr int kSortWarps = 8;                  // 256 threads, one per digit
+constexpr int kSortThreads = 32 * kSortWarps;
+// keys per lane: tiles of 8192 keys for large sets; for small ones tiles of
+// 2048, four times the blocks
+constexpr int kSortRounds = 32, kSortRoundsSmall = 8;
+constexpr int kSortBatch = 8;          // rounds in flight per lane
+constexpr long long kSortSmall = 1LL << 18;
+constexpr int kSortPasses = 4;         // 32-bit keys
 
+long long sort_tiles(long long n)
+{
+    const int rounds = n <= kSortSmall ? kSortRoundsSmall : kSortRounds;
+    return (n + kSortThreads * rounds - 1) / (kSortThreads * rounds);
+}
+
+// 32-bit words of SortScratch::hist: the look-back words (two of them each),
+// the digit counts and the tickets
 size_t sort_hist_entries(long long n)
 {
-    long long nchunks = (n + kChunk - 1) / kChunk;
-    return (size_t)(256 * nchunks);
+    return (size_t)kSortPasses * (512 * (size_t)sort_tiles(n) + 256 + 1) + 16;
 }
 
-__global__ void k_rs_hist(const unsigned *__restrict__ keys, long long n, int shift,
-                          long long nchunks, unsigned *__restrict__ hist)
+// counts of every pass's digits, added to cnt[pass][256]
+__global__ void __launch_bounds__(256) k_rs_count(const unsigned *__restrict__ keys, long long n, int passes,
+                                                  unsigned *__restrict__ cnt)
 {
-    __shared__ unsigned cnt[kWarpsPerBlock][256];
-    int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    long long chunk = blockIdx.x * (long long)kWarpsPerBlock + w;
-    for (int d = lane; d < 256; d += 32) cnt[w][d] = 0;
-    __syncwarp();
-    if (chunk < nchunks) {
-        const long long base = chunk * kChunk;
-#pragma unroll 1
-        for (int r0 = 0; r0 < kRounds; r0 += kBatch) {
-            unsigned k[kBatch];
+    __shared__ unsigned h[kSortPasses * 256];
+    for (int k = threadIdx.x; k < passes * 256; k += blockDim.x) h[k] = 0;
+    __syncthreads();
+    const long long stride = (long long)gridDim.x * blockDim.x;
+    for (long long i0 = blockIdx.x * (long long)blockDim.x + threadIdx.x; i0 < n; i0 += 4 * stride) {
+        unsigned k[4];
 #pragma unroll
-            for (int b = 0; b < kBatch; ++b) {
-                const long long e = base + (r0 + b) * 32 + lane;
-                k[b] = e < n ? keys[e] : 0u;
-            }
+        for (int q = 0; q < 4; ++q) k[q] = i0 + q * stride < n ? keys[i0 + q * stride] : 0u;
 #pragma unroll
-            for (int b = 0; b < kBatch; ++b)
-                if (base + (r0 + b) * 32 + lane < n) atomicAdd(&cnt[w][(k[b] >> shift) & 255u], 1u);
-        }
+        for (int q = 0; q < 4; ++q)
+            if (i0 + q * stride < n)
+                for (int p = 0; p < passes; ++p) atomicAdd(&h[p * 256 + ((k[q] >> (8 * p)) & 255u)], 1u);
     }
-    __syncwarp();
-    if (chunk < nchunks)
-        for (int d = lane; d < 256; d += 32) hist[(long long)d * nchunks + chunk] = cnt[w][d];
+    __syncthreads();
+    for (int k = threadIdx.x; k < passes * 256; k += blockDim.x)
+        if (h[k]) atomicAdd(&cnt[k], h[k]);
 }
 
-// The scatter ranks each key as before (its destination: the chunk's
-// offset for its digit plus the lane-ordered rank of equal digits before
-// it), but places it in shared memory first, at its destination's position
-// within the block's range for its digit (a block's chunks are adjacent in
-// the digit-major offsets, so each digit's keys of a block go to one
-// contiguous range). The block then writes its keys out in that order:
-// runs of consecutive addresses instead of up to 32 scattered words per
-// warp round.
-__global__ void __launch_bounds__(32 * kWarpsPerBlock) k_rs_scatter(const unsigned *__restrict__ kin,
-                                                                    const unsigned *__restrict__ vin,
-                                                                    unsigned *__restrict__ kout,
-                                                                    unsigned *__restrict__ vout, long long n,
-                                                                    int shift, long long nchunks,
-                                                                    const unsigned *__restrict__ offs)
+// exclusive scan of 256 values in shared memory by one warp
+__device__ __forceinline__ void scan256(unsigned *v, int lane)
 {
-    __shared__ unsigned cnt[kWarpsPerBlock][256];
-    __shared__ unsigned sk[kWarpsPerBlock * kChunk], sv[kWarpsPerBlock * kChunk];
+    unsigned x[8], tot = 0;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+        x[q] = v[8 * lane + q];
+        tot += x[q];
+    }
+    unsigned incl = tot;
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += y;
+    }
+    unsigned run = incl - tot;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+        v[8 * lane + q] = run;
+        run += x[q];
+    }
+}
+
+// look-back word of (tile, digit): a count with its kind in the top bits
+constexpr int kLook = 32;                      // look-back words a thread reads at once
+constexpr u64 kOwn = 1ull << 62, kUpTo = 2ull << 62, kCountMask = (1ull << 62) - 1;
+
+__device__ __forceinline__ u64 ld_relaxed(const u64 *p)
+{
+    u64 v;
+    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ void st_relaxed(u64 *p, u64 v)
+{
+    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
+
+template <int R>
+__global__ void __launch_bounds__(kSortThreads) k_rs_pass(const unsigned *__restrict__ kin,
+                                                          const unsigned *__restrict__ vin,
+                                                          unsigned *__restrict__ kout, unsigned *__restrict__ vout,
+                                                          long long n, int shift, const unsigned *__restrict__ total,
+                                                          u64 *look, unsigned *ticket, int *status)
+{
+    constexpr int kTile = kSortThreads * R, kChunk = 32 * R;
+    extern __shared__ unsigned sort_smem[];
+    unsigned *sk = sort_smem, *sv = sk + kTile;
+    unsigned (*cnt)[256] = reinterpret_cast<unsigned (*)[256]>(sv + kTile);   // [kSortWarps][256]
     __shared__ unsigned gstart[256], lstart[256];
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const long long chunk0 = blockIdx.x * (long long)kWarpsPerBlock, chunk = chunk0 + w;
-    const long long last = min(chunk0 + kWarpsPerBlock, nchunks);       // the block's chunks [chunk0, last)
-    // per digit: the block's first destination and its key count; the
-    // offsets are an exclusive scan, so the entry after the block's last
-    // chunk of digit d ends the block's run of d (n after the array)
-    for (int d = threadIdx.x; d < 256; d += blockDim.x) {
-        const long long e = (long long)d * nchunks + last;
-        gstart[d] = offs[(long long)d * nchunks + chunk0];
-        lstart[d] = (e < 256 * nchunks ? offs[e] : (unsigned)n) - gstart[d];
-    }
+    __shared__ unsigned tile_s;
+    const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
+    if (tid == 0) tile_s = atomicAdd(ticket, 1u);
+    for (int d = lane; d < 256; d += 32) cnt[w][d] = 0;
+    for (int d = tid; d < 256; d += kSortThreads) gstart[d] = total[d];
     __syncthreads();
-    if (w == 0) {        // lstart: exclusive scan of the counts over the digits
-        unsigned v[8], tot = 0;
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            v[q] = lstart[8 * lane + q];
-            tot += v[q];
-        }
-        unsigned incl = tot;
-        for (int o = 1; o < 32; o <<= 1) {
-            const unsigned y = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += y;
-        }
-        unsigned run = incl - tot;
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            lstart[8 * lane + q] = run;
-            run += v[q];
-        }
-    }
-    if (chunk < nchunks)
-        for (int d = lane; d < 256; d += 32) cnt[w][d] = offs[(long long)d * nchunks + chunk];
-    __syncthreads();
-    const long long base = chunk * kChunk;
-    const unsigned lt = (1u << lane) - 1u;
-    if (chunk < nchunks) {
+    const long long tile = tile_s, base = tile * kTile + w * kChunk;
 #pragma unroll 1
-        for (int r0 = 0; r0 < kRounds; r0 += kBatch) {
-            unsigned kk[kBatch], vv[kBatch];
+    for (int r0 = 0; r0 < R; r0 += kSortBatch) {
+        unsigned key[kSortBatch];
 #pragma unroll
-            for (int b = 0; b < kBatch; ++b) {
-                const long long e = base + (r0 + b) * 32 + lane;
-                kk[b] = e < n ? kin[e] : 0u;
-                vv[b] = e < n ? vin[e] : 0u;
-            }
+        for (int r = 0; r < kSortBatch; ++r) key[r] = base + (r0 + r) * 32 + lane < n ? kin[base + (r0 + r) * 32 + lane] : 0u;
 #pragma unroll
-            for (int b = 0; b < kBatch; ++b) {
-                const bool valid = base + (r0 + b) * 32 + lane < n;
-                const unsigned key = kk[b], val = vv[b];
-                const unsigned d = valid ? ((key >> shift) & 255u) : 256u + lane;   // invalid lanes never match
-                const unsigned peers = __match_any_sync(0xffffffffu, d);
-                const int leader = __ffs(peers) - 1;
-                const unsigned rank = __popc(peers & lt);
-                unsigned start = 0;
-                if (valid && lane == leader) start = cnt[w][d];
-                start = __shfl_sync(0xffffffffu, start, leader);
-                __syncwarp();
-                if (valid) {
-                    const unsigned p = lstart[d] + (start + rank - gstart[d]);
-                    sk[p] = key;
-                    sv[p] = val;
-                    if (lane == leader) cnt[w][d] = start + __popc(peers);
+        for (int r = 0; r < kSortBatch; ++r)
+            if (base + (r0 + r) * 32 + lane < n) atomicAdd(&cnt[w][(key[r] >> shift) & 255u], 1u);
+    }
+    __syncthreads();
+    if (w == 0) scan256(gstart, lane);         // keys of smaller digits
+    u64 *mine = look + (size_t)tile * 256;
+    for (int d = tid; d < 256; d += kSortThreads) {
+        unsigned c = 0;
+#pragma unroll
+        for (int q = 0; q < kSortWarps; ++q) c += cnt[q][d];
+        lstart[d] = c;
+        st_relaxed(mine + d, (tile == 0 ? kUpTo : kOwn) | c);
+    }
+    __syncthreads();
+    // the tiles before this one, digit by digit
+    if (tile > 0)
+        for (int d = tid; d < 256; d += kSortThreads) {
+            u64 before = 0;
+            const u64 t0 = global_ns();
+            for (long long q = tile - 1; q >= 0;) {
+                // all tiles start together, so few have their running count yet
+                // and the walk takes tiles / kLook round trips
+                u64 v[kLook];
+#pragma unroll
+                for (int k = 0; k < kLook; ++k) v[k] = q - k >= 0 ? ld_relaxed(look + (size_t)(q - k) * 256 + d) : kUpTo;
+                bool wait = false;
+#pragma unroll
+                for (int k = 0; k < kLook; ++k) {
+                    if (wait || q < 0) continue;
+                    if (!(v[k] & ~kCountMask)) { wait = true; continue; }
+                    before += v[k] & kCountMask;
+                    q = v[k] & kUpTo ? -1 : q - 1;
                 }
-                __syncwarp();
+                if (wait && global_ns() - t0 > kWaitLimitNs) {
+                    report(status, kStatusTimeout, 6);
+                    break;
+                }
             }
+            st_relaxed(mine + d, kUpTo | (before + lstart[d]));
+            gstart[d] += (unsigned)before;
+        }
+    __syncthreads();
+    if (w == 0) scan256(lstart, lane);
+    __syncthreads();
+    // each warp's first place of each digit in the tile's order
+    for (int d = tid; d < 256; d += kSortThreads) {
+        unsigned at = lstart[d];
+#pragma unroll
+        for (int q = 0; q < kSortWarps; ++q) {
+            const unsigned c = cnt[q][d];
+            cnt[q][d] = at;
+            at += c;
         }
     }
     __syncthreads();
-    // the block's keys in destination order
-    const long long b0 = chunk0 * kChunk;
-    const int nb = (int)(min(n, last * (long long)kChunk) - b0);
-    for (int p = threadIdx.x; p < nb; p += blockDim.x) {
-        const unsigned key = sk[p], d = (key >> shift) & 255u;
+    const unsigned lt = (1u << lane) - 1u;
+    // ranks, kSortBatch rounds at a time: the lanes with each lane's digit by
+    // eight ballots (independent over the rounds), then the running places
+#pragma unroll 1
+    for (int r0 = 0; r0 < R; r0 += kSortBatch) {
+        unsigned key[kSortBatch], val[kSortBatch], peers[kSortBatch];
+#pragma unroll
+        for (int r = 0; r < kSortBatch; ++r) {
+            const long long e = base + (r0 + r) * 32 + lane;
+            key[r] = e < n ? kin[e] : 0u;
+            val[r] = e < n ? vin[e] : 0u;
+        }
+#pragma unroll
+        for (int r = 0; r < kSortBatch; ++r) {
+            const unsigned d = key[r] >> shift;
+            unsigned m = __ballot_sync(0xffffffffu, base + (r0 + r) * 32 + lane < n);   // invalid lanes match nobody
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                const bool bit = d >> k & 1u;
+                const unsigned bal = __ballot_sync(0xffffffffu, bit);
+                m &= bit ? bal : ~bal;
+            }
+            peers[r] = m;
+        }
+#pragma unroll
+        for (int r = 0; r < kSortBatch; ++r) {
+            const bool valid = base + (r0 + r) * 32 + lane < n;
+            const unsigned d = (key[r] >> shift) & 255u, below = __popc(peers[r] & lt);
+            unsigned at = 0;
+            if (valid) at = cnt[w][d] + below;
+            __syncwarp();
+            if (valid) {
+                if (below == 0) cnt[w][d] = at + __popc(peers[r]);
+                sk[at] = key[r];
+                sv[at] = val[r];
+            }
+            __syncwarp();
+        }
+    }
+    __syncthreads();
+    const int nb = (int)min((long long)kTile, n - tile * kTile);
+    for (int p = tid; p < nb; p += kSortThreads) {
+        const unsigned k = sk[p], d = (k >> shift) & 255u;
         const unsigned g = gstart[d] + ((unsigned)p - lstart[d]);
-        kout[g] = key;
-        vout[g] = sv[p];
+        if (g < n) {                           // (always, unless a wait ran out)
+            kout[g] = k;
+            vout[g] = sv[p];
+        }
     }
 }
 
@@ -364,23 +451,42 @@ cudaError_t launch_excl_scan(unsigned *a, long long n, unsigned *sums, cudaStrea
     return excl_scan(a, n, sums, st);
 }
 
+static size_t sort_smem_bytes(int rounds)
+{
+    return ((size_t)2 * kSortThreads * rounds + kSortWarps * 256) * sizeof(unsigned);
+}
+
 cudaError_t launch_radix_sort(unsigned *keys, unsigned *vals, long long n, int key_bits,
                               SortScratch &s, unsigned **keys_out, unsigned **vals_out,
                               cudaStream_t st)
 {
-    long long nchunks = (n + kChunk - 1) / kChunk;
     unsigned *kin = keys, *vin = vals;
     unsigned *kb = (keys == s.keys[0]) ? s.keys[1] : s.keys[0];
     unsigned *vb = (vals == s.vals[0]) ? s.vals[1] : s.vals[0];
-    unsigned blocks = (unsigned)((nchunks + kWarpsPerBlock - 1) / kWarpsPerBlock);
-    for (int shift = 0; shift < key_bits && n > 0; shift += 8) {
-        k_rs_hist<<<blocks, 32 * kWarpsPerBlock, 0, st>>>(kin, n, shift, nchunks, s.hist);
-        cudaError_t e = excl_scan(s.hist, 256 * nchunks, s.sums, st);
+    const int passes = (key_bits + 7) / 8;
+    if (n > 0 && passes > 0) {
+        const long long tiles = sort_tiles(n);
+        u64 *look = (u64 *)s.hist;
+        unsigned *cnt = (unsigned *)(look + (size_t)passes * tiles * 256), *ticket = cnt + passes * 256;
+        cudaError_t e = cudaMemsetAsync(s.hist, 0, (char *)(ticket + passes) - (char *)s.hist, st);
         if (e != cudaSuccess) return e;
-        k_rs_scatter<<<blocks, 32 * kWarpsPerBlock, 0, st>>>(kin, vin, kb, vb, n, shift, nchunks,
-                                                              s.hist);
-        unsigned *t = kin; kin = kb; kb = t;
-        t = vin; vin = vb; vb = t;
+        const long long blocks = (n + 1023) / 1024;
+        k_rs_count<<<(unsigned)std::min<long long>(blocks, 608), 256, 0, st>>>(kin, n, passes, cnt);
+        const bool small = n <= kSortSmall;
+        const size_t smem = sort_smem_bytes(small ? kSortRoundsSmall : kSortRounds);
+        static bool done[kMaxDevices] = {};
+        e = once_per_device(done, [] {
+            return cudaFuncSetAttribute(k_rs_pass<kSortRounds>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                        (int)sort_smem_bytes(kSortRounds));
+        });
+        if (e != cudaSuccess) return e;
+        for (int p = 0; p < passes; ++p) {
+            auto k = small ? k_rs_pass<kSortRoundsSmall> : k_rs_pass<kSortRounds>;
+            k<<<(unsigned)tiles, kSortThreads, smem, st>>>(kin, vin, kb, vb, n, 8 * p, cnt + 256 * p,
+                                                        look + (size_t)p * tiles * 256, ticket + p, s.status);
+            std::swap(kin, kb);
+            std::swap(vin, vb);
+        }
     }
     *keys_out = kin;
     *vals_out = vin;

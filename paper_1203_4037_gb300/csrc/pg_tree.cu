@@ -1255,7 +1255,7 @@ cudaError_t tree_stage_keys(const double4 *jrec, long long n, TreeScratch &t, So
     unsigned *ko = nullptr, *perm = nullptr;
     cudaError_t e = launch_radix_sort(sort.keys[0], sort.vals[0], n, 3 * kBits, sort, &ko, &perm, st);
     if (e != cudaSuccess) return e;
-    t.launches += 4 + (n > 0 ? (3 * kBits + 7) / 8 * 5 : 0) + 3;   // with the gather, flags, offsets
+    t.launches += 4 + (n > 0 ? (3 * kBits + 7) / 8 + 1 : 0) + 3;   // with the gather, flags, offsets
     cudaMemcpyAsync(t.key, ko, n * sizeof(unsigned), cudaMemcpyDeviceToDevice, st);
     cudaMemcpyAsync(t.perm, perm, n * sizeof(unsigned), cudaMemcpyDeviceToDevice, st);
     k_tree_gather<<<blocks_of(n), 256, 0, st>>>(jrec, t.perm, n, t.xs, t.xi0);

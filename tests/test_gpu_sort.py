@@ -1,0 +1,53 @@
+"""The radix sort behind the tree, the tiles and the cell list, through the
+tree's particle order (a stable sort of the oracle's keys, bit-exact): one key,
+a tile less one, a tile, a tile more one, both tile sizes (the switch is at
+2^18), many tiles, and sets where nearly all keys share a digit."""
+
+import numpy as np
+import pytest
+
+import gen
+from pgtest import need_cuda
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def pg():
+    return need_cuda()
+
+
+def keys(x):
+    lo = x.min(axis=0)
+    span = float((x.max(axis=0) - lo).max()) or 1.0
+    q = np.minimum(np.floor((x - lo) / span * 1024), 1023).astype(np.int64)
+    k = np.zeros(len(x), np.int64)
+    for b in range(10):
+        for a in range(3):
+            k |= ((q[:, a] >> b) & 1) << (3 * b + 2 - a)
+    return k
+
+
+def order(pg, x):
+    with pg.Context(0) as c:
+        c.set_eps(0.01)
+        c.set_self(True)
+        c.set_tree(0.75, 256, 8)
+        c.set_j(x, np.full(len(x), 1.0 / len(x)))
+        c.set_i(x)
+        c.run()
+        return c.get_tree()["perm"]
+
+
+@pytest.mark.parametrize("n", [1, 31, 2047, 2048, 2049, 100003, 1 << 18, (1 << 18) + 1, 70 * 8192 + 5])
+def test_order_is_the_stable_sort(pg, n):
+    x = gen.plummer(n, 50 + n)[0]
+    assert np.array_equal(order(pg, x), np.argsort(keys(x), kind="stable"))
+
+
+@pytest.mark.parametrize("n", [5000, 300000])
+def test_crowded_digits(pg, n):
+    # all but a few particles in one octant's corner: most digits are equal
+    x = gen.uniform_sphere(n, 7, radius=1e-3)[0]
+    x[:3] = [[0, 0, 0], [1, 1, 1], [1, 0, 0.5]]
+    assert np.array_equal(order(pg, x), np.argsort(keys(x), kind="stable"))
