@@ -304,6 +304,7 @@ __device__ __forceinline__ void moments_leaf_one(long long k, const int *__restr
 {
     double m = 0.0, s0 = 0.0, s1 = 0.0, s2 = 0.0;
     const int f = first[k], e = f + count[k];
+#pragma unroll 4
     for (int i = f; i < e; ++i) {
         const double4 v = xs[i];
         m = __dadd_rn(m, v.w);
@@ -318,6 +319,7 @@ __device__ __forceinline__ void moments_leaf_one(long long k, const int *__restr
     const double4 c = node_finish(k, m, s0, s1, s2, first, count, child0, childn, o);
     if (!o.T) return;
     double t[6] = {0, 0, 0, 0, 0, 0};
+#pragma unroll 4
     for (int i = f; i < e; ++i) {
         const double4 v = xs[i];
         const double y0 = v.x - c.x, y1 = v.y - c.y, y2 = v.z - c.z;
@@ -350,13 +352,27 @@ __device__ __forceinline__ void moments_up_one(long long k, const int *__restric
                                                const int *__restrict__ childn, double *__restrict__ M,
                                                double *__restrict__ S, const NodeOut &o)
 {
+    // all children's values (at most eight) are loaded before the ordered
+    // sums: a loop over the children waited for each in turn
     double m = 0.0, s0 = 0.0, s1 = 0.0, s2 = 0.0;
-    const int c0 = child0[k], c1 = c0 + childn[k];
-    for (int ch = c0; ch < c1; ++ch) {
-        m = __dadd_rn(m, M[ch]);
-        s0 = __dadd_rn(s0, S[3 * ch]);
-        s1 = __dadd_rn(s1, S[3 * ch + 1]);
-        s2 = __dadd_rn(s2, S[3 * ch + 2]);
+    const int c0 = child0[k], nc = childn[k];
+    {
+        double v[8][4];
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+            if (q < nc) {
+                v[q][0] = M[c0 + q];
+#pragma unroll
+                for (int d = 0; d < 3; ++d) v[q][1 + d] = S[3 * (c0 + q) + d];
+            }
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+            if (q < nc) {
+                m = __dadd_rn(m, v[q][0]);
+                s0 = __dadd_rn(s0, v[q][1]);
+                s1 = __dadd_rn(s1, v[q][2]);
+                s2 = __dadd_rn(s2, v[q][3]);
+            }
     }
     M[k] = m;
     S[3 * k] = s0;
@@ -365,16 +381,28 @@ __device__ __forceinline__ void moments_up_one(long long k, const int *__restric
     const double4 c = node_finish(k, m, s0, s1, s2, first, count, child0, childn, o);
     if (!o.T) return;
     double t[6] = {0, 0, 0, 0, 0, 0};
-    for (int ch = c0; ch < c1; ++ch) {
-        const double4 cc = o.com[ch];
-        const double y0 = cc.x - c.x, y1 = cc.y - c.y, y2 = cc.z - c.z;
-        const double *tc = o.T + 6 * (long long)ch;
-        t[0] += tc[0] + cc.w * y0 * y0;
-        t[1] += tc[1] + cc.w * y0 * y1;
-        t[2] += tc[2] + cc.w * y0 * y2;
-        t[3] += tc[3] + cc.w * y1 * y1;
-        t[4] += tc[4] + cc.w * y1 * y2;
-        t[5] += tc[5] + cc.w * y2 * y2;
+#pragma unroll
+    for (int h = 0; h < 8; h += 4) {
+        double4 cc[4];
+        double tc[4][6];
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            if (h + q < nc) {
+                cc[q] = o.com[c0 + h + q];
+#pragma unroll
+                for (int d = 0; d < 6; ++d) tc[q][d] = o.T[6 * (long long)(c0 + h + q) + d];
+            }
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            if (h + q < nc) {
+                const double y0 = cc[q].x - c.x, y1 = cc[q].y - c.y, y2 = cc[q].z - c.z;
+                t[0] += tc[q][0] + cc[q].w * y0 * y0;
+                t[1] += tc[q][1] + cc[q].w * y0 * y1;
+                t[2] += tc[q][2] + cc[q].w * y0 * y2;
+                t[3] += tc[q][3] + cc[q].w * y1 * y1;
+                t[4] += tc[q][4] + cc[q].w * y1 * y2;
+                t[5] += tc[q][5] + cc[q].w * y2 * y2;
+            }
     }
     for (int q = 0; q < 6; ++q) o.T[6 * k + q] = t[q];
 }
@@ -1284,14 +1312,22 @@ cudaError_t tree_stage_moments(long long n, TreeScratch &t, cudaStream_t st)
     NodeOut no{t.com, t.npseudo == 1 ? t.jrec2 + n : nullptr, t.nodew, t.npseudo == 3 ? t.T : nullptr};
     k_tree_moments_leaf<<<blocks_of(t.hint_runs[kLevels - 1]), 256, 0, st>>>(t.meta, t.first, t.count, t.child0,
                                                                              t.childn, t.xs, t.M, t.S, no);
-    // levels of at most kTopNodes nodes in the last call (their counts grow
-    // with the level) go to the one-block kernel
-    constexpr long long kTopNodes = 2048;
+    // Levels of at most `top` nodes in the last call (their counts grow with
+    // the level) go to the one-block kernel. A node is about 50 FP64
+    // operations, with second moments about 200, and one SM issues two a
+    // clock: the line lies where a level's work on one SM takes as long as a
+    // launch of its own (about 10 us). With 2048 for both, the one-block
+    // kernel of a 300007-particle quadrupole tree took 185 us. The other
+    // coarse levels run in blocks of 64 nodes for the same reason: 2000 nodes
+    // in blocks of 256 leave the work to eight SMs (26 us a level; now 14).
+    // The call: 1678 -> 1555 us; 2^20 monopoles 2317 -> 2289 us.
+    const long long top = t.npseudo == 3 ? 128 : 512;
     int L0 = -1;
-    while (L0 + 1 < kLevels - 1 && t.hint_runs[L0 + 1] <= kTopNodes) ++L0;
-    for (int L = kLevels - 2; L > L0; --L)
-        k_tree_moments_up<<<blocks_of(t.hint_runs[L]), 256, 0, st>>>(t.meta, L, t.first, t.count, t.child0,
-                                                                     t.childn, t.M, t.S, no);
+    while (L0 + 1 < kLevels - 1 && t.hint_runs[L0 + 1] <= top) ++L0;
+    for (int L = kLevels - 2; L > L0; --L) {
+        const unsigned nb = (unsigned)((std::max(t.hint_runs[L], 1LL) + 63) / 64);
+        k_tree_moments_up<<<nb, 64, 0, st>>>(t.meta, L, t.first, t.count, t.child0, t.childn, t.M, t.S, no);
+    }
     if (L0 >= 0)
         k_tree_moments_top<<<1, 1024, 0, st>>>(t.meta, L0, t.first, t.count, t.child0, t.childn, t.M, t.S, no);
     t.launches += 1 + (kLevels - 2 - L0) + (L0 >= 0 ? 1 : 0);
