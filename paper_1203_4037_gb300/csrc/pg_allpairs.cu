@@ -558,18 +558,21 @@ cudaError_t launch_allpairs(const AllPairsArgs &a, int grid, int np, bool table,
 __global__ void k_combine(CombineArgs c)
 {
     long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (p >= c.ni) return;
-    long long t = p / c.Bi;
+    const bool in = p < c.ni;
+    if (!in && !c.start) return;
+    long long t = (in ? p : c.ni - 1) / c.Bi;
     int li = (int)(p % c.Bi);
     double ax = 0, ay = 0, az = 0, ph = 0;
-    if (c.start && *c.near) {
-        for (long long b = plan_first(c.start, c.near_grid, t * c.nch);
-             b < c.near_grid && c.start[b] < (t + 1) * c.nch; ++b) {
-            if (c.start[b + 1] <= c.start[b]) continue;
-            const double4 v = c.part[(size_t)(t + b) * c.Bi + li];
+    if (c.start && *c.near) {          // (a block's i are of one tile, whose search all threads share)
+        int b0, b1;
+        plan_ctas(c.start, c.near_grid, t * c.nch, (t + 1) * c.nch, b0, b1);
+#pragma unroll 8
+        for (int b = b0; b < b1; ++b) {
+            if (!in || c.start[b + 1] <= c.start[b]) continue;
+            const double4 v = ldg_d4(c.part + (size_t)(t + b) * c.Bi + li);
             ax += v.x; ay += v.y; az += v.z; ph += v.w;
         }
-    } else if (c.njsub > 0) {
+    } else if (in && c.njsub > 0) {
         long long bf = stream_k_owner(t * c.njsub, c.grid, c.W);
         long long bl = stream_k_owner((t + 1) * c.njsub - 1, c.grid, c.W);
         for (long long s = 0; s <= bl - bf; ++s) {
@@ -577,6 +580,7 @@ __global__ void k_combine(CombineArgs c)
             ax += v.x; ay += v.y; az += v.z; ph += v.w;
         }
     }
+    if (!in) return;
     long long k = c.perm ? (long long)c.perm[p] : p;
     if (c.self && c.njsub > 0) ph -= self_potential(c, k);
     if (c.fail_nan && *c.fail_nan != 0) ax = ay = az = ph = __longlong_as_double(0x7ff8000000000000ll);

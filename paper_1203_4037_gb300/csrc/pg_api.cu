@@ -1418,7 +1418,7 @@ int near_args(pg_ctx *c, NearArgs &a, const double4 *xt, const double4 *jrec, lo
     const int ntiles = (int)((ni + Bi - 1) / Bi);
     a.unit = near_unit(ntiles, nj, grid);
     if ((rc = ensure(c, c->j_f32, (size_t)nj * sizeof(float4))) ||
-        (rc = ensure(c, c->t_cost, (size_t)ntiles * sizeof(unsigned))) || (rc = ensure(c, c->t_dense, ntiles)) ||
+        (rc = ensure(c, c->t_cost, (size_t)ntiles * (sizeof(unsigned long long) + sizeof(unsigned)))) || (rc = ensure(c, c->t_dense, ntiles)) ||
         (rc = ensure(c, c->t_start, (size_t)(grid + 2) * sizeof(long long))) ||
         (rc = ensure(c, c->part, ((size_t)ntiles + grid) * Bi * sizeof(double4))))
         return rc;
@@ -1441,7 +1441,9 @@ int near_args(pg_ctx *c, NearArgs &a, const double4 *xt, const double4 *jrec, lo
     a.tab = table_dev(c);
     a.part = (double4 *)c->part.p;
     a.status = (int *)c->status.p;
-    PG_CUDA(c, launch_near_plan(a, Bi, run, pair_cost, 1500.0f, grid, (unsigned *)c->t_cost.p,
+    PG_CUDA(c, launch_near_plan(a, Bi, run, pair_cost, 1500.0f, grid,
+                                (unsigned *)((unsigned long long *)c->t_cost.p + ntiles),
+                                (unsigned long long *)c->t_cost.p,
                                 (unsigned char *)c->t_dense.p, (long long *)c->t_start.p, near, c->stream));
     c->last_launches += 3;
     return PG_OK;

@@ -548,25 +548,29 @@ __global__ void k_bw_combine(const double4 *__restrict__ part, const unsigned *_
                              double *__restrict__ dx, double *__restrict__ dm, NearCombine near)
 {
     long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (p >= n) return;
-    long long t = p / kBiB;
+    const bool in = p < n;
+    if (!in && !near.start) return;
+    long long t = (in ? p : n - 1) / kBiB;
     int li = (int)(p % kBiB);
     double gx = 0, gy = 0, gz = 0, gm = 0;
     if (near.start && *near.near) {
         const long long *start = near.start;
-        for (long long b = plan_first(start, near.grid, t * near.nch);
-             b < near.grid && start[b] < (t + 1) * near.nch; ++b) {
-            if (start[b + 1] <= start[b]) continue;
-            const double4 v = part[(size_t)(t + b) * kBiB + li];
+        int b0, b1;
+        plan_ctas(start, near.grid, t * near.nch, (t + 1) * near.nch, b0, b1);
+#pragma unroll 8
+        for (int b = b0; b < b1; ++b) {
+            if (!in || start[b + 1] <= start[b]) continue;
+            const double4 v = ldg_d4(part + (size_t)(t + b) * kBiB + li);
             gx += v.x; gy += v.y; gz += v.z; gm += v.w;
         }
-    } else if (njsub > 0) {
+    } else if (in && njsub > 0) {
         long long bf = sk_owner(t * njsub, grid, W), bl = sk_owner((t + 1) * njsub - 1, grid, W);
         for (long long s = 0; s <= bl - bf; ++s) {
             double4 v = part[((size_t)t * slots + (size_t)s) * kBiB + li];
             gx += v.x; gy += v.y; gz += v.z; gm += v.w;
         }
     }
+    if (!in) return;
     long long k = perm ? (long long)perm[p] : p;
     dx[3 * k] = gx;
     dx[3 * k + 1] = gy;

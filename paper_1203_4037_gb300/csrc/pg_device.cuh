@@ -198,16 +198,20 @@ __device__ __forceinline__ void bulk_g2s(void *dst, const void *src, unsigned by
 }
 
 // ---------------------------------------------------------------- planned splits
-// the CTA of a culled run that holds unit u or starts last before it
-__device__ __forceinline__ long long plan_first(const long long *start, int grid, long long u)
+// Of a near-pair run: the CTAs that hold units of [u, v), for one range that
+// all threads of the block ask for: b0 the last that starts at or before u,
+// b1 past the last that starts before v (CTAs without units in between).
+__device__ __forceinline__ void plan_ctas(const long long *start, int grid, long long u, long long v, int &b0, int &b1)
 {
-    int lo = 0, hi = grid - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (start[mid] <= u) lo = mid;
-        else hi = mid - 1;
+    int n0 = 0, n1 = 0;
+    for (int q = 0; q < grid; q += blockDim.x) {
+        const int b = q + threadIdx.x;
+        const long long s = b < grid ? start[b] : v;
+        n0 += __syncthreads_count(s <= u && b < grid);
+        n1 += __syncthreads_count(s < v);
     }
-    return lo;
+    b0 = n0 > 0 ? n0 - 1 : 0;
+    b1 = n1;
 }
 
 // ---------------------------------------------------------------- misc

@@ -303,13 +303,14 @@ cudaError_t launch_near_backward(const NearArgs &a, int grid, size_t smem, cudaS
 // against the boxes of its warps' runs (run i each); the plan cuts the total
 // cost into grid equal ranges of consecutive units. pair_cost: clocks of one
 // record against one run, unit_cost: clocks of a unit that keeps nothing.
-// Fills cost (ntiles words), dense (ntiles bytes), start (grid + 1) and near:
+// Fills cost and prefix (ntiles words), dense (ntiles bytes), start (grid + 1) and near:
 // 1 where the tiles' mean kept share (of each tile's worst warp) is below
 // kNearShare, else 0, and the all-pairs kernel runs instead (65536 Plummer:
 // at a share of 0.85 the near kernel took 3.1 ms, the all-pairs kernel 2.8).
 constexpr float kNearShare = 0.5f;
 cudaError_t launch_near_plan(const NearArgs &a, int Bi, int run, float pair_cost, float unit_cost, int grid,
-                             unsigned *cost, unsigned char *dense, long long *start, int *near, cudaStream_t st);
+                             unsigned *cost, unsigned long long *prefix, unsigned char *dense, long long *start,
+                             int *near, cudaStream_t st);
 // a step through nch units that spreads neighbours (coprime to nch)
 int near_stride(int nch);
 // records rounded to FP32

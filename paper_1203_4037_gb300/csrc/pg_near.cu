@@ -594,15 +594,19 @@ __global__ void __launch_bounds__(kNT) k_near_backward(NearArgs a)
 }
 
 // ---------------------------------------------------------------- split
-// One CTA per tile, one warp per run of `run` i-particles: each warp takes
-// its run's box and counts the sampled j records within r_cut of it.
-constexpr int kCostSample = 4096;      // records sampled: 1 % of the j kept is then 41 +- 6
+// One CTA per tile, one warp per run of `run` i-particles: each warp takes its
+// run's box, then every thread counts its sampled j records within r_cut of
+// each box.
+constexpr int kCostSample = 2048;      // records sampled: 1 % of the j kept is then 20 +- 4.5
+constexpr int kCostWarps = 4;
 
-__global__ void k_near_cost(NearArgs a, int Bi, int run, float pair_cost, float unit_cost,
-                            unsigned *__restrict__ cost, unsigned char *__restrict__ dense)
+__global__ void __launch_bounds__(32 * kCostWarps) k_near_cost(NearArgs a, int Bi, int run, float pair_cost,
+                                                               float unit_cost, unsigned *__restrict__ cost,
+                                                               unsigned char *__restrict__ dense)
 {
-    __shared__ float part[32];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    __shared__ float box[kCostWarps][6];
+    __shared__ int hits[kCostWarps];
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     const long long t = blockIdx.x;
     const float inf = __int_as_float(0x7f800000);
     float l[3] = {inf, inf, inf}, h[3] = {-inf, -inf, -inf};
@@ -618,92 +622,101 @@ __global__ void k_near_cost(NearArgs a, int Bi, int run, float pair_cost, float 
             l[c] = fminf(l[c], __shfl_xor_sync(0xffffffffu, l[c], o));
             h[c] = fmaxf(h[c], __shfl_xor_sync(0xffffffffu, h[c], o));
         }
-    const bool all = isinf(a.ext[t].x);
-    const long long step = (a.nj + kCostSample - 1) / kCostSample;
-    const long long ns = (a.nj + step - 1) / step;
-    int hits = 0;
-    for (long long q = lane; q < ns; q += 32) {
-        const float4 j = a.jf[q * step];
-        const float dx = fmaxf(fmaxf(l[0] - j.x, j.x - h[0]), 0.0f);
-        const float dy = fmaxf(fmaxf(l[1] - j.y, j.y - h[1]), 0.0f);
-        const float dz = fmaxf(fmaxf(l[2] - j.z, j.z - h[2]), 0.0f);
-        if (all || !(dx * dx + dy * dy + dz * dz > a.r_cut * a.r_cut)) ++hits;
+    if (lane == 0) {
+        for (int c = 0; c < 3; ++c) { box[w][c] = l[c]; box[w][3 + c] = h[c]; }
+        hits[w] = 0;
     }
-    for (int o = 16; o; o >>= 1) hits += __shfl_xor_sync(0xffffffffu, hits, o);
-    if (lane == 0) part[w] = ns > 0 ? (float)hits / (float)ns : 0.0f;
     __syncthreads();
-    if (threadIdx.x == 0) {
+    const bool all = isinf(a.ext[t].x);
+    const long long step = (a.nj + kCostSample - 1) / kCostSample, ns = (a.nj + step - 1) / step;
+    const float lim = a.r_cut * a.r_cut;
+    int n[kCostWarps] = {};
+#pragma unroll 4
+    for (long long q = tid; q < ns; q += 32 * kCostWarps) {
+        const float4 j = a.jf[q * step];
+#pragma unroll
+        for (int k = 0; k < kCostWarps; ++k) {
+            const float dx = fmaxf(fmaxf(box[k][0] - j.x, j.x - box[k][3]), 0.0f);
+            const float dy = fmaxf(fmaxf(box[k][1] - j.y, j.y - box[k][4]), 0.0f);
+            const float dz = fmaxf(fmaxf(box[k][2] - j.z, j.z - box[k][5]), 0.0f);
+            if (all || !(dx * dx + dy * dy + dz * dz > lim)) ++n[k];
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < kCostWarps; ++k) {
+        const int v = __reduce_add_sync(0xffffffffu, n[k]);
+        if (lane == 0) atomicAdd(&hits[k], v);
+    }
+    __syncthreads();
+    if (tid == 0) {
         // the CTA's barriers make its slowest warp set the time
-        float f = 0.0f;
-        for (int q = 0; q < (int)(blockDim.x >> 5); ++q) f = fmaxf(f, part[q]);
+        int m = 0;
+        for (int k = 0; k < kCostWarps; ++k) m = max(m, hits[k]);
+        const float f = ns > 0 ? (float)m / (float)ns : 0.0f;
         cost[t] = (unsigned)(unit_cost + f * (float)a.unit * pair_cost) + 1u;
         dense[t] = f > 0.8f;
     }
 }
 
-// Scans the tiles' costs and places the CTAs' first units: CTA b starts at
-// cost b C / grid, in its tile at the unit that cost falls in.
+// Scans the tiles' costs (per unit, times nch units) into prefix, then places
+// the CTAs' first units: CTA b starts at cost b C / grid, in the tile that
+// holds it at the unit it falls in.
 __global__ void __launch_bounds__(1024) k_near_split(const unsigned *__restrict__ cost, int ntiles, int nch, int grid,
-                                                     double all_near, long long *__restrict__ start,
+                                                     double all_near, u64 *prefix, long long *__restrict__ start,
                                                      int *__restrict__ near)
 {
-    __shared__ unsigned long long wsum[32], tot;
+    __shared__ u64 wsum[32];
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-    auto scan = [&](unsigned long long v, unsigned long long &total) {   // exclusive, over the block
-        unsigned long long x = v;
+    u64 base = 0;
+    for (int t0 = 0; t0 < ntiles; t0 += 1024) {
+        const u64 c = t0 + tid < ntiles ? (u64)cost[t0 + tid] * nch : 0ull;
+        u64 x = c;
         for (int o = 1; o < 32; o <<= 1) {
-            const unsigned long long y = __shfl_up_sync(0xffffffffu, x, o);
+            const u64 y = __shfl_up_sync(0xffffffffu, x, o);
             if (lane >= o) x += y;
         }
-        __syncthreads();
         if (lane == 31) wsum[w] = x;
         __syncthreads();
-        unsigned long long add = 0, all = 0;
-        for (int q = 0; q < 32; ++q) {
-            if (q < w) add += wsum[q];
-            all += wsum[q];
+        const u64 mine = wsum[lane];
+        u64 y = mine;
+        for (int o = 1; o < 32; o <<= 1) {
+            const u64 z = __shfl_up_sync(0xffffffffu, y, o);
+            if (lane >= o) y += z;
         }
-        total = all;
-        return add + x - v;
-    };
-    unsigned long long C = 0;
-    for (int t0 = 0; t0 < ntiles; t0 += 1024) {
-        unsigned long long all;
-        (void)scan(t0 + tid < ntiles ? (unsigned long long)cost[t0 + tid] * nch : 0ull, all);
-        C += all;
+        const u64 before = __shfl_sync(0xffffffffu, y - mine, w), total = __shfl_sync(0xffffffffu, y, 31);
+        if (t0 + tid < ntiles) prefix[t0 + tid] = base + before + x - c;
+        base += total;
+        __syncthreads();
     }
+    const u64 C = base;
     if (tid == 0) {
-        tot = C;
         *near = (double)C < kNearShare * all_near;
+        start[grid] = (long long)ntiles * nch;
     }
-    __syncthreads();
-    C = tot;
-    unsigned long long base = 0;
-    for (int t0 = 0; t0 < ntiles; t0 += 1024) {
-        const int t = t0 + tid;
-        const unsigned long long c = t < ntiles ? cost[t] : 0ull;
-        unsigned long long all;
-        const unsigned long long lo = base + scan(c * nch, all), hi = lo + c * nch;
-        // the CTAs that start in this tile: lo <= b C / grid < hi
-        if (t < ntiles)
-            for (long long b = (long long)((lo * grid + C - 1) / C); b < grid && (unsigned long long)b * C / grid < hi; ++b)
-                if ((unsigned long long)b * C / grid >= lo)
-                    start[b] = (long long)t * nch + (long long)(((unsigned long long)b * C / grid - lo) / c);
-        base += all;
+    for (int b = tid; b < grid; b += 1024) {
+        const u64 at = (u64)b * C / (unsigned)grid;
+        int lo = 0, hi = ntiles - 1;           // the last tile that starts at or before `at`
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (prefix[mid] <= at) lo = mid;
+            else hi = mid - 1;
+        }
+        start[b] = (long long)lo * nch + (long long)((at - prefix[lo]) / cost[lo]);
     }
-    if (tid == 0) start[grid] = (long long)ntiles * nch;
 }
 
 }  // namespace
 
 cudaError_t launch_near_plan(const NearArgs &a, int Bi, int run, float pair_cost, float unit_cost, int grid,
-                             unsigned *cost, unsigned char *dense, long long *start, int *near, cudaStream_t st)
+                             unsigned *cost, u64 *prefix, unsigned char *dense, long long *start, int *near,
+                             cudaStream_t st)
 {
     if (a.ntiles <= 0 || grid <= 0) return cudaSuccess;
-    k_near_cost<<<a.ntiles, Bi / run * 32, 0, st>>>(a, Bi, run, pair_cost, unit_cost, cost, dense);
+    if (Bi != run * kCostWarps) return cudaErrorInvalidValue;
+    k_near_cost<<<a.ntiles, 32 * kCostWarps, 0, st>>>(a, Bi, run, pair_cost, unit_cost, cost, dense);
     // the cost if every warp kept everything
     const double all = (double)a.ntiles * a.nch * ((double)a.unit * pair_cost + unit_cost);
-    k_near_split<<<1, 1024, 0, st>>>(cost, a.ntiles, a.nch, grid, all, start, near);
+    k_near_split<<<1, 1024, 0, st>>>(cost, a.ntiles, a.nch, grid, all, prefix, start, near);
     return cudaGetLastError();
 }
 
