@@ -185,7 +185,7 @@ __global__ void __launch_bounds__(kNT, MinBlocks<NP, TABLE, DF>::value) k_allpai
     const long long G = gridDim.x;
     const long long b = blockIdx.x;
     const long long u0 = b * a.W / G, u1 = (b + 1) * a.W / G;
-    if (u0 >= u1 || (TABLE && a.skip && *a.skip)) return;
+    if (u0 >= u1 || ((TABLE || DF) && a.skip && *a.skip)) return;
 
     if (tid == 0) {
         mbar_init(&bar[0], 1);
@@ -558,6 +558,7 @@ cudaError_t launch_allpairs(const AllPairsArgs &a, int grid, int np, bool table,
 __global__ void k_combine(CombineArgs c)
 {
     long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    if (c.skip && *c.skip) return;
     const bool in = p < c.ni;
     if (!in && !c.start) return;
     long long t = (in ? p : c.ni - 1) / c.Bi;
@@ -599,6 +600,7 @@ constexpr int kWideThreads = 128;
 
 __global__ void __launch_bounds__(kWideThreads) k_combine_wide(CombineArgs c)
 {
+    if (c.skip && *c.skip) return;
     __shared__ double4 wsum[kWideThreads / 32];
     const long long p = blockIdx.x;
     const int lane = threadIdx.x & 31;

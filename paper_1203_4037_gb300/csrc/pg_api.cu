@@ -155,6 +155,13 @@ struct pg_ctx {
     long long jhl_n = -1;         // j records in g_jhl as double-float pairs (-1: stale)
     long long ihl_n = -1;         // i-particles in g_ihl as double-float pairs, caller order (-1: stale)
 
+    // Newton all pairs on the tensor cores: j digits and masses (of tc_n
+    // records, -1: stale), geometry and flag words, i digits
+    DevBuf tc_dig, tc_mass, tc_geo, tc_idig;
+    long long tc_n = -1;
+    bool graph_tc = false;        // the captured run reads the j digits
+    const int *skip = nullptr;    // set while the run's stand-in is enqueued: it runs where this word is zero
+
     // backward
     DevBuf bw_wj, bw_wt, bw_dv;
 
@@ -308,6 +315,7 @@ void drop_graph(pg_ctx *c)
     c->gexec = nullptr;
     c->gkey.clear();
     c->graph_jhl = false;
+    c->graph_tc = false;
 }
 
 long long nj_of(const pg_ctx *c) { return c->nj_n >= 0 ? c->nj_n : c->nj_hw; }
@@ -510,7 +518,8 @@ void pg_destroy(pg_ctx *c)
                       &c->c_wrapped, &c->c_xs, &c->c_xo, &c->c_perm, &c->c_start, &c->c_jcount,
                       &c->c_icount, &c->c_ioff,
                       &c->c_items_raw, &c->c_items, &c->c_pairs, &c->n_part, &c->bw_wj,
-                      &c->bw_wt, &c->bw_dv, &c->tickets, &c->t_ext, &c->j_f32, &c->t_cost, &c->t_dense, &c->t_start};
+                      &c->bw_wt, &c->bw_dv, &c->tickets, &c->t_ext, &c->j_f32, &c->t_cost, &c->t_dense, &c->t_start,
+                      &c->tc_dig, &c->tc_mass, &c->tc_geo, &c->tc_idig};
     for (DevBuf *b : bufs) free_dev(*b);
     for (DevBuf &b : c->tb) free_dev(b);
     for (DevBuf *b : {&c->pm_rec, &c->pm_x, &c->pm_m, &c->pm_acc, &c->pm_pot}) free_dev(*b);
@@ -953,6 +962,7 @@ int pg_set_j(pg_ctx *c, long long adr, long long nj, const double *x, const doub
     PG_CUDA(c, launch_pack_j(dx, dx + 3 * nj, (double4 *)c->jrec.p + adr, nj, c->stream));
     c->nj_hw = std::max(c->nj_hw, adr + nj);
     c->jhl_n = -1;
+    c->tc_n = -1;
     return PG_OK;
 }
 
@@ -968,6 +978,7 @@ int pg_set_j_rec_dev(pg_ctx *c, long long adr, long long nj, const double *rec)
                                cudaMemcpyDeviceToDevice, c->stream));
     c->nj_hw = std::max(c->nj_hw, adr + nj);
     c->jhl_n = -1;
+    c->tc_n = -1;
     return PG_OK;
 }
 
@@ -982,6 +993,7 @@ int pg_set_j_dev(pg_ctx *c, long long adr, long long nj, const double *x, const 
     PG_CUDA(c, launch_pack_j(x, m, (double4 *)c->jrec.p + adr, nj, c->stream));
     c->nj_hw = std::max(c->nj_hw, adr + nj);
     c->jhl_n = -1;
+    c->tc_n = -1;
     return PG_OK;
 }
 
@@ -1483,7 +1495,7 @@ int enqueue_allpairs(pg_ctx *c, const Plan &p, double *acc, double *pot)
             return rc;
         a.jhl = (const float4 *)c->g_jhl.p;
     }
-    a.skip = na.near;
+    a.skip = near ? na.near : c->skip;
     a.ni = p.ni;
     a.nj = p.nj;
     a.ntiles = p.ntiles;
@@ -1518,6 +1530,7 @@ int enqueue_allpairs(pg_ctx *c, const Plan &p, double *acc, double *pot)
     cb.smax_slots = p.slots;
     cb.grid = std::max(p.grid, 1);
     cb.W = std::max<long long>(p.W, 1);
+    cb.skip = c->skip;
     cb.start = na.start;
     cb.near = na.near;
     cb.nch = na.nch;
@@ -1739,6 +1752,8 @@ bool use_narrow(const pg_ctx *c)
     return c->ni > 0 && c->ni <= 4096 && nj_of(c) >= 64 * c->ni;
 }
 
+int pack_j_for(pg_ctx *c, long long nj);   // below
+
 int enqueue_narrow(pg_ctx *c, double *acc, double *pot)
 {
     int rc;
@@ -1791,9 +1806,10 @@ int enqueue_narrow(pg_ctx *c, double *acc, double *pot)
     PG_CUDA(c, launch_narrow_prep((const double4 *)c->xi.p, ni, Bi, nic, (double4 *)c->g_ctr.p,
                                   (float4 *)c->g_ihl.p, (int *)c->g_queue.p, c->stream));
     c->ihl_n = ni;
-    if ((rc = pack_j_hilo(c, nj))) return rc;
+    if ((rc = pack_j_for(c, nj))) return rc;
     c->last_launches += 1;
     GroupArgs g = group_args(c);
+    g.skip = c->skip;
     g.xi = (const double4 *)c->xi.p;
     g.jrec = (const double4 *)c->jrec.p;
     g.j_off = nullptr;
@@ -1826,9 +1842,111 @@ int enqueue_narrow(pg_ctx *c, double *acc, double *pot)
     cb.accscale = g.accscale;
     cb.acc = acc;
     cb.pot = pot;
+    cb.skip = c->skip;
     PG_CUDA(c, launch_group_partials_combine(cb, (int)nch, c->stream));
     c->last_launches += 1;
     c->last_slots = nch;
+    return PG_OK;
+}
+
+// the double-float j records of a run that may stand in for another: packed
+// on every run where that one cannot run (so never counted as packed)
+int pack_j_for(pg_ctx *c, long long nj)
+{
+    if (!c->skip) return pack_j_hilo(c, nj);
+    if (c->jhl_n == nj && !c->capturing) return PG_OK;
+    PG_CUDA(c, launch_pack_hilo((const double4 *)c->jrec.p, nj, (float4 *)c->g_jhl.p, c->stream, c->skip));
+    c->last_launches += 1;
+    return PG_OK;
+}
+
+// The tensor-core path (pg_tc.cu): Newton runs of the default shape that
+// would difference in double-float, with enough pairs for its preparation and
+// the stand-in's empty launches. Whether this call's values fit its fixed
+// point (every i within the j-set's cube, eps / cube side within 1e-9 ...)
+// is known on the device only: the double-float path is enqueued behind it
+// and runs where they do not. From 48 i on: fewer leave most of a 32- or
+// 64-particle tile empty (2^20 j, kernel: 16 i 25 us, as the warp-mode
+// kernel's 25; 64 i 41 against 72; 1000 i 460 against 840).
+bool use_tc(const pg_ctx *c)
+{
+    if (c->mode != PG_NEWTON || use_ext(c) || c->np || c->split || c->ctas_per_sm || c->path != PG_PATH_AUTO ||
+        c->diff_mode == PG_DIFF_SINGLE || !c->packed)
+        return false;
+    const long long ni = c->ni, nj = nj_of(c);
+    if (ni < 48 || nj < 4096 || ni * nj < (1LL << 24)) return false;
+    return use_narrow(c) || (tiled_df(c, ni, nj) && ni * nj >= (1LL << 28));
+}
+
+int pack_tc(pg_ctx *c, long long nj)
+{
+    if (c->tc_n == nj) return PG_OK;
+    unsigned long long *words = (unsigned long long *)c->tc_geo.p;
+    PG_CUDA(c, launch_tc_pack((const double4 *)c->jrec.p, nj, words, (TcGeo *)(words + 10),
+                              (unsigned char *)c->tc_dig.p, (float *)c->tc_mass.p, c->stream));
+    c->last_launches += 2;
+    c->tc_n = nj;
+    return PG_OK;
+}
+
+int enqueue_tc(pg_ctx *c, double *acc, double *pot)
+{
+    int rc;
+    const long long ni = c->ni, nj = nj_of(c);
+    const int Bi = tc_bi(ni), njt = tc_jtiles(nj);
+    const long long ntiles = (ni + Bi - 1) / Bi, W = ntiles * njt;
+    const int grid = (int)std::min<long long>(c->sms, W), slots = tc_slots(ntiles, njt, W, grid);
+    const bool fresh = c->tc_geo.cap == 0;
+    if ((rc = ensure(c, c->tc_geo, 10 * 8 + sizeof(TcGeo) + 16)) || (rc = ensure(c, c->tc_dig, tc_dig_bytes(nj))) ||
+        (rc = ensure(c, c->tc_mass, (size_t)njt * 128 * sizeof(float))) ||
+        (rc = ensure(c, c->tc_idig, tc_dig_bytes(ni))) ||
+        (rc = ensure(c, c->part, (size_t)ntiles * slots * Bi * sizeof(double4))))
+        return rc;
+    if (fresh) PG_CUDA(c, cudaMemsetAsync(c->tc_geo.p, 0, c->tc_geo.cap, c->stream));
+    unsigned long long *words = (unsigned long long *)c->tc_geo.p;   // 8: box, 1: the i flags, 1: the verdict
+    TcArgs a{};
+    a.dig = (const unsigned char *)c->tc_dig.p;
+    a.mass = (const float *)c->tc_mass.p;
+    a.idig = (const unsigned char *)c->tc_idig.p;
+    a.geo = (const TcGeo *)(words + 10);
+    int *ok = (int *)(words + 9);
+    a.ok = ok;
+    a.ni = ni;
+    a.W = W;
+    a.njt = njt;
+    a.slots = slots;
+    a.part = (double4 *)c->part.p;
+    a.status = (int *)c->status.p;
+    if (c->capturing) c->graph_tc = true;
+    else if ((rc = pack_tc(c, nj))) return rc;
+    PG_CUDA(c, launch_tc_prep((const double4 *)c->xi.p, ni, (float)(c->eps * c->eps), (TcGeo *)(words + 10),
+                              (unsigned char *)c->tc_idig.p, (unsigned *)(words + 8), ok, c->stream));
+    if (c->timing) PG_CUDA(c, record_timing(c, c->tk0));
+    PG_CUDA(c, launch_tc(a, grid, c->stream));
+    const bool timing = c->timing;
+    PG_CUDA(c, launch_tc_combine(a, grid, c->self, c->self_off, acc, pot, c->stream));
+    c->last_launches += 3;
+    // where the values do not fit: the double-float path
+    c->skip = ok;
+    c->timing = false;
+    if (use_narrow(c)) {
+        rc = enqueue_narrow(c, acc, pot);
+    } else {
+        Plan p;
+        plan_allpairs(c, p);
+        rc = enqueue_allpairs(c, p, acc, pot);
+    }
+    c->skip = nullptr;
+    c->timing = timing;
+    if (rc) return rc;
+    if (timing) PG_CUDA(c, record_timing(c, c->tk1));
+    c->timed = timing;
+    c->last_np = Bi / 2;
+    c->last_df = true;
+    c->last_split = 1;
+    c->last_pairs = ni * nj;
+    c->last_grid = grid;
+    c->last_slots = std::max(slots, 2);
     return PG_OK;
 }
 
@@ -2372,6 +2490,12 @@ int enqueue_run(pg_ctx *c, double *acc, double *pot)
         c->last_launches += launches;
         return PG_OK;
     }
+    {
+        Plan p;
+        plan_allpairs(c, p);
+        int nchunk = 0, jchunk = 0;
+        if (use_tc(c) && (use_narrow(c) || !use_small(c, p, nchunk, jchunk))) return enqueue_tc(c, acc, pot);
+    }
     if (use_narrow(c)) return enqueue_narrow(c, acc, pot);
     Plan p;
     plan_allpairs(c, p);
@@ -2439,6 +2563,9 @@ int run_into(pg_ctx *c, double *acc, double *pot)
         PG_CUDA(c, launch_pack_hilo((const double4 *)c->jrec.p, nj_of(c), (float4 *)c->g_jhl.p,
                                     c->stream));
         c->jhl_n = nj_of(c);
+    }
+    if (c->graph_tc) {
+        if ((rc = pack_tc(c, nj_of(c)))) return rc;
     }
     PG_CUDA(c, cudaGraphLaunch(c->gexec, c->stream));
     return PG_OK;
@@ -2727,6 +2854,8 @@ int pg_tune(pg_ctx *c)
     };
     const int nps[3] = {1, 2, 4};
     const int shapes[4][2] = {{kGroupsTJ, kGroupsNT}, {256, 128}, {1024, 256}, {512, 256}};
+    // the library's own choice (which may be a path the fixed shapes do not take)
+    if (!groups_path && best_np == 0) trial(0, c->packed, 0, 0, c->g_tj, c->g_nt);
     for (int np : nps) {
         if (rc) break;
         if (narrow) {

@@ -892,6 +892,9 @@ template <int NPMAX, bool TABLE, bool CELL, bool EXT, bool HL = false, bool DF =
           int NT = kNT>
 __global__ void __launch_bounds__(NT) k_groups(GroupArgs a)
 {
+    if constexpr (DF) {
+        if (a.skip && *a.skip) return;
+    }
     constexpr int kW = GroupWords<DF>::value;
     static_assert(TJ % NT == 0 && NT % 32 == 0, "j tile and block size");
     extern __shared__ __align__(128) unsigned char smem[];
@@ -978,6 +981,9 @@ constexpr int kWMinBlocks = 2;     // resident blocks per SM wanted (register ca
 template <bool TABLE, bool CELL, bool EXT, bool HL = false, bool DF = false>
 __global__ void __launch_bounds__(kWNT, kWMinBlocks) k_groups_warp(GroupArgs a)
 {
+    if constexpr (DF) {
+        if (a.skip && *a.skip) return;
+    }
     constexpr int kW = GroupWords<DF>::value;
     extern __shared__ __align__(128) unsigned char smem[];
     u64 *wcvt = reinterpret_cast<u64 *>(smem);                             // [warps][kW kWarpTJ]
@@ -1267,6 +1273,7 @@ constexpr int kCombineThreads = 128;
 __global__ void __launch_bounds__(kCombineThreads)
 k_group_partials_combine(CombineArgs c, int nchunks)
 {
+    if (c.skip && *c.skip) return;
     __shared__ double4 wsum[kCombineThreads / 32];
     const long long i = blockIdx.x;
     const int t = threadIdx.x, lane = t & 31;
@@ -1316,17 +1323,18 @@ __device__ __forceinline__ void pack_hilo_one(const double4 *__restrict__ in, lo
                                  (float)(v.z - (double)hz), (float)v.w);
 }
 
-__global__ void k_pack_hilo(const double4 *__restrict__ in, long long n, float4 *__restrict__ out)
+__global__ void k_pack_hilo(const double4 *__restrict__ in, long long n, float4 *__restrict__ out,
+                            const int *__restrict__ skip)
 {
     long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (i >= n) return;
+    if (i >= n || (skip && *skip)) return;
     pack_hilo_one(in, i, out);
 }
 
-cudaError_t launch_pack_hilo(const double4 *in, long long n, float4 *out, cudaStream_t st)
+cudaError_t launch_pack_hilo(const double4 *in, long long n, float4 *out, cudaStream_t st, const int *skip)
 {
     if (n <= 0) return cudaSuccess;
-    k_pack_hilo<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(in, n, out);
+    k_pack_hilo<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(in, n, out, skip);
     return cudaGetLastError();
 }
 

@@ -75,6 +75,7 @@ struct CombineArgs {
     const long long *start = nullptr;   // a near-pair run's split (NearArgs), used where *near is nonzero
     const int *near = nullptr;
     int nch = 0, near_grid = 0;
+    const int *skip = nullptr;       // set: a nonzero word here means another kernel does this run
     const int *fail_nan = nullptr;   // set: a nonzero word here (a force kernel's failure
                                      // status) makes every output NaN
 };
@@ -151,6 +152,7 @@ struct GroupArgs {
     double accscale;
     double *acc, *pot;
     int *status;
+    const int *skip = nullptr;   // double-float items: a nonzero word here means another kernel does this run
     float4 *hl = nullptr;  // Newton lists: the sums as FP32 (hi, lo) pairs, two float4 per i
                            // (x, y, z, phi), converted by the finish kernel (nullptr: FP64 out)
 };
@@ -262,6 +264,41 @@ int pm_solve(PmState *s, const float *rho, const double4 *tgt, long long nt, dou
 // half extents of each tile's box
 cudaError_t launch_tile_prep(const double4 *xi, const unsigned *perm, long long n, int Bi,
                              double4 *xi_tiled, double4 *ctr, cudaStream_t st, float4 *ext = nullptr);
+// ---------------------------------------------------------------- tensor cores
+// Newton all pairs with the differences formed by tcgen05.mma (pg_tc.cu)
+struct TcGeo {             // set on the device from the j-set
+    double cx, cy, cz;     // the cube's centre
+    double scale;          // position -> fixed point, 2^47 / R
+    double mscale;         // mass -> staged mass, 2^mexp
+    int e, mexp;           // R = 2^e
+    int ok;                // finite and in range
+    float e2;              // eps^2 in the kernel's unit (R 2^-23), set by each call's preparation
+};
+struct TcArgs {
+    const unsigned char *dig;   // j digits, tiles of 128 records
+    const float *mass;          // staged masses, padded with zeros
+    const unsigned char *idig;  // i digits, the same layout
+    const TcGeo *geo;
+    const int *ok;         // zero: this call's values do not fit, nothing runs
+    long long ni, W;       // i-particles; units, i tiles times j tiles
+    int njt, slots;        // j tiles; partial slots per i tile
+    double4 *part;         // [i tiles][slots][tc_bi]
+    int *status;
+};
+int tc_bi(long long ni);                   // i-particles per tile
+size_t tc_dig_bytes(long long n);
+int tc_jtiles(long long nj);
+int tc_slots(long long ntiles, int njt, long long W, int grid);
+// words: 8 u64, zero before the first call and kept so
+cudaError_t launch_tc_pack(const double4 *jrec, long long nj, unsigned long long *words, TcGeo *geo,
+                           unsigned char *dig, float *mass, cudaStream_t st);
+// words: 2, zero before the first call and kept so; ok: the verdict
+cudaError_t launch_tc_prep(const double4 *xi, long long ni, float eps2, TcGeo *geo, unsigned char *idig,
+                           unsigned *words, int *ok, cudaStream_t st);
+cudaError_t launch_tc(const TcArgs &a, int grid, cudaStream_t st);
+cudaError_t launch_tc_combine(const TcArgs &a, int grid, int self, long long self_off, double *acc, double *pot,
+                              cudaStream_t st);
+
 // ---------------------------------------------------------------- near pairs
 // The tabulated force on compact (sorted) i-tiles, pg_near.cu: g is exactly 0
 // from r_cut on, so each tile evaluates only the j within r_cut of its box.
@@ -341,7 +378,9 @@ cudaError_t launch_groups(const GroupArgs &g, int grid, int np, bool table, bool
 cudaError_t launch_groups_finish(const GroupArgs &g, cudaStream_t st);
 // one device-side bounded wait that nothing ends (the timeout path's self-test)
 cudaError_t launch_wait_selftest(int *status, unsigned long long limit_ns, cudaStream_t st);
-cudaError_t launch_pack_hilo(const double4 *in, long long n, float4 *out, cudaStream_t st);
+// skip: a nonzero word there leaves the records as they are
+cudaError_t launch_pack_hilo(const double4 *in, long long n, float4 *out, cudaStream_t st,
+                             const int *skip = nullptr);
 // narrow path: chunk centres (chunks of `chunk` i, nic of them), double-float
 // i records and the two work counters zeroed, in one launch
 cudaError_t launch_narrow_prep(const double4 *xi, long long ni, long long chunk, long long nic,

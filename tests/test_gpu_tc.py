@@ -1,0 +1,134 @@
+"""Newton runs of a few i-particles against many j with the differences formed
+on the tensor cores (the automatic choice from 48 i on), against the FP64
+oracle: the edges of its i tiles (32, 64) and j tiles (128), i spread over the
+whole system at 0.5 to 2 eps from j-particles, the self mode, masses of both
+signs and many magnitudes, graph replays with new positions, and values that
+do not fit its fixed point, where the double-float path stands in (i far
+outside the j-set, eps too small or too large for the range, non-finite
+records). Tolerances as for the double-float paths (median 2e-6, maximum
+1e-4)."""
+
+import numpy as np
+import pytest
+
+import gen
+from pgtest import assert_parity, need_cuda, rel_scalar, rel_vec
+
+pytestmark = pytest.mark.gpu
+
+EPS = 1e-3
+
+
+@pytest.fixture(scope="module")
+def pg():
+    return need_cuda()
+
+
+def run(pg, xi, xj, mj, eps, self_=False, off=0, path=0):
+    with pg.Context(0) as c:
+        c.set_allpairs_path(path)
+        c.set_eps(eps)
+        if self_:
+            c.set_self(True)
+            if off:
+                c.set_self_offset(off)
+        c.set_j(xj, mj)
+        c.set_i(xi)
+        c.run()
+        return (*c.get_force(len(xi)), c.info())
+
+
+def near_j(xj, ni, seed, eps):
+    rng = np.random.default_rng(seed)
+    u = rng.normal(size=(ni, 3))
+    u /= np.linalg.norm(u, axis=1, keepdims=True)
+    return xj[rng.choice(len(xj), size=ni, replace=False)] + u * (eps * rng.uniform(0.5, 2.0, ni))[:, None]
+
+
+def check(orc, a, p, xi, xj, mj, eps, skip=None):
+    ao, po = orc.newton(xi, xj, mj, eps, skip=skip)
+    assert_parity(rel_vec(a, ao), what="a")
+    assert_parity(rel_scalar(p, po), what="phi")
+
+
+# 349526 j against 48 i: the fewest that take the path (2^24 pairs)
+@pytest.mark.parametrize("ni, nj", [(48, 349526), (64, 262144), (65, 262145), (96, 200001), (512, 32769), (1000, 64000),
+                                    (4096, 262271)])
+def test_spread_sets(pg, orc, ni, nj):
+    xj, mj = gen.plummer_cube_mix(nj, 900 + nj % 97)
+    xi = near_j(xj, ni, ni, EPS)
+    a, p, info = run(pg, xi, xj, mj, EPS)
+    assert info["i_per_thread"] in (32, 64) and info["df"] == 1      # the tensor-core tiles
+    idx = np.arange(ni) if ni <= 512 else gen.sample_indices(ni, 400, 1)
+    check(orc, a[idx], p[idx], xi[idx], xj, mj, EPS)
+
+
+@pytest.mark.parametrize("off", [0, 777])
+def test_self_mode(pg, orc, off):
+    x, m = gen.plummer(70000, 31)
+    xi = x[off:off + 300]
+    a, p, info = run(pg, xi, x, m, 0.01, self_=True, off=off)
+    assert info["i_per_thread"] == 64
+    check(orc, a, p, xi, x, m, 0.01, skip=np.arange(off, off + 300, dtype=np.int64))
+
+
+def test_masses(pg, orc):
+    x, m = gen.plummer(90001, 5)
+    rng = np.random.default_rng(5)
+    m = m * 10.0 ** rng.uniform(-12, 3, len(m)) * rng.choice([-1.0, 1.0, 0.0], len(m), p=[0.1, 0.8, 0.1])
+    xi = gen.plummer(200, 6)[0]
+    a, p, info = run(pg, xi, x, m, 0.01)
+    assert info["i_per_thread"] == 64
+    ao, po = orc.newton(xi, x, m, 0.01)
+    # signs cancel: the error is held against the sums of magnitudes
+    aa, pa = orc.newton(xi, x, np.abs(m), 0.01)
+    assert np.max(np.abs(p - po) / np.abs(pa)) <= 1e-6
+    assert np.max(np.linalg.norm(a - ao, axis=1) / (np.abs(pa) / 0.01)) <= 1e-6
+
+
+def test_graph_replays_with_new_positions(pg, orc):
+    xj, mj = gen.plummer_cube_mix(60000, 12)
+    with pg.Context(0) as c:
+        c.set_eps(EPS)
+        c.set_graph(True)
+        for k in range(5):
+            y = xj * (1.0 + 0.1 * k)
+            xi = near_j(y, 300, k, EPS)
+            if k != 3:                  # call 3 keeps the j records of call 2
+                c.set_j(y, mj)
+                last = y
+            c.set_i(xi)
+            c.run()
+            a, p = c.get_force(300)
+            check(orc, a, p, xi, last, mj, EPS)
+
+
+@pytest.mark.parametrize("what", ["i outside", "eps small", "eps large", "j outlier", "i at the edge"])
+def test_values_that_do_not_fit(pg, orc, what):
+    xj, mj = gen.plummer(60000, 3)
+    xi = gen.plummer(300, 4)[0]
+    eps = EPS
+    if what == "i outside":
+        xi[7] = [500.0, -3.0, 2.0]
+    elif what == "i at the edge":
+        xi[7] = xj.max(axis=0) * 1.2
+    elif what == "eps small":
+        eps = 1e-12
+    elif what == "eps large":
+        eps = 1e8
+    else:
+        xj[11] = [1e9, 0.0, 0.0]
+    a, p, _ = run(pg, xi, xj, mj, eps)
+    check(orc, a, p, xi, xj, mj, eps)
+
+
+@pytest.mark.parametrize("which", ["x", "m", "xi"])
+def test_nonfinite_as_on_the_narrow_path(pg, which):
+    xj, mj = gen.plummer(60000, 3)
+    xi = gen.plummer(300, 4)[0]
+    {"x": xj, "m": mj, "xi": xi}[which][5] = np.nan
+    a, p, _ = run(pg, xi, xj, mj, EPS)
+    a2, p2, _ = run(pg, xi, xj, mj, EPS, path=pg.PG_PATH_NARROW)
+    assert np.array_equal(np.isnan(a), np.isnan(a2)) and np.array_equal(np.isnan(p), np.isnan(p2))
+    ok = np.isfinite(a2).all(axis=1)
+    assert np.array_equal(a[ok], a2[ok])
