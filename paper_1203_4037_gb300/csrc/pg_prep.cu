@@ -170,11 +170,13 @@ long long sort_tiles(long long n)
     return (n + kSortThreads * rounds - 1) / (kSortThreads * rounds);
 }
 
-// 32-bit words of SortScratch::hist: the look-back words (two of them each),
-// the digit counts and the tickets
+// 32-bit words of SortScratch::hist for sorts of up to n keys: the look-back
+// words (two of them each), the digit counts and the tickets (a set at the
+// switch to large tiles has more tiles than a somewhat larger one)
 size_t sort_hist_entries(long long n)
 {
-    return (size_t)kSortPasses * (512 * (size_t)sort_tiles(n) + 256 + 1) + 16;
+    const long long tiles = std::max(sort_tiles(n), sort_tiles(std::min(n, kSortSmall)));
+    return (size_t)kSortPasses * (512 * (size_t)tiles + 256 + 1) + 16;
 }
 
 // counts of every pass's digits, added to cnt[pass][256]

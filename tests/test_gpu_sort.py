@@ -51,3 +51,25 @@ def test_crowded_digits(pg, n):
     x = gen.uniform_sphere(n, 7, radius=1e-3)[0]
     x[:3] = [[0, 0, 0], [1, 1, 1], [1, 0, 0.5]]
     assert np.array_equal(order(pg, x), np.argsort(keys(x), kind="stable"))
+
+
+def test_more_cells_than_particles(pg, orc):
+    # the cell list sorts its particles (small tiles) and its items (as many
+    # as cells, large tiles) in one scratch
+    n, nc, E, F = 100000, 70, 3, 5
+    x, m = gen.clustered_box(n, 8)
+    r_cut = 1.0 / nc * 0.999
+    v = orc.table_values(E, F, r_cut, orc.SHAPE_GAUSS_SPLIT, [r_cut / 4.5, r_cut / 16])
+    with pg.Context(0) as c:
+        c.set_mode(pg.PG_TABLE)
+        c.set_table_values(v, r_cut, E, F)
+        c.set_self(True)
+        c.set_periodic(1.0)
+        a, _ = c.forces(x, x, m)
+    idx = gen.sample_indices(n, 500, 2)
+    G0, G1 = orc.table_from_values(E, F, v)
+    ao, amb = orc.table_forces(x[idx], x, m, E, F, r_cut, G0, G1, box=1.0, skip=idx, window=1e-6)
+    na = np.linalg.norm(ao, axis=1)
+    some = na > 0
+    assert np.max((np.maximum(np.linalg.norm(a[idx] - ao, axis=1) - amb, 0))[some] / na[some]) <= 1e-4
+    assert np.all(np.linalg.norm(a[idx][~some], axis=1) <= amb[~some])
