@@ -156,8 +156,8 @@ struct pg_ctx {
     long long ihl_n = -1;         // i-particles in g_ihl as double-float pairs, caller order (-1: stale)
 
     // Newton all pairs on the tensor cores: j digits and masses (of tc_n
-    // records, -1: stale), geometry and flag words, i digits
-    DevBuf tc_dig, tc_mass, tc_geo, tc_idig;
+    // records, -1: stale), geometry and flag words
+    DevBuf tc_dig, tc_geo;
     long long tc_n = -1;
     bool graph_tc = false;        // the captured run reads the j digits
     const int *skip = nullptr;    // set while the run's stand-in is enqueued: it runs where this word is zero
@@ -519,7 +519,7 @@ void pg_destroy(pg_ctx *c)
                       &c->c_icount, &c->c_ioff,
                       &c->c_items_raw, &c->c_items, &c->c_pairs, &c->n_part, &c->bw_wj,
                       &c->bw_wt, &c->bw_dv, &c->tickets, &c->t_ext, &c->j_f32, &c->t_cost, &c->t_dense, &c->t_start,
-                      &c->tc_dig, &c->tc_mass, &c->tc_geo, &c->tc_idig};
+                      &c->tc_dig, &c->tc_geo};
     for (DevBuf *b : bufs) free_dev(*b);
     for (DevBuf &b : c->tb) free_dev(b);
     for (DevBuf *b : {&c->pm_rec, &c->pm_x, &c->pm_m, &c->pm_acc, &c->pm_pot}) free_dev(*b);
@@ -1863,8 +1863,8 @@ int pack_j_for(pg_ctx *c, long long nj)
 // The tensor-core path (pg_tc.cu): Newton runs of the default shape that
 // would difference in double-float, with enough pairs for its preparation and
 // the stand-in's empty launches. Whether this call's values fit its fixed
-// point (every i within the j-set's cube, eps / cube side within 1e-9 ...)
-// is known on the device only: the double-float path is enqueued behind it
+// point (every i within the j-set's cube, eps within 2^-30 to 2^10 of its half
+// side) is known on the device only: the double-float path is enqueued behind it
 // and runs where they do not. From 48 i on: fewer leave most of a 32- or
 // 64-particle tile empty (2^20 j, kernel: 16 i 25 us, as the warp-mode
 // kernel's 25; 64 i 41 against 72; 1000 i 460 against 840).
@@ -1878,53 +1878,86 @@ bool use_tc(const pg_ctx *c)
     return use_narrow(c) || (tiled_df(c, ni, nj) && ni * nj >= (1LL << 28));
 }
 
+// tc_dig holds the j digits and, behind them, the staged masses
+float *tc_mass(const pg_ctx *c, long long nj) { return (float *)((char *)c->tc_dig.p + tc_dig_bytes(nj)); }
+
 int pack_tc(pg_ctx *c, long long nj)
 {
     if (c->tc_n == nj) return PG_OK;
     unsigned long long *words = (unsigned long long *)c->tc_geo.p;
     PG_CUDA(c, launch_tc_pack((const double4 *)c->jrec.p, nj, words, (TcGeo *)(words + 10),
-                              (unsigned char *)c->tc_dig.p, (float *)c->tc_mass.p, c->stream));
+                              (unsigned char *)c->tc_dig.p, tc_mass(c, nj), c->stream));
     c->last_launches += 2;
     c->tc_n = nj;
     return PG_OK;
+}
+
+// the path's memory: the geometry and flags (zeroed once), the j digits and
+// masses, and in part the partial sums with the i digits behind them
+struct TcShape {
+    int Bi, njt, grid, slots;
+    long long ntiles, W;
+    size_t part;          // bytes of partial sums
+};
+
+TcShape tc_shape(const pg_ctx *c)
+{
+    TcShape t;
+    t.Bi = tc_bi(c->ni);
+    t.njt = tc_jtiles(nj_of(c));
+    t.ntiles = (c->ni + t.Bi - 1) / t.Bi;
+    t.W = t.ntiles * t.njt;
+    t.grid = (int)std::min<long long>(c->sms, t.W);
+    t.slots = tc_slots(t.ntiles, t.njt, t.W, t.grid);
+    t.part = (size_t)t.ntiles * t.slots * t.Bi * sizeof(double4);
+    return t;
+}
+
+int tc_room(pg_ctx *c)
+{
+    int rc;
+    const TcShape t = tc_shape(c);
+    const size_t dig = tc_dig_bytes(nj_of(c)) + (size_t)t.njt * 128 * sizeof(float);
+    const size_t part = t.part + tc_dig_bytes(c->ni);
+    // a capture allocates nothing: it records the path the run before it took
+    if (c->capturing)
+        return c->tc_geo.cap && c->tc_dig.cap >= dig && c->part.cap >= part ? PG_OK : PG_ENOMEM;
+    if (c->tc_geo.cap == 0) {
+        if ((rc = ensure(c, c->tc_geo, 10 * 8 + sizeof(TcGeo) + 16))) return rc;
+        PG_CUDA(c, cudaMemsetAsync(c->tc_geo.p, 0, c->tc_geo.cap, c->stream));
+    }
+    if ((rc = ensure(c, c->tc_dig, dig))) return rc;
+    return ensure(c, c->part, part);
 }
 
 int enqueue_tc(pg_ctx *c, double *acc, double *pot)
 {
     int rc;
     const long long ni = c->ni, nj = nj_of(c);
-    const int Bi = tc_bi(ni), njt = tc_jtiles(nj);
-    const long long ntiles = (ni + Bi - 1) / Bi, W = ntiles * njt;
-    const int grid = (int)std::min<long long>(c->sms, W), slots = tc_slots(ntiles, njt, W, grid);
-    const bool fresh = c->tc_geo.cap == 0;
-    if ((rc = ensure(c, c->tc_geo, 10 * 8 + sizeof(TcGeo) + 16)) || (rc = ensure(c, c->tc_dig, tc_dig_bytes(nj))) ||
-        (rc = ensure(c, c->tc_mass, (size_t)njt * 128 * sizeof(float))) ||
-        (rc = ensure(c, c->tc_idig, tc_dig_bytes(ni))) ||
-        (rc = ensure(c, c->part, (size_t)ntiles * slots * Bi * sizeof(double4))))
-        return rc;
-    if (fresh) PG_CUDA(c, cudaMemsetAsync(c->tc_geo.p, 0, c->tc_geo.cap, c->stream));
+    const TcShape t = tc_shape(c);
     unsigned long long *words = (unsigned long long *)c->tc_geo.p;   // 8: box, 1: the i flags, 1: the verdict
     TcArgs a{};
     a.dig = (const unsigned char *)c->tc_dig.p;
-    a.mass = (const float *)c->tc_mass.p;
-    a.idig = (const unsigned char *)c->tc_idig.p;
+    a.mass = tc_mass(c, nj);
+    unsigned char *idig = (unsigned char *)c->part.p + t.part;
+    a.idig = idig;
     a.geo = (const TcGeo *)(words + 10);
     int *ok = (int *)(words + 9);
     a.ok = ok;
     a.ni = ni;
-    a.W = W;
-    a.njt = njt;
-    a.slots = slots;
+    a.W = t.W;
+    a.njt = t.njt;
+    a.slots = t.slots;
     a.part = (double4 *)c->part.p;
     a.status = (int *)c->status.p;
     if (c->capturing) c->graph_tc = true;
     else if ((rc = pack_tc(c, nj))) return rc;
     PG_CUDA(c, launch_tc_prep((const double4 *)c->xi.p, ni, (float)(c->eps * c->eps), (TcGeo *)(words + 10),
-                              (unsigned char *)c->tc_idig.p, (unsigned *)(words + 8), ok, c->stream));
+                              idig, (unsigned *)(words + 8), ok, c->stream));
     if (c->timing) PG_CUDA(c, record_timing(c, c->tk0));
-    PG_CUDA(c, launch_tc(a, grid, c->stream));
+    PG_CUDA(c, launch_tc(a, t.grid, c->stream));
     const bool timing = c->timing;
-    PG_CUDA(c, launch_tc_combine(a, grid, c->self, c->self_off, acc, pot, c->stream));
+    PG_CUDA(c, launch_tc_combine(a, t.grid, c->self, c->self_off, acc, pot, c->stream));
     c->last_launches += 3;
     // where the values do not fit: the double-float path
     c->skip = ok;
@@ -1941,12 +1974,12 @@ int enqueue_tc(pg_ctx *c, double *acc, double *pot)
     if (rc) return rc;
     if (timing) PG_CUDA(c, record_timing(c, c->tk1));
     c->timed = timing;
-    c->last_np = Bi / 2;
+    c->last_np = t.Bi / 2;
     c->last_df = true;
     c->last_split = 1;
     c->last_pairs = ni * nj;
-    c->last_grid = grid;
-    c->last_slots = std::max(slots, 2);
+    c->last_grid = t.grid;
+    c->last_slots = std::max(t.slots, 2);
     return PG_OK;
 }
 
@@ -2494,7 +2527,13 @@ int enqueue_run(pg_ctx *c, double *acc, double *pot)
         Plan p;
         plan_allpairs(c, p);
         int nchunk = 0, jchunk = 0;
-        if (use_tc(c) && (use_narrow(c) || !use_small(c, p, nchunk, jchunk))) return enqueue_tc(c, acc, pot);
+        if (use_tc(c) && (use_narrow(c) || !use_small(c, p, nchunk, jchunk))) {
+            // without room for the digits the double-float path runs alone
+            const int rc = tc_room(c);
+            if (rc == PG_OK) return enqueue_tc(c, acc, pot);
+            if (rc != PG_ENOMEM) return rc;
+            c->tc_n = -1;
+        }
     }
     if (use_narrow(c)) return enqueue_narrow(c, acc, pot);
     Plan p;

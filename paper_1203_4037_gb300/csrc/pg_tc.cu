@@ -17,7 +17,9 @@
 // a second adds the lower 24 bits' difference, rounded by the tensor core at
 // the last place of the result: d carries one rounding relative to |d|,
 // however far the i-particles are spread (measured: mean -3.2e-8, at most
-// 1.5e-7 relative, against 64 bits).
+// 1.5e-7 relative, against 64 bits). The sums take that mean back (kShort):
+// forces and potentials are then nearer to 64 bits than the double-float
+// kernel's (1048 i, 563704 j: 4.8e-8 and 2.3e-8 against 5.8e-8 and 2.5e-8).
 //
 // A CTA owns units (tile of 32 GI i, tile of 128 j), an equal contiguous
 // range of them. One thread copies the j tiles in (cp.async.bulk), two issue
@@ -52,6 +54,12 @@ constexpr int kDigBytes = kTcJ * 32;   // digits of a j tile
 constexpr int kSlotBytes = kDigBytes + kTcJ * 4;   // and its masses
 constexpr int kSums = 4 * kIW, kLaneSums = kSums / 32;
 constexpr int kFoldTiles = 128;        // j tiles per FP32 partial sum of a lane
+// The differences come out short by this on average (the tensor cores round
+// them toward zero), so the unit they are read in is longer by it. From the
+// signed errors of forces (2 kShort) and potentials (kShort) against 64
+// bits, 12 sets of 112 to 2080 i against 3e5 to 1e6 j: +4.7e-8 and +2.6e-8
+// without it
+constexpr double kShort = 2.5e-8;
 
 // GI groups of kIW i per CTA tile; the groups' warps (four each, one per TMEM
 // quadrant) share every j tile, with GI = 1 two streams take alternate tiles
@@ -533,7 +541,7 @@ __global__ void __launch_bounds__(256) k_tc_prep(const double4 *__restrict__ xi,
     __threadfence();
     const bool far = __ldcg(words) != 0;
     // eps in units of the upper digits' last place, u = R 2^-23
-    const double e2 = ldexp((double)eps2, 2 * (23 - g.e));
+    const double e2 = ldexp((double)eps2, 2 * (23 - g.e)) * ((1.0 - kShort) * (1.0 - kShort));
     const bool range = e2 >= 0x1p-14 && e2 <= 0x1p66;
     geo->e2 = (float)e2;
     *ok = g.ok && !far && range;
@@ -563,7 +571,8 @@ __global__ void __launch_bounds__(256) k_tc_combine(TcArgs a, int Bi, int grid, 
     const TcGeo &g = *a.geo;
     // the own pair as the loop added it: d = 0 exactly
     if (self) s[3] += (double)__fmul_rn(a.mass[i + self_off], rsq(g.e2));
-    const double fa = ldexp(1.0, 2 * (23 - g.e) - g.mexp), fp = ldexp(1.0, 23 - g.e - g.mexp);
+    const double fa = ldexp((1.0 - kShort) * (1.0 - kShort), 2 * (23 - g.e) - g.mexp),
+                 fp = ldexp(1.0 - kShort, 23 - g.e - g.mexp);
     acc[3 * i] = s[0] * fa;
     acc[3 * i + 1] = s[1] * fa;
     acc[3 * i + 2] = s[2] * fa;

@@ -132,3 +132,17 @@ def test_nonfinite_as_on_the_narrow_path(pg, which):
     assert np.array_equal(np.isnan(a), np.isnan(a2)) and np.array_equal(np.isnan(p), np.isnan(p2))
     ok = np.isfinite(a2).all(axis=1)
     assert np.array_equal(a[ok], a2[ok])
+
+
+@pytest.mark.parametrize("ni, nj", [(200, 100003), (2000, 131072)])
+def test_no_signed_error(pg, orc, ni, nj):
+    # the tensor cores round the differences toward zero; the unit they are
+    # read in makes up for the mean (2.6e-8 of a potential without that). A
+    # quarter of an FP32 ulp, 1.5e-8, is allowed for what depends on the set.
+    # Against the masses as the sums hold them (FP32: 1/100003 rounds by 3.9e-8)
+    xj, mj = gen.plummer(nj, ni)
+    xi = gen.plummer(ni, nj)[0]
+    _, p, info = run(pg, xi, xj, mj, EPS)
+    assert info["i_per_thread"] == 64
+    _, po = orc.newton(xi, xj, mj.astype(np.float32).astype(np.float64), EPS)
+    assert abs(np.mean(p / po - 1)) <= 1.5e-8
