@@ -2523,11 +2523,11 @@ int enqueue_run(pg_ctx *c, double *acc, double *pot)
         c->last_launches += launches;
         return PG_OK;
     }
-    {
+    if (use_tc(c)) {
         Plan p;
         plan_allpairs(c, p);
         int nchunk = 0, jchunk = 0;
-        if (use_tc(c) && (use_narrow(c) || !use_small(c, p, nchunk, jchunk))) {
+        if (use_narrow(c) || !use_small(c, p, nchunk, jchunk)) {
             // without room for the digits the double-float path runs alone
             const int rc = tc_room(c);
             if (rc == PG_OK) return enqueue_tc(c, acc, pot);

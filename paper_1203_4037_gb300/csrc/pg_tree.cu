@@ -851,34 +851,65 @@ __device__ __forceinline__ void place_emitters(const GroupWalkArgs &a, TreeMeta 
     __syncwarp();
 }
 
-// the fill pass of a recorded group: its cnt emitters from emit[first]
-// expanded into list entries from pos, in order
+// The fill pass of a recorded group: its cnt emitters from emit[first]
+// expanded into list entries from pos, in order. Bound by the latency of a
+// step's loads (the emitter, then a leaf's record) and, when each lane
+// stored its own run, by stores that touched a line per lane. So a lane
+// takes kExpand consecutive emitters (one scan per 32 * kExpand of them),
+// the entries are laid out in the warp's shared words (`stage`, kGwWords)
+// and go out 32 consecutive ones at a time; a step with more entries than
+// that (large nleaf) stores them lane by lane. 2^20 Plummer particles,
+// theta 0.75: 123 -> 80 us.
+constexpr int kExpand = 4;
+
 __device__ __forceinline__ void expand_emitters(const GroupWalkArgs &a, int first, int cnt, long long pos,
-                                                long long hi, int lane)
+                                                long long hi, unsigned *stage, int lane)
 {
-    for (int b = 0; b < cnt; b += 32) {
-        unsigned e = 0;
-        int p0 = 0;
-        if (b + lane < cnt) {
-            const unsigned code = a.emit[first + b + lane];
-            const int k = (int)(code & 0x7fffffffu);
-            if (code >> 31) {
-                e = (unsigned)a.npseudo;
-                p0 = (int)(a.n + (long long)a.npseudo * k);
-            } else {
-                const TreeNodeW nd = a.nodew[k];
-                e = (unsigned)nd.count;
-                p0 = nd.first;
+    for (int b = 0; b < cnt; b += 32 * kExpand) {
+        const int q0 = b + lane * kExpand;
+        unsigned code[kExpand], e[kExpand], sum = 0;
+        int p0[kExpand];
+#pragma unroll
+        for (int u = 0; u < kExpand; ++u) code[u] = q0 + u < cnt ? a.emit[(long long)first + q0 + u] : 0u;
+#pragma unroll
+        for (int u = 0; u < kExpand; ++u) {
+            const int k = (int)(code[u] & 0x7fffffffu);
+            e[u] = 0;
+            p0[u] = 0;
+            if (q0 + u < cnt) {
+                if (code[u] >> 31) {
+                    e[u] = (unsigned)a.npseudo;
+                    p0[u] = (int)(a.n + (long long)a.npseudo * k);
+                } else {
+                    e[u] = (unsigned)a.nodew[k].count;
+                    p0[u] = a.nodew[k].first;
+                }
+            }
+            sum += e[u];
+        }
+        const unsigned ei = warp_incl_scan(sum, lane);
+        const unsigned total = __shfl_sync(0xffffffffu, ei, 31);
+        unsigned o = ei - sum;
+        if (pos + total > hi) {
+            if (lane == 0) report(a.status, kStatusBadIndex, 13);
+        } else if (total <= (unsigned)kGwWords) {
+#pragma unroll
+            for (int u = 0; u < kExpand; ++u) {
+                for (unsigned t = 0; t < e[u]; ++t) stage[o + t] = (unsigned)(p0[u] + (int)t);
+                o += e[u];
+            }
+            __syncwarp();
+            int *dst = a.jlist + pos;
+            for (unsigned t = lane; t < total; t += 32) dst[t] = (int)stage[t];
+            __syncwarp();
+        } else {
+#pragma unroll
+            for (int u = 0; u < kExpand; ++u) {
+                for (unsigned t = 0; t < e[u]; ++t) a.jlist[pos + o + t] = p0[u] + (int)t;
+                o += e[u];
             }
         }
-        const unsigned ei = warp_incl_scan(e, lane);
-        if (e) {
-            const long long d = pos + (ei - e);
-            if (d + e > hi) report(a.status, kStatusBadIndex, 13);
-            else
-                for (unsigned t = 0; t < e; ++t) a.jlist[d + t] = p0 + (int)t;
-        }
-        pos += __shfl_sync(0xffffffffu, ei, 31);
+        pos += total;
     }
     if (pos != hi && lane == 0) report(a.status, kStatusBadIndex, 12);
 }
@@ -915,7 +946,7 @@ __global__ void __launch_bounds__(32 * kGwWarps) k_walk_groups(GroupWalkArgs a)
             // the count pass recorded this group's emitters: expand them
             const int2 ge = a.gemit[g];
             if (ge.x >= 0) {
-                expand_emitters(a, ge.x, ge.y, pos, hi, lane);
+                expand_emitters(a, ge.x, ge.y, pos, hi, qa, lane);
                 continue;
             }
         }

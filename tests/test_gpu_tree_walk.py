@@ -203,3 +203,20 @@ def test_recorded_and_rewalked_groups(pg, orc):
     same_lists(t1, o)
     same_lists(t2, o)
     assert np.array_equal(a1, a2) and np.array_equal(p1, p2)
+
+
+@pytest.mark.parametrize("nleaf,quad", [(1, False), (40, False), (300, True)])
+def test_expanded_runs_of_every_length(pg, orc, nleaf, quad):
+    # the fill pass lays out the entries of 128 emitters at a time: at most
+    # 1280 of them in shared memory, more than that (leaves of up to 300
+    # particles) lane by lane. The lists equal the oracle's either way
+    x, m = gen.plummer(9001, 7109)
+    o = orc.tree_build(x, m, 0.6, 128, nleaf, quadrupole=quad)
+    with pg.Context(0) as c:
+        c.set_eps(1e-3)
+        c.set_self(True)
+        c.set_tree(0.6, 128, nleaf, quadrupole=quad)
+        run_once(pg, c, x, m)
+        a, p, t, s = run_once(pg, c, x, m)
+    assert s["exact"] == 0 and s["walk"] == 1
+    same_lists(t, o)
