@@ -22,8 +22,10 @@ namespace pg {
 constexpr int kTJG = 512;          // j entries staged per step
 
 // unroll depth of a CTA-mode item's j loop (measured on GB300: 8 for the
-// table lookups, whose latency wants more terms in flight; 2 for Newton)
-template <bool TABLE> struct GroupsUnrollJ { static constexpr int value = TABLE ? 8 : 2; };
+// table lookups, whose latency wants more terms in flight; 4 for Newton:
+// 2, 4 and 8 take 2.66, 2.37, 2.39 ms on lists of 4000 groups and 2.21, 2.17,
+// 2.23 ms for a tree of 2^20)
+template <bool TABLE> struct GroupsUnrollJ { static constexpr int value = TABLE ? 8 : 4; };
 
 // Records come in two forms.
 //  CELL = false: any particle as a double-float pair, hi = (x, y, z, m) in
@@ -48,10 +50,10 @@ template <bool TABLE> struct GroupsUnrollJ { static constexpr int value = TABLE 
 // Table mode scales d afterwards (one multiply, relative error 2^-24).
 //
 // Thread layout of an item: nsets sets of 2*NP i-particles; each set owns L
-// consecutive lanes of one warp (any L from 1 to 32, sets never straddle a
-// warp), lane l of a set takes the j with index = l (mod L), and the set's
-// lanes are combined by a segmented shuffle reduction at the end. NP (i-pairs
-// per thread) is chosen per item, 2 or 4, for the better thread use.
+// consecutive threads of the CTA, thread l of a set takes the j with index =
+// l (mod L), and the set's threads are combined in shared memory at the end.
+// NP (i-pairs per thread) is chosen per item, NPMAX or half of it, for the
+// better thread use.
 
 // floor(a / b) for 0 <= a < 2^16 and 1 <= b <= 128 as one high multiply by
 // ceil(2^32 / b) (exact in that range), not the generic division sequence
@@ -81,8 +83,14 @@ __device__ __forceinline__ int div_small(int a, int b)
     return b == 1 ? a : (int)__umulhi((unsigned)a, kRecip[b]);
 }
 
+// An item's shape with np i-pairs per thread: nsets sets of 2 np i-particles,
+// each with L consecutive threads that share the j-list. A set may cross a
+// warp boundary (its lanes are added in shared memory), so nsets L comes near
+// NT: 72 i-particles with two pairs a thread keep 126 of 128 threads, sets
+// held inside warps 108. Tree lists of 2^20 Plummer (72 i a group): a call
+// takes 2.20 ms instead of 2.27.
 struct ItemShape {
-    int nsets, L, spw;
+    int nsets, L;
 };
 
 template <int NT = kNT>
@@ -90,11 +98,7 @@ __device__ __forceinline__ ItemShape item_shape(int ni, int np)
 {
     ItemShape s;
     s.nsets = (ni + 2 * np - 1) / (2 * np);
-    int L = div_small(NT, s.nsets > 0 ? s.nsets : 1);
-    L = L > 32 ? 32 : L < 1 ? 1 : L;
-    while (L > 1 && (NT / 32) * div_small(32, L) < s.nsets) --L;
-    s.L = L;
-    s.spw = div_small(32, L);
+    s.L = min(max(NT / max(s.nsets, 1), 1), 128);
     return s;
 }
 
@@ -215,6 +219,72 @@ __device__ __forceinline__ void pair_term(float ra, float rb, u64 dx, u64 dy, u6
     }
 }
 
+// The L lanes of each set, added in shared memory: one thread per (set,
+// i-pair, component), (hi, lo) FP32 pairs with TwoSum, the lanes in turn
+// from one that differs between neighbouring sets (no two of them in a
+// bank when L is a multiple of 16). One conversion to FP64 on as many
+// lanes as there are sums: an FP64 instruction takes a warp the same
+// time however few lanes need it.
+template <int NP, bool TABLE, bool CELL, bool EXT, bool HL, int NT>
+__device__ __forceinline__ void group_sums(const GroupArgs &a, const GroupItem &it, const ItemShape &sh,
+                                           const u64 *run, const float2 *tab, int tid)
+{
+    const int L = sh.L;
+    __syncthreads();
+#pragma unroll 1
+    for (int o = tid; o < sh.nsets * (4 * NP); o += NT) {
+        const int pk = o / sh.nsets, st = o - pk * sh.nsets;
+        const int p = pk >> 2, k = pk & 3;
+        const u64 *rh = run + (8 * p + k) * NT + st * L, *rl = rh + 4 * NT;
+        int l = st & 15;
+        l = l < L ? l : 0;
+        u64 h = rh[l], lo = rl[l];
+#pragma unroll 1
+        for (int t = 1; t < L; ++t) {
+            l = l + 1 < L ? l + 1 : 0;
+            fold2(h, lo, rh[l]);
+            lo = f2add(lo, rl[l]);
+        }
+        float hv[2], lv[2];
+        up2(h, hv[0], hv[1]);
+        up2(lo, lv[0], lv[1]);
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const int k_i = st * 2 * NP + 2 * p + q;
+            if (k_i >= it.ni) continue;
+            const long long i = it.i0 + k_i;
+            if constexpr (HL) {
+                // FP32 (hi, lo) sums out; the finish kernel converts them
+                float *hlf = reinterpret_cast<float *>(a.hl) + 8 * i;
+                hlf[k] = hv[q];
+                hlf[4 + k] = lv[q];
+            } else {
+                const double v = (double)hv[q] + (double)lv[q];
+                if (a.part) {          // one partial of a narrow all-pairs sum
+                    reinterpret_cast<double *>(a.part + (long long)it.pad * a.part_stride + i)[k] = v;
+                    continue;
+                }
+                const long long oi = a.perm ? (long long)a.perm[i] : i;
+                if (k < 3)
+                    a.acc[3 * oi + k] = v * a.accscale;
+                else if (a.pot)        // zero in table mode without a potential
+                    a.pot[oi] = CELL && EXT ? v - cell_self_pot(a, tab, i)
+                                : !TABLE && a.list_self ? v - list_self_pot(a, i) : v;
+            }
+        }
+    }
+}
+
+// The same out of line, for the particle records' kernels: inlined, it costs
+// their j loop its schedule (lists of 4000 groups: 2.71 against 2.58 ms; the
+// cell list's kernel is the faster inlined, 2.51 against 2.53).
+template <int NP, bool TABLE, bool EXT, bool HL, int NT>
+__device__ __noinline__ void group_sums_call(const GroupArgs &a, const GroupItem &it, const ItemShape &sh,
+                                             const u64 *run, const float2 *tab, int tid)
+{
+    group_sums<NP, TABLE, false, EXT, HL, NT>(a, it, sh, run, tab, tid);
+}
+
 template <int NP, bool TABLE, bool CELL, bool EXT, bool HL = false, bool DF = false, int TJ = kTJG,
           int NT = kNT>
 __device__ __forceinline__ void group_item(const GroupArgs &a, const GroupItem &it, const ItemShape sh,
@@ -253,10 +323,8 @@ __device__ __forceinline__ void group_item(const GroupArgs &a, const GroupItem &
     auto RL = [&](int p, int k) -> u64 & { return run[(8 * p + 4 + k) * NT + tid]; };
 
     const int L = sh.L;
-    const int wl = tid & 31;
-    const int wq = div_small(wl, L);
-    const int set = (tid >> 5) * sh.spw + wq, lane = wl - wq * L;
-    const bool active = wl < sh.spw * L && set < sh.nsets;
+    const int set = div_small(tid, L), lane = tid - set * L;
+    const bool active = set < sh.nsets;
 
     u64 xi[NP], yi[NP], zi[NP];
     u64 lxi[DF ? NP : 1], lyi[DF ? NP : 1], lzi[DF ? NP : 1];   // DF: the records' lo parts
@@ -459,73 +527,8 @@ __device__ __forceinline__ void group_item(const GroupArgs &a, const GroupItem &
         __syncthreads();   // everyone done with this tile before it is overwritten
     }
 
-    // combine the L lanes of each set: segmented shuffle reduction of the
-    // (hi, lo) FP32 pairs with TwoSum (FP64 would dominate small items on
-    // GB300), one conversion to FP64 on the set's first lane
-#pragma unroll
-    for (int p = 0; p < NP; ++p) {
-        float h[8], l[8];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            up2(RH(p, k), h[2 * k], h[2 * k + 1]);
-            up2(RL(p, k), l[2 * k], l[2 * k + 1]);
-        }
-        for (int off = 1; off < L; off <<= 1) {
-            const bool take = lane + off < L;
-#pragma unroll
-            for (int k = 0; k < 8; ++k) {
-                if (TABLE && !EXT && (k == 6 || k == 7)) continue;   // no potential
-                const float oh = __shfl_down_sync(0xffffffffu, h[k], off);
-                const float ol = __shfl_down_sync(0xffffffffu, l[k], off);
-                if (take) {
-                    float sm, er;
-                    two_sum(h[k], oh, sm, er);
-                    h[k] = sm;
-                    l[k] = __fadd_rn(l[k], __fadd_rn(ol, er));
-                }
-            }
-        }
-        if constexpr (HL) {
-            // FP32 (hi, lo) sums out; the finish kernel converts them on full warps
-            if (active && lane == 0) {
-#pragma unroll
-                for (int q = 0; q < 2; ++q) {
-                    const int k_i = set * 2 * NP + 2 * p + q;
-                    if (k_i < it.ni) {
-                        const long long i = it.i0 + k_i;
-                        a.hl[2 * i] = make_float4(h[0 + q], h[2 + q], h[4 + q], h[6 + q]);
-                        a.hl[2 * i + 1] = make_float4(l[0 + q], l[2 + q], l[4 + q], l[6 + q]);
-                    }
-                }
-            }
-            continue;
-        }
-        if (active && lane == 0) {
-            double v[8];
-#pragma unroll
-            for (int k = 0; k < 8; ++k) v[k] = (double)h[k] + (double)l[k];
-#pragma unroll
-            for (int q = 0; q < 2; ++q) {
-                int k = set * 2 * NP + 2 * p + q;
-                if (k < it.ni) {
-                    long long i = it.i0 + k;
-                    const double phi = TABLE && !EXT ? 0.0 : v[6 + q];
-                    if (a.part) {          // one partial of a narrow all-pairs sum
-                        a.part[(long long)it.pad * a.part_stride + i] =
-                            make_double4(v[0 + q], v[2 + q], v[4 + q], phi);
-                        continue;
-                    }
-                    long long o = a.perm ? (long long)a.perm[i] : i;
-                    a.acc[3 * o] = v[0 + q] * a.accscale;
-                    a.acc[3 * o + 1] = v[2 + q] * a.accscale;
-                    a.acc[3 * o + 2] = v[4 + q] * a.accscale;
-                    if (a.pot)
-                        a.pot[o] = CELL && EXT ? phi - cell_self_pot(a, tab, i)
-                                 : !TABLE && a.list_self ? phi - list_self_pot(a, i) : phi;
-                }
-            }
-        }
-    }
+    if constexpr (CELL) group_sums<NP, TABLE, true, EXT, HL, NT>(a, it, sh, run, tab, tid);
+    else group_sums_call<NP, TABLE, EXT, HL, NT>(a, it, sh, run, tab, tid);
 }
 
 // Warp mode: one warp evaluates one small item at a time (at most 64
@@ -943,17 +946,17 @@ __global__ void __launch_bounds__(NT) k_groups(GroupArgs a)
             break;
         }
         const GroupItem it = item_at(a, item);
+        ItemShape best = item_shape<NT>(it.ni, NPMAX);
         if (NPMAX > 1 && it.ni <= NT * NPMAX) {
-            const ItemShape big = item_shape<NT>(it.ni, NPMAX);
-            const ItemShape small = item_shape<NT>(it.ni, NPMAX / 2);
-            if (small.nsets <= 4 * small.spw && small.nsets * small.L > big.nsets * big.L) {
-                group_item<(NPMAX > 1 ? NPMAX / 2 : 1), TABLE, CELL, EXT, HL, DF, TJ, NT>(a, it, small, cvt, run,
-                                                                                 cr, tab, dirt, tid);
+            // a thread's step costs about np pair terms and an eighth of one
+            constexpr int kHalf = NPMAX > 1 ? NPMAX / 2 : 1;
+            const ItemShape half = item_shape<NT>(it.ni, kHalf);
+            if ((8 * NPMAX + 1) * half.L > (8 * kHalf + 1) * best.L) {
+                group_item<kHalf, TABLE, CELL, EXT, HL, DF, TJ, NT>(a, it, half, cvt, run, cr, tab, dirt, tid);
                 continue;
             }
         }
-        group_item<NPMAX, TABLE, CELL, EXT, HL, DF, TJ, NT>(a, it, item_shape<NT>(it.ni, NPMAX), cvt, run, cr, tab,
-                                                  dirt, tid);
+        group_item<NPMAX, TABLE, CELL, EXT, HL, DF, TJ, NT>(a, it, best, cvt, run, cr, tab, dirt, tid);
     }
 
     // warp mode: warp 0 takes the item that ended CTA mode and thread 0's
