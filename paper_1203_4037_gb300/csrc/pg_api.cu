@@ -1592,7 +1592,7 @@ int check_run_state(pg_ctx *c)
 // largest i-pairs per thread of the groups kernel (items may use half of it):
 // 4 for the caller's groups (hundreds of i against thousands of j); 2 for
 // the tree's lists (groups of at most ncrit against about 2000 entries:
-// measured 1.29 against 1.42 ms on 2^20 Plummer, monopoles) and the cells
+// measured 2.17 against 2.22 ms a call on 2^20 Plummer, monopoles) and the cells
 int groups_np(const pg_ctx *c) { return c->np ? c->np : (c->have_groups ? 4 : 2); }
 
 // the caller's plain Newton lists (no per-i softening, eps > 0) can run any
@@ -1603,17 +1603,30 @@ int groups_nt(const pg_ctx *c) { return c->g_nt && groups_plain(c) ? c->g_nt : k
 
 int upload_group_items(pg_ctx *c)
 {
-    int Bi = groups_bi(groups_np(c), groups_nt(c));
+    const int Bi = groups_bi(groups_np(c), groups_nt(c));
     std::vector<GroupItem> items;
     std::vector<long long> cost;
+    // A CTA takes an item at a time, so the longest item bounds the run: a
+    // group above half a CTA's share of the pairs (three CTAs an SM) is cut
+    // into chunks of Bi / 2, Bi / 4, ... i-particles, at least 64 (each chunk
+    // stages the j-list anew). Whole, 4000 groups of 16 to 512 i and 1024 to
+    // 16384 j took 2.37 ms with the SMs busy 77 % of it. Cut at 1, 1/2, 1/4
+    // and 1/8 of the share: 2.34, 2.04, 2.13, 2.21 ms; 1500 such groups 1.10,
+    // 0.84, 0.83 at 1, 1/2, 1/3; 500 groups 0.45 (0.61 in chunks of 128 or more).
+    double total = 0;
+    for (long long g = 0; g < c->ngroups; ++g)
+        total += (double)(c->h_ioff[g + 1] - c->h_ioff[g]) * (double)(c->h_joff[g + 1] - c->h_joff[g]);
+    const double cap = total / (3.0 * c->sms * 2.0);
     for (long long g = 0; g < c->ngroups; ++g) {
         long long i0 = c->h_ioff[g], ni = c->h_ioff[g + 1] - i0;
         long long nj = c->h_joff[g + 1] - c->h_joff[g];
-        for (long long k = 0; k < ni; k += Bi) {
+        int chunk = Bi;
+        while (chunk > 64 && (double)std::min<long long>(chunk, ni) * (double)nj > cap) chunk /= 2;
+        for (long long k = 0; k < ni; k += chunk) {
             GroupItem it;
             it.group = (int)g;
             it.i0 = (int)(i0 + k);
-            it.ni = (int)std::min<long long>(Bi, ni - k);
+            it.ni = (int)std::min<long long>(chunk, ni - k);
             it.pad = 0;
             items.push_back(it);
             cost.push_back((long long)it.ni * nj);

@@ -167,3 +167,32 @@ def test_tree_workload_20000_groups_sampled(pg, orc):
     sel = np.concatenate([np.arange(d["i_off"][g], d["i_off"][g + 1]) for g in gs])
     assert_parity(rel_vec(a[sel], ao), what="a")
     assert_parity(rel_scalar(p[sel], po), what="phi")
+
+
+@pytest.mark.parametrize("np_, tile", [(1, None), (2, None), (4, None), (4, (256, 128)), (2, (512, 256)), (4, (1024, 256))])
+def test_sets_across_warps_and_cut_groups(pg, orc, np_, tile):
+    # a set's threads may cross a warp boundary: one to 256 sets of 1 to 128
+    # threads, with lists about the tile's depth; the last group holds most of
+    # the pairs and is cut into chunks of 64 i-particles
+    rng = np.random.default_rng(11)
+    xj, mj = gen.plummer(5000, 12)
+    sizes_i = [33, 34, 36, 40, 41, 63, 64, 65, 72, 100, 127, 129, 200, 255, 256, 257, 300, 341, 511, 512, 2, 700]
+    sizes_j = [int(k) for k in rng.integers(200, 1100, len(sizes_i))]
+    sizes_j[1], sizes_j[-2], sizes_j[-1] = 1, 40000, 41003
+    i_off = np.concatenate([[0], np.cumsum(sizes_i)])
+    j_off = np.concatenate([[0], np.cumsum(sizes_j)])
+    jlist = np.concatenate([rng.integers(0, len(xj), k) for k in sizes_j]).astype(np.int32)
+    xi = gen.plummer(int(i_off[-1]), 13)[0]
+    with pg.Context(0) as c:
+        c.set_eps(0.01)
+        c.set_shape(np_)
+        if tile:
+            c.set_groups_tile(*tile)
+        c.set_j(xj, mj)
+        c.set_i(xi)
+        c.set_groups(i_off, j_off, jlist)
+        c.run()
+        a, p = c.get_force(len(xi))
+    ao, po = orc.newton_groups(i_off, j_off, jlist, xi, xj, mj, 0.01)
+    assert_parity(rel_vec(a, ao), what="a")
+    assert_parity(rel_scalar(p, po), what="phi")
