@@ -157,9 +157,12 @@ __global__ void k_morton(const double4 *__restrict__ x, long long n,
 // long as the five kernels it replaces.
 constexpr int kSortWarps = 8;                  // 256 threads, one per digit
 constexpr int kSortThreads = 32 * kSortWarps;
-// keys per lane: tiles of 8192 keys for large sets; for small ones tiles of
-// 2048, four times the blocks
-constexpr int kSortRounds = 32, kSortRoundsSmall = 8;
+// keys per lane: tiles of 4096 keys for large sets; for small ones tiles of
+// 2048, twice the blocks. Tiles of 8192 are as fast from 2^21 keys on and
+// leave SMs idle below: a tree call on 2^20 particles takes 2172 us with them,
+// 2145 with 4096 and 2171 with 2048, on 300007 1517, 1488 and 1486; cells of
+// 2^21 particles 2509, 2512 and 2538
+constexpr int kSortRounds = 16, kSortRoundsSmall = 8;
 constexpr int kSortBatch = 8;          // rounds in flight per lane
 constexpr long long kSortSmall = 1LL << 18;
 constexpr int kSortPasses = 4;         // 32-bit keys
