@@ -553,42 +553,56 @@ cudaError_t launch_allpairs(const AllPairsArgs &a, int grid, int np, bool table,
 }
 
 // ------------------------------------------------------------------ combine
-// One thread per i (tile order): add the CTA partials of its tile in slot
-// order in FP64, take out the self pair's potential term, rescale, scatter.
-__global__ void k_combine(CombineArgs c)
+__device__ __forceinline__ void combine_out(const CombineArgs &c, long long p, double ax, double ay, double az,
+                                            double ph)
 {
-    long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (c.skip && *c.skip) return;
-    const bool in = p < c.ni;
-    if (!in && !c.start) return;
-    long long t = (in ? p : c.ni - 1) / c.Bi;
-    int li = (int)(p % c.Bi);
-    double ax = 0, ay = 0, az = 0, ph = 0;
-    if (c.start && *c.near) {          // (a block's i are of one tile, whose search all threads share)
-        int b0, b1;
-        plan_ctas(c.start, c.near_grid, t * c.nch, (t + 1) * c.nch, b0, b1);
-#pragma unroll 8
-        for (int b = b0; b < b1; ++b) {
-            if (!in || c.start[b + 1] <= c.start[b]) continue;
-            const double4 v = ldg_d4(c.part + (size_t)(t + b) * c.Bi + li);
-            ax += v.x; ay += v.y; az += v.z; ph += v.w;
-        }
-    } else if (in && c.njsub > 0) {
-        long long bf = stream_k_owner(t * c.njsub, c.grid, c.W);
-        long long bl = stream_k_owner((t + 1) * c.njsub - 1, c.grid, c.W);
-        for (long long s = 0; s <= bl - bf; ++s) {
-            double4 v = c.part[((size_t)t * c.smax_slots + (size_t)s) * c.Bi + li];
-            ax += v.x; ay += v.y; az += v.z; ph += v.w;
-        }
-    }
-    if (!in) return;
-    long long k = c.perm ? (long long)c.perm[p] : p;
+    const long long k = c.perm ? (long long)c.perm[p] : p;
     if (c.self && c.njsub > 0) ph -= self_potential(c, k);
     if (c.fail_nan && *c.fail_nan != 0) ax = ay = az = ph = __longlong_as_double(0x7ff8000000000000ll);
     c.acc[3 * k] = ax * c.accscale;
     c.acc[3 * k + 1] = ay * c.accscale;
     c.acc[3 * k + 2] = az * c.accscale;
     if (c.pot) c.pot[k] = c.newton || c.tabpot ? ph : 0.0;
+}
+
+// i-particle p's partials in slot order
+__device__ __forceinline__ double4 combine_slots(const CombineArgs &c, long long p)
+{
+    const long long t = p / c.Bi;
+    const int li = (int)(p % c.Bi);
+    double4 s = make_double4(0, 0, 0, 0);
+    if (c.njsub <= 0) return s;
+    const long long bf = stream_k_owner(t * c.njsub, c.grid, c.W);
+    const long long bl = stream_k_owner((t + 1) * c.njsub - 1, c.grid, c.W);
+    for (long long q = 0; q <= bl - bf; ++q) {
+        const double4 v = c.part[((size_t)t * c.smax_slots + (size_t)q) * c.Bi + li];
+        s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
+    }
+    return s;
+}
+
+// One thread per i (tile order): add the CTA partials of its tile in slot
+// order in FP64, take out the self pair's potential term, rescale, scatter.
+__global__ void k_combine(CombineArgs c)
+{
+    const long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    if ((c.skip && *c.skip) || p >= c.ni) return;
+    const double4 s = combine_slots(c, p);
+    combine_out(c, p, s.x, s.y, s.z, s.w);
+}
+
+// The same for a run that may have taken the near-pair kernel, 64 i-particles
+// (of one tile) a block. With one thread an i the sums of 65536 Plummer, whose
+// core tiles have most of the partials, took 39 us.
+__global__ void __launch_bounds__(256) k_combine_near(CombineArgs c)
+{
+    const long long p = blockIdx.x * (long long)kNearCombineI + threadIdx.x % kNearCombineI;
+    const bool in = p < c.ni;
+    const long long t = blockIdx.x * (long long)kNearCombineI / c.Bi;
+    double4 s;
+    if (*c.near) s = near_sum(c.start, c.near_grid, c.nch, c.part, c.Bi, t, (int)(p - t * c.Bi), in);
+    else if (in && threadIdx.x < kNearCombineI) s = combine_slots(c, p);
+    if (in && threadIdx.x < kNearCombineI) combine_out(c, p, s.x, s.y, s.z, s.w);
 }
 
 // The same sum with a 128-thread block per i, for few i-particles with many
@@ -629,19 +643,15 @@ __global__ void __launch_bounds__(kWideThreads) k_combine_wide(CombineArgs c)
     for (int w = 0; w < kWideThreads / 32; ++w) {
         ax += wsum[w].x; ay += wsum[w].y; az += wsum[w].z; ph += wsum[w].w;
     }
-    const long long k = c.perm ? (long long)c.perm[p] : p;
-    if (c.self && c.njsub > 0) ph -= self_potential(c, k);
-    if (c.fail_nan && *c.fail_nan != 0) ax = ay = az = ph = __longlong_as_double(0x7ff8000000000000ll);
-    c.acc[3 * k] = ax * c.accscale;
-    c.acc[3 * k + 1] = ay * c.accscale;
-    c.acc[3 * k + 2] = az * c.accscale;
-    if (c.pot) c.pot[k] = c.newton || c.tabpot ? ph : 0.0;
+    combine_out(c, p, ax, ay, az, ph);
 }
 
 cudaError_t launch_combine(const CombineArgs &c, cudaStream_t st)
 {
     if (c.ni <= 0) return cudaSuccess;
-    if (c.smax_slots >= 32 && !c.start)
+    if (c.start)
+        k_combine_near<<<(unsigned)((c.ni + kNearCombineI - 1) / kNearCombineI), 256, 0, st>>>(c);
+    else if (c.smax_slots >= 32)
         k_combine_wide<<<(unsigned)c.ni, kWideThreads, 0, st>>>(c);
     else
         k_combine<<<(unsigned)((c.ni + 255) / 256), 256, 0, st>>>(c);

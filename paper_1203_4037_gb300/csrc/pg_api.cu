@@ -1251,9 +1251,14 @@ bool tiled_df(const pg_ctx *c, long long ni, long long nj)
 
 // The tabulated force is exactly 0 from r_cut on, so compact (sorted) tiles
 // evaluate only the j within r_cut of their box (pg_near.cu).
-// Clocks of one kept record against a warp's run, for the split: per i-pair
-// of a thread in the forward kernel, and in the backward kernel.
+// The split's costs, in clocks: one kept record against a warp's run (per
+// i-pair of a thread in the forward kernel; in the backward kernel) and one
+// tested record, fitted to the CTAs' times on 65536 Plummer (r_cut = 0.1);
+// with 1500 a unit for the tests the last CTA took 1.7 times the mean (a fit
+// step on 65536, r_cut = 0.1, and on 60000, r_cut = 0.2: 1544 and 1814 us,
+// with these 1508 and 1700).
 constexpr float kNearPairCost = 215.0f, kNearBackCost = 670.0f;
+constexpr float kNearTestCost = 4.7f, kNearBackTestCost = 7.3f, kNearUnitCost = 900.0f;
 bool tiled_cull(const pg_ctx *c, long long ni) { return c->mode == PG_TABLE && tiles_sorted(c, ni); }
 
 // the narrow path's i chunks are the caller's i-particles in the caller's
@@ -1424,7 +1429,7 @@ int near_unit(int ntiles, long long nj, int grid)
 // the table's near-pair runs (pg_near.cu): the FP32 j records, the tiles'
 // extents (in t_ext already) and the split of the units by cost
 int near_args(pg_ctx *c, NearArgs &a, const double4 *xt, const double4 *jrec, long long ni, long long nj, int Bi,
-              int run, float pair_cost, int grid)
+              int run, float pair_cost, float test_cost, int grid)
 {
     int rc;
     const int ntiles = (int)((ni + Bi - 1) / Bi);
@@ -1453,7 +1458,7 @@ int near_args(pg_ctx *c, NearArgs &a, const double4 *xt, const double4 *jrec, lo
     a.tab = table_dev(c);
     a.part = (double4 *)c->part.p;
     a.status = (int *)c->status.p;
-    PG_CUDA(c, launch_near_plan(a, Bi, run, pair_cost, 1500.0f, grid,
+    PG_CUDA(c, launch_near_plan(a, Bi, run, pair_cost, kNearUnitCost + test_cost * a.unit, grid,
                                 (unsigned *)((unsigned long long *)c->t_cost.p + ntiles),
                                 (unsigned long long *)c->t_cost.p,
                                 (unsigned char *)c->t_dense.p, (long long *)c->t_start.p, near, c->stream));
@@ -1482,7 +1487,7 @@ int enqueue_allpairs(pg_ctx *c, const Plan &p, double *acc, double *pot)
         const int occ = near_max_blocks_per_sm(p.np, tab_units(c), ext, p.df);
         ngrid = c->sms * (c->ctas_per_sm > 0 ? std::min(c->ctas_per_sm, occ) : occ);
         if ((rc = near_args(c, na, (const double4 *)c->xt.p, (const double4 *)c->jrec.p, p.ni, p.nj, p.Bi, 64 * p.np,
-                            kNearPairCost * p.np, ngrid)))
+                            kNearPairCost * p.np, kNearTestCost, ngrid)))
             return rc;
     }
     AllPairsArgs a{};
@@ -2816,7 +2821,7 @@ int pg_backward_dev(pg_ctx *c, const double *w, double *dx, double *dm, float *d
     if (cull) {
         const int nocc = near_backward_max_blocks_per_sm(c->ntab);
         const int ngrid = c->sms * (c->ctas_per_sm > 0 ? std::min(c->ctas_per_sm, nocc) : nocc);
-        if ((rc = near_args(c, na, a.xi, a.jx, n, n, Bi, Bi / 4, kNearBackCost, ngrid))) return rc;
+        if ((rc = near_args(c, na, a.xi, a.jx, n, n, Bi, Bi / 4, kNearBackCost, kNearBackTestCost, ngrid))) return rc;
         a.skip = na.near;
         nc.start = na.start;
         nc.near = na.near;

@@ -543,39 +543,35 @@ cudaError_t launch_pack_w(const double *w, const unsigned *perm, long long n, do
     return cudaGetLastError();
 }
 
-__global__ void k_bw_combine(const double4 *__restrict__ part, const unsigned *__restrict__ perm,
-                             long long n, int njsub, int slots, int grid, long long W, double mscale,
-                             double *__restrict__ dx, double *__restrict__ dm, NearCombine near)
+// one thread per particle, or for a run that may have taken the near-pair
+// kernel 64 of them (of one tile) a block
+template <bool NEAR>
+__global__ void __launch_bounds__(256) k_bw_combine(const double4 *__restrict__ part, const unsigned *__restrict__ perm,
+                                                    long long n, int njsub, int slots, int grid, long long W,
+                                                    double mscale, double *__restrict__ dx, double *__restrict__ dm,
+                                                    NearCombine near)
 {
-    long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    const bool in = p < n;
-    if (!in && !near.start) return;
-    long long t = (in ? p : n - 1) / kBiB;
-    int li = (int)(p % kBiB);
-    double gx = 0, gy = 0, gz = 0, gm = 0;
-    if (near.start && *near.near) {
-        const long long *start = near.start;
-        int b0, b1;
-        plan_ctas(start, near.grid, t * near.nch, (t + 1) * near.nch, b0, b1);
-#pragma unroll 8
-        for (int b = b0; b < b1; ++b) {
-            if (!in || start[b + 1] <= start[b]) continue;
-            const double4 v = ldg_d4(part + (size_t)(t + b) * kBiB + li);
-            gx += v.x; gy += v.y; gz += v.z; gm += v.w;
-        }
-    } else if (in && njsub > 0) {
+    const int span = NEAR ? kNearCombineI : 256;
+    const long long p = blockIdx.x * (long long)span + threadIdx.x % span;
+    const bool in = p < n, out = in && threadIdx.x < span;
+    const long long t = blockIdx.x * (long long)span / kBiB;
+    const int li = (int)(p - t * kBiB);
+    double4 g = make_double4(0, 0, 0, 0);
+    if (NEAR && *near.near) {
+        g = near_sum(near.start, near.grid, near.nch, part, kBiB, t, li, in);
+    } else if (out && njsub > 0) {
         long long bf = sk_owner(t * njsub, grid, W), bl = sk_owner((t + 1) * njsub - 1, grid, W);
         for (long long s = 0; s <= bl - bf; ++s) {
             double4 v = part[((size_t)t * slots + (size_t)s) * kBiB + li];
-            gx += v.x; gy += v.y; gz += v.z; gm += v.w;
+            g.x += v.x; g.y += v.y; g.z += v.z; g.w += v.w;
         }
     }
-    if (!in) return;
+    if (!out) return;
     long long k = perm ? (long long)perm[p] : p;
-    dx[3 * k] = gx;
-    dx[3 * k + 1] = gy;
-    dx[3 * k + 2] = gz;
-    dm[k] = gm * mscale;
+    dx[3 * k] = g.x;
+    dx[3 * k + 1] = g.y;
+    dx[3 * k + 2] = g.z;
+    dm[k] = g.w * mscale;
 }
 
 cudaError_t launch_backward_combine(const double4 *part, const unsigned *perm, long long n, int njsub,
@@ -583,9 +579,10 @@ cudaError_t launch_backward_combine(const double4 *part, const unsigned *perm, l
                                     double *dm, cudaStream_t st, const NearCombine &near)
 {
     if (n <= 0) return cudaSuccess;
-    k_bw_combine<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(part, perm, n, njsub, slots,
-                                                              grid > 0 ? grid : 1, W > 0 ? W : 1,
-                                                              mscale, dx, dm, near);
+    const int span = near.start ? kNearCombineI : 256;
+    auto k = near.start ? k_bw_combine<true> : k_bw_combine<false>;
+    k<<<(unsigned)((n + span - 1) / span), 256, 0, st>>>(part, perm, n, njsub, slots, grid > 0 ? grid : 1,
+                                                         W > 0 ? W : 1, mscale, dx, dm, near);
     return cudaGetLastError();
 }
 

@@ -198,22 +198,6 @@ __device__ __forceinline__ void bulk_g2s(void *dst, const void *src, unsigned by
 }
 
 // ---------------------------------------------------------------- planned splits
-// Of a near-pair run: the CTAs that hold units of [u, v), for one range that
-// all threads of the block ask for: b0 the last that starts at or before u,
-// b1 past the last that starts before v (CTAs without units in between).
-__device__ __forceinline__ void plan_ctas(const long long *start, int grid, long long u, long long v, int &b0, int &b1)
-{
-    int n0 = 0, n1 = 0;
-    for (int q = 0; q < grid; q += blockDim.x) {
-        const int b = q + threadIdx.x;
-        const long long s = b < grid ? start[b] : v;
-        n0 += __syncthreads_count(s <= u && b < grid);
-        n1 += __syncthreads_count(s < v);
-    }
-    b0 = n0 > 0 ? n0 - 1 : 0;
-    b1 = n1;
-}
-
 // ---------------------------------------------------------------- misc
 __device__ __forceinline__ double4 ldg_d4(const double4 *p)
 {
@@ -222,6 +206,62 @@ __device__ __forceinline__ double4 ldg_d4(const double4 *p)
     double2 a = __ldg(q), b = __ldg(q + 1);
     r.x = a.x; r.y = a.y; r.z = b.x; r.w = b.y;
     return r;
+}
+
+// Of a near-pair run: the CTAs that hold units of [u, v), asked for by all
+// threads of the block: b0 the last that starts at or before u, b1 past the
+// last that starts before v (CTAs without units in between). w: two words of
+// shared memory.
+__device__ __forceinline__ void plan_ctas(const long long *start, int grid, long long u, long long v, int *w,
+                                            int &b0, int &b1)
+{
+    if (threadIdx.x < 2) w[threadIdx.x] = 0;
+    __syncthreads();
+    int n0 = 0, n1 = 0;
+#pragma unroll 8
+    for (int b = threadIdx.x; b < grid; b += blockDim.x) {
+        const long long s = start[b];
+        n0 += s <= u;
+        n1 += s < v;
+    }
+    n0 = __reduce_add_sync(0xffffffffu, n0);
+    n1 = __reduce_add_sync(0xffffffffu, n1);
+    if ((threadIdx.x & 31) == 0) {
+        atomicAdd(&w[0], n0);
+        atomicAdd(&w[1], n1);
+    }
+    __syncthreads();
+    b0 = w[0] > 0 ? w[0] - 1 : 0;
+    b1 = w[1];
+}
+
+// The sum of a tile's partials for the 64 i-particles of a 256-thread block,
+// i-particle li of its tile: four threads an i take the CTAs in turn and
+// are added in order; the tiles of a dense core have most of the CTAs.
+// The sum is valid on the first 64 threads.
+constexpr int kNearCombineI = 64;
+__device__ __forceinline__ double4 near_sum(const long long *start, int grid, int nch, const double4 *part, int Bi,
+                                            long long t, int li, bool in)
+{
+    __shared__ int w[2];
+    __shared__ double4 seg[3][kNearCombineI];
+    int b0, b1;
+    plan_ctas(start, grid, t * nch, (t + 1) * nch, w, b0, b1);
+    const int q = threadIdx.x / kNearCombineI, k = threadIdx.x % kNearCombineI;
+    double4 s = make_double4(0, 0, 0, 0);
+#pragma unroll 4
+    for (int b = b0 + q; b < b1; b += 4) {
+        if (!in || start[b + 1] <= start[b]) continue;
+        const double4 v = ldg_d4(part + (size_t)(t + b) * Bi + li);
+        s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
+    }
+    if (q > 0) seg[q - 1][k] = s;
+    __syncthreads();
+    if (q == 0)
+        for (int g = 0; g < 3; ++g) {
+            s.x += seg[g][k].x; s.y += seg[g][k].y; s.z += seg[g][k].z; s.w += seg[g][k].w;
+        }
+    return s;
 }
 
 // The potential term i's own pair added in the loop (d = 0 exactly; i-particle
