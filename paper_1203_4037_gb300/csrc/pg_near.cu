@@ -19,7 +19,7 @@
 // of a unit (copy, two barriers, list) and of a batch (gather, conversion,
 // barrier); the pair terms are a few per cent of n^2. Measured (kernel, Plummer
 // spheres, r_cut = 0.1 scale lengths, against the all-pairs kernels): forward
-// 2.72 -> 0.42 ms at 65536, 43.1 -> 2.7 ms at 262144; backward 5.96 -> 0.64 ms
+// 2.72 -> 0.36 ms at 65536, 43.1 -> 2.7 ms at 262144; backward 5.96 -> 0.60 ms
 // and 94 -> 4.4 ms. With equal unit counts instead of the split by cost the
 // forward kernel took 0.56 ms (an earlier form), converting records in place
 // instead of from a list about 8000 clocks per 256 j.
