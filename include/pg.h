@@ -386,6 +386,13 @@ int pg_backward_dev(pg_ctx *ctx, const double *w, double *dx, double *dm, float 
  * not give up (a defect). Synchronises. */
 int pg_selftest_wait(pg_ctx *ctx, double limit_ms);
 
+/* The sort's way out of a wait, checked without a stall: n keys (1 to 2^22,
+ * PG_EINVAL otherwise) sorted on the device with every block taking the path
+ * of one whose wait for the blocks before it ran out (it counts their keys
+ * itself). PG_OK if the order is the stable sort's, PG_ECUDA otherwise (a
+ * defect). Synchronises. */
+int pg_selftest_sort(pg_ctx *ctx, long long n);
+
 /* Wait for the context's stream and report device-side status. */
 int pg_sync(pg_ctx *ctx);
 

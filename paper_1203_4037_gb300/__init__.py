@@ -74,6 +74,7 @@ SIGNATURES = {
     "pg_set_differencing": (_I, [_P, _I]),
     "pg_set_groups_tile": (_I, [_P, _I, _I]),
     "pg_selftest_wait": (_I, [_P, _D]),
+    "pg_selftest_sort": (_I, [_P, _LL]),
     "pg_set_allpairs_path": (_I, [_P, _I]),
     "pg_set_eps_i": (_I, [_P, _P, _LL]),
     "pg_set_eps_i_dev": (_I, [_P, _P, _LL]),
@@ -429,6 +430,10 @@ def pg_selftest_wait(ctx, limit_ms):
     return _check(ctx, lib().pg_selftest_wait(ctx, float(limit_ms)))
 
 
+def pg_selftest_sort(ctx, n):
+    return _check(ctx, lib().pg_selftest_sort(ctx, int(n)))
+
+
 def pg_set_split(ctx, items_per_warp):
     return _check(ctx, lib().pg_set_split(ctx, int(items_per_warp)))
 
@@ -673,6 +678,9 @@ class Context:
 
     def selftest_wait(self, limit_ms):
         pg_selftest_wait(self.h, limit_ms)
+
+    def selftest_sort(self, n):
+        pg_selftest_sort(self.h, n)
 
     def set_timing(self, on=True):
         pg_set_timing(self.h, on)

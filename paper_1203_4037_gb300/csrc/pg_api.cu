@@ -499,7 +499,6 @@ int pg_create(pg_ctx **out, int device)
         pg_destroy(c);
         return PG_ENOMEM;
     }
-    c->sort.status = (int *)c->status.p;
     *out = c;
     return PG_OK;
 }
@@ -1194,6 +1193,30 @@ int pg_selftest_wait(pg_ctx *c, double limit_ms)
     if (!(limit_ms > 0.0 && limit_ms <= 2000.0)) return fail(c, PG_EINVAL, "limit_ms must be in (0, 2000]");
     PG_CUDA(c, launch_wait_selftest((int *)c->status.p, (unsigned long long)(limit_ms * 1e6), c->stream));
     return read_status(c);
+}
+
+int pg_selftest_sort(pg_ctx *c, long long n)
+{
+    if (!c) return PG_EINVAL;
+    if (n < 1 || n > (1LL << 22)) return fail(c, PG_EINVAL, "n must be in [1, 2^22]");
+    int rc;
+    if ((rc = prep_sort(c, n))) return rc;
+    std::vector<unsigned> key(n), val(n), ref(n);
+    unsigned v = 1u;
+    for (long long k = 0; k < n; ++k) {
+        v = v * 1664525u + 1013904223u;
+        key[k] = (v >> 8) & (k % 3 ? 0xffffffu : 0xff00u);    // many equal digits in between
+        val[k] = ref[k] = (unsigned)k;
+    }
+    PG_CUDA(c, cudaStreamSynchronize(c->stream));
+    PG_CUDA(c, cudaMemcpy(c->sort.keys[0], key.data(), n * 4, cudaMemcpyHostToDevice));
+    PG_CUDA(c, cudaMemcpy(c->sort.vals[0], val.data(), n * 4, cudaMemcpyHostToDevice));
+    unsigned *ko = nullptr, *vo = nullptr;
+    PG_CUDA(c, launch_radix_sort(c->sort.keys[0], c->sort.vals[0], n, 24, c->sort, &ko, &vo, c->stream, 0));
+    PG_CUDA(c, cudaStreamSynchronize(c->stream));
+    PG_CUDA(c, cudaMemcpy(val.data(), vo, n * 4, cudaMemcpyDeviceToHost));
+    std::stable_sort(ref.begin(), ref.end(), [&](unsigned a, unsigned b) { return key[a] < key[b]; });
+    return val == ref ? PG_OK : fail(c, PG_ECUDA, "a sort whose blocks do not wait is out of order");
 }
 
 }  // extern "C"

@@ -207,7 +207,6 @@ struct SortScratch {
     unsigned *keys[2];
     unsigned *vals[2];
     unsigned *hist;        // sort_hist_entries words: look-back words, digit counts, tickets
-    int *status;           // where a look-back that gives up reports
     unsigned *sums;
     unsigned long long *bbox;  // 6 ordered-int words
     size_t cap;            // elements
@@ -216,9 +215,11 @@ struct SortScratch {
 size_t sort_hist_entries(long long n);
 cudaError_t launch_morton_sort(const double4 *xi, long long n, SortScratch &s, unsigned **perm_out,
                                cudaStream_t st);
+// wait_ns: how long a block waits for earlier blocks' counts before it counts
+// their keys itself (0: every block counts, without looking)
 cudaError_t launch_radix_sort(unsigned *keys, unsigned *vals, long long n, int key_bits,
                               SortScratch &s, unsigned **keys_out, unsigned **vals_out,
-                              cudaStream_t st);
+                              cudaStream_t st, unsigned long long wait_ns = kWaitLimitNs);
 
 // ---------------------------------------------------------------- PM
 // The particle-mesh long-range force (pg_pm.cu): mesh, plans and tables,

@@ -144,7 +144,9 @@ __global__ void k_morton(const double4 *__restrict__ x, long long n,
 // have published (the decoupled look-back of Merrill and Garland's scan,
 // 2016, and of Adinets and Merrill's one-sweep radix sort, 2022): its own
 // count first, then, once known, the count up to and including itself. A
-// block waits only on blocks with earlier tickets, which are running or done.
+// block waits only on blocks with earlier tickets, which are running or done;
+// one whose wait runs out counts the keys before its tile itself, so that a
+// pass always writes a permutation (what follows a sort indexes with it).
 // Ranking by lane order within rounds keeps the sort stable. The keys are
 // placed in shared memory in destination order first and written out as runs
 // of consecutive addresses.
@@ -246,7 +248,7 @@ __global__ void __launch_bounds__(kSortThreads) k_rs_pass(const unsigned *__rest
                                                           const unsigned *__restrict__ vin,
                                                           unsigned *__restrict__ kout, unsigned *__restrict__ vout,
                                                           long long n, int shift, const unsigned *__restrict__ total,
-                                                          u64 *look, unsigned *ticket, int *status)
+                                                          u64 *look, unsigned *ticket, u64 wait_ns)
 {
     constexpr int kTile = kSortThreads * R, kChunk = 32 * R;
     extern __shared__ unsigned sort_smem[];
@@ -281,33 +283,48 @@ __global__ void __launch_bounds__(kSortThreads) k_rs_pass(const unsigned *__rest
     }
     __syncthreads();
     // the tiles before this one, digit by digit
-    if (tile > 0)
-        for (int d = tid; d < 256; d += kSortThreads) {
-            u64 before = 0;
-            const u64 t0 = global_ns();
-            for (long long q = tile - 1; q >= 0;) {
-                // all tiles start together, so few have their running count yet
-                // and the walk takes tiles / kLook round trips
-                u64 v[kLook];
+    static_assert(kSortThreads == 256, "one digit a thread");
+    const int dg = tid;
+    bool late = tile > 0 && wait_ns == 0;
+    if (tile > 0 && !late) {
+        u64 before = 0;
+        const u64 t0 = global_ns();
+        for (long long q = tile - 1; q >= 0;) {
+            // all tiles start together, so few have their running count yet
+            // and the walk takes tiles / kLook round trips
+            u64 v[kLook];
 #pragma unroll
-                for (int k = 0; k < kLook; ++k) v[k] = q - k >= 0 ? ld_relaxed(look + (size_t)(q - k) * 256 + d) : kUpTo;
-                bool wait = false;
+            for (int k = 0; k < kLook; ++k) v[k] = q - k >= 0 ? ld_relaxed(look + (size_t)(q - k) * 256 + dg) : kUpTo;
+            bool wait = false;
 #pragma unroll
-                for (int k = 0; k < kLook; ++k) {
-                    if (wait || q < 0) continue;
-                    if (!(v[k] & ~kCountMask)) { wait = true; continue; }
-                    before += v[k] & kCountMask;
-                    q = v[k] & kUpTo ? -1 : q - 1;
-                }
-                if (wait && global_ns() - t0 > kWaitLimitNs) {
-                    report(status, kStatusTimeout, 6);
-                    break;
-                }
+            for (int k = 0; k < kLook; ++k) {
+                if (wait || q < 0) continue;
+                if (!(v[k] & ~kCountMask)) { wait = true; continue; }
+                before += v[k] & kCountMask;
+                q = v[k] & kUpTo ? -1 : q - 1;
             }
-            st_relaxed(mine + d, kUpTo | (before + lstart[d]));
-            gstart[d] += (unsigned)before;
+            if (wait && global_ns() - t0 > wait_ns) {
+                late = true;
+                break;
+            }
         }
-    __syncthreads();
+        if (!late) {
+            st_relaxed(mine + dg, kUpTo | (before + lstart[dg]));
+            gstart[dg] += (unsigned)before;
+        }
+    }
+    if (__syncthreads_or(late)) {
+        unsigned *h = sk;                      // not in use yet
+        h[dg] = 0;
+        __syncthreads();
+        for (long long e = tid; e < tile * kTile; e += kSortThreads) atomicAdd(&h[(kin[e] >> shift) & 255u], 1u);
+        __syncthreads();
+        if (late) {
+            st_relaxed(mine + dg, kUpTo | (h[dg] + lstart[dg]));
+            gstart[dg] += h[dg];
+        }
+        __syncthreads();
+    }
     if (w == 0) scan256(lstart, lane);
     __syncthreads();
     // each warp's first place of each digit in the tile's order
@@ -365,10 +382,8 @@ __global__ void __launch_bounds__(kSortThreads) k_rs_pass(const unsigned *__rest
     for (int p = tid; p < nb; p += kSortThreads) {
         const unsigned k = sk[p], d = (k >> shift) & 255u;
         const unsigned g = gstart[d] + ((unsigned)p - lstart[d]);
-        if (g < n) {                           // (always, unless a wait ran out)
-            kout[g] = k;
-            vout[g] = sv[p];
-        }
+        kout[g] = k;
+        vout[g] = sv[p];
     }
 }
 
@@ -463,7 +478,7 @@ static size_t sort_smem_bytes(int rounds)
 
 cudaError_t launch_radix_sort(unsigned *keys, unsigned *vals, long long n, int key_bits,
                               SortScratch &s, unsigned **keys_out, unsigned **vals_out,
-                              cudaStream_t st)
+                              cudaStream_t st, unsigned long long wait_ns)
 {
     unsigned *kin = keys, *vin = vals;
     unsigned *kb = (keys == s.keys[0]) ? s.keys[1] : s.keys[0];
@@ -488,7 +503,7 @@ cudaError_t launch_radix_sort(unsigned *keys, unsigned *vals, long long n, int k
         for (int p = 0; p < passes; ++p) {
             auto k = small ? k_rs_pass<kSortRoundsSmall> : k_rs_pass<kSortRounds>;
             k<<<(unsigned)tiles, kSortThreads, smem, st>>>(kin, vin, kb, vb, n, 8 * p, cnt + 256 * p,
-                                                        look + (size_t)p * tiles * 256, ticket + p, s.status);
+                                                        look + (size_t)p * tiles * 256, ticket + p, wait_ns);
             std::swap(kin, kb);
             std::swap(vin, vb);
         }

@@ -73,3 +73,11 @@ def test_more_cells_than_particles(pg, orc):
     some = na > 0
     assert np.max((np.maximum(np.linalg.norm(a[idx] - ao, axis=1) - amb, 0))[some] / na[some]) <= 1e-4
     assert np.all(np.linalg.norm(a[idx][~some], axis=1) <= amb[~some])
+
+
+# a block whose wait for the tiles before it runs out counts their keys
+# itself: all blocks do here, with one tile, a remainder, both tile sizes
+@pytest.mark.parametrize("n", [1, 2048, 2049, 40001, 1 << 18, (1 << 18) + 1, 70 * 8192 + 5])
+def test_order_without_waiting(pg, n):
+    with pg.Context(0) as c:
+        c.selftest_sort(n)
