@@ -73,7 +73,7 @@ struct pg_ctx {
 
     // tiles and ordering
     DevBuf xt, ctr;
-    // table on compact tiles: half extents of the tiles, FP32 j records, the
+    // table on compact tiles: half extents of the tiles, scaled FP32 j records, the
     // tiles' costs and density flags, and the CTAs' first units
     DevBuf t_ext, j_f32, t_cost, t_dense, t_start;
     bool tiled_ext = false;       // the current tiles have their extents
@@ -1334,7 +1334,7 @@ int enqueue_tiles(pg_ctx *c, const Plan &p)
         (rc = ensure(c, c->ctr, (size_t)std::max(p.ntiles, 1) * sizeof(double4))))
         return rc;
     const bool ext = tiled_cull(c, n);
-    if (ext && (rc = ensure(c, c->t_ext, (size_t)std::max(p.ntiles, 1) * sizeof(float4)))) return rc;
+    if (ext && (rc = ensure(c, c->t_ext, (size_t)std::max(p.ntiles, 1) * sizeof(double4)))) return rc;
     bool do_sort = tiles_sorted(c, n);
     c->perm = nullptr;
     if (do_sort && n > 1) {
@@ -1356,7 +1356,7 @@ int enqueue_tiles(pg_ctx *c, const Plan &p)
         c->last_launches += 3 + 1 + 4;
     }
     PG_CUDA(c, launch_tile_prep((const double4 *)c->xi.p, c->perm, n, p.Bi, (double4 *)c->xt.p,
-                                (double4 *)c->ctr.p, c->stream, ext ? (float4 *)c->t_ext.p : nullptr));
+                                (double4 *)c->ctr.p, c->stream, ext ? (double4 *)c->t_ext.p : nullptr));
     c->last_launches += 1;
     c->tiled_np = p.np;
     c->tiled_ext = ext;
@@ -1462,10 +1462,11 @@ int near_args(pg_ctx *c, NearArgs &a, const double4 *xt, const double4 *jrec, lo
         (rc = ensure(c, c->t_start, (size_t)(grid + 2) * sizeof(long long))) ||
         (rc = ensure(c, c->part, ((size_t)ntiles + grid) * Bi * sizeof(double4))))
         return rc;
-    PG_CUDA(c, launch_pack_f32(jrec, nj, (float4 *)c->j_f32.p, c->stream));
+    a.tab = table_dev(c);
+    PG_CUDA(c, launch_pack_f32(jrec, nj, a.tab.scale, (float4 *)c->j_f32.p, c->stream));
     a.xi = xt;
     a.ctr = (const double4 *)c->ctr.p;
-    a.ext = (const float4 *)c->t_ext.p;
+    a.ext = (const double4 *)c->t_ext.p;
     a.jrec = jrec;
     a.jf = (const float4 *)c->j_f32.p;
     a.ni = ni;
@@ -1477,8 +1478,6 @@ int near_args(pg_ctx *c, NearArgs &a, const double4 *xt, const double4 *jrec, lo
     a.dense = (const unsigned char *)c->t_dense.p;
     int *near = (int *)((long long *)c->t_start.p + grid + 1);
     a.near = near;
-    a.r_cut = (float)c->r_cut;
-    a.tab = table_dev(c);
     a.part = (double4 *)c->part.p;
     a.status = (int *)c->status.p;
     PG_CUDA(c, launch_near_plan(a, Bi, run, pair_cost, kNearUnitCost + test_cost * a.unit, grid,
@@ -2814,9 +2813,9 @@ int pg_backward_dev(pg_ctx *c, const double *w, double *dx, double *dm, float *d
     }
     c->i_dirty = true;      // the tile buffers now hold the backward's order
     const bool cull = table && n >= 16384;
-    if (cull && (rc = ensure(c, c->t_ext, ntiles * sizeof(float4)))) return rc;
+    if (cull && (rc = ensure(c, c->t_ext, ntiles * sizeof(double4)))) return rc;
     PG_CUDA(c, launch_tile_prep((const double4 *)c->jrec.p, c->perm, n, Bi, (double4 *)c->xt.p,
-                                (double4 *)c->ctr.p, c->stream, cull ? (float4 *)c->t_ext.p : nullptr));
+                                (double4 *)c->ctr.p, c->stream, cull ? (double4 *)c->t_ext.p : nullptr));
     PG_CUDA(c, launch_pack_w(w, c->perm, n, (double4 *)c->bw_wj.p, (double4 *)c->bw_wt.p, c->stream));
     if (table && dv) PG_CUDA(c, cudaMemsetAsync(c->bw_dv.p, 0, c->ntab * sizeof(double), c->stream));
     BackwardArgs a{};

@@ -262,9 +262,9 @@ int pm_solve(PmState *s, const float *rho, const double4 *tgt, long long nt, dou
 
 
 // gather i into tile order and compute tile centres, and with ext set the
-// half extents of each tile's box
+// half extents of each tile's box (infinite with a non-finite particle)
 cudaError_t launch_tile_prep(const double4 *xi, const unsigned *perm, long long n, int Bi,
-                             double4 *xi_tiled, double4 *ctr, cudaStream_t st, float4 *ext = nullptr);
+                             double4 *xi_tiled, double4 *ctr, cudaStream_t st, double4 *ext = nullptr);
 // ---------------------------------------------------------------- tensor cores
 // Newton all pairs with the differences formed by tcgen05.mma (pg_tc.cu)
 struct TcGeo {             // set on the device from the j-set
@@ -308,11 +308,10 @@ struct NearArgs {
     const double4 *xi;     // i positions (backward: and masses) in tile order
     const double4 *wi;     // backward: loss weights in tile order
     const double4 *ctr;    // FP64 centre of each i-tile
-    const float4 *ext;     // half extents of each tile's box, rounded up; infinite with a
-                           // non-finite particle
+    const double4 *ext;    // half extents of each tile's box; infinite with a non-finite particle
     const double4 *jrec;   // j records (x, y, z, m)
     const double4 *jw;     // backward: loss weights in j order
-    const float4 *jf;      // j records rounded to FP32
+    const float4 *jf;      // j records in FP32, positions times tab.scale
     long long ni, nj;
     int unit;              // j records per unit: kNearJ, or kNearJ / 2 or / 4 when that leaves few units
     int ntiles, nch;       // i-tiles; units per tile, ceil(nj / unit)
@@ -320,7 +319,6 @@ struct NearArgs {
     const long long *start;    // first unit of each CTA, grid + 1 (launch_near_plan)
     const unsigned char *dense;    // tiles whose warps keep most of what the tile keeps
     const int *near;       // zero: most pairs are near, the all-pairs kernel does this run
-    float r_cut;
     TableDev tab;
     double4 *part;         // CTA b's sums of tile t at part[(t + b) Bi ...]
     double *dv;            // backward: knot-gradient accumulators, may be null
@@ -351,8 +349,8 @@ cudaError_t launch_near_plan(const NearArgs &a, int Bi, int run, float pair_cost
                              int *near, cudaStream_t st);
 // a step through nch units that spreads neighbours (coprime to nch)
 int near_stride(int nch);
-// records rounded to FP32
-cudaError_t launch_pack_f32(const double4 *rec, long long n, float4 *out, cudaStream_t st);
+// records in FP32, positions times scale
+cudaError_t launch_pack_f32(const double4 *rec, long long n, double scale, float4 *out, cudaStream_t st);
 
 // df: double-float differencing (i-tiles that are not compact; packed
 // arithmetic whatever `packed` says)

@@ -37,24 +37,29 @@ constexpr int kIdx = kTJ + kPadIdx;
 constexpr int kTests = kNearJ / kNT;           // records a thread tests per unit
 static_assert(kNearJ % kNT == 0 && kIdx % 4 == 0, "whole rounds and whole words");
 
-// A tile's box as the test uses it: its centre in FP32 and half extents grown
-// past every rounding of the test. For a j in range, |x_j| <= |c| + h + r_cut,
-// so its FP32 coordinate, the FP32 centre and their difference are together
-// within 2^-22 of that sum per axis (three roundings of 2^-24 of it at most);
-// r_cut is grown by 1e-5, past the roundings of the squared sum.
+// A tile's box as the test uses it, in units of the table's s (lengths times
+// sc; the cutoff is R = sqrt(s_max - 2)): FP32 squares in the caller's unit
+// would leave the range for an r_cut below 1e-19 or above 1e19. Its centre in
+// FP32 and half extents grown past every rounding of the test: for a j in
+// range, |x_j| <= |c| + h + R, so its FP32 coordinate, the FP32 centre and
+// half extent, their difference and the growth are together within 6 2^-24 of
+// that sum per axis; R^2 is grown by 1e-5, past the roundings of the squares.
 struct TileBox {
     float cx, cy, cz, hx, hy, hz, lim;
 };
 
-__device__ __forceinline__ TileBox tile_box(const double4 c, const float4 h, float r_cut)
+__device__ __forceinline__ TileBox tile_box(const double4 c, const double4 h, double sc, float R)
 {
-    constexpr float u = 2.4e-7f;   // just above 2^-22
+    constexpr float u = 3.6e-7f;   // just above 6 2^-24
     TileBox b;
-    b.cx = (float)c.x; b.cy = (float)c.y; b.cz = (float)c.z;
-    b.hx = h.x + u * (fabsf(b.cx) + h.x + r_cut);
-    b.hy = h.y + u * (fabsf(b.cy) + h.y + r_cut);
-    b.hz = h.z + u * (fabsf(b.cz) + h.z + r_cut);
-    b.lim = r_cut * r_cut * (1.0f + 1e-5f);
+    b.cx = (float)(c.x * sc);
+    b.cy = (float)(c.y * sc);
+    b.cz = (float)(c.z * sc);
+    const float hx = (float)(h.x * sc), hy = (float)(h.y * sc), hz = (float)(h.z * sc);
+    b.hx = hx + u * (fabsf(b.cx) + hx + R);
+    b.hy = hy + u * (fabsf(b.cy) + hy + R);
+    b.hz = hz + u * (fabsf(b.cz) + hz + R);
+    b.lim = R * R * (1.0f + 1e-5f);
     return b;
 }
 
@@ -209,7 +214,7 @@ __device__ __forceinline__ bool near_stream(const NearArgs &a, const NearShared 
             }
             cur = t;
             held = 0;
-            box = tile_box(a.ctr[t], a.ext[t], a.r_cut);
+            box = tile_box(a.ctr[t], a.ext[t], a.tab.scale, sqrtf(a.tab.s_max - 2.0f));
             begin(t);
         }
         if (tid == 0) {
@@ -609,12 +614,13 @@ __global__ void __launch_bounds__(32 * kCostWarps) k_near_cost(NearArgs a, int B
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     const long long t = blockIdx.x;
     const float inf = __int_as_float(0x7f800000);
+    const double sc = a.tab.scale;
     float l[3] = {inf, inf, inf}, h[3] = {-inf, -inf, -inf};
     for (int k = lane; k < run; k += 32) {
         const long long i = t * Bi + (long long)w * run + k;
         if (i >= a.ni) break;
         const double4 v = a.xi[i];
-        const float f[3] = {(float)v.x, (float)v.y, (float)v.z};
+        const float f[3] = {(float)(v.x * sc), (float)(v.y * sc), (float)(v.z * sc)};
         for (int c = 0; c < 3; ++c) { l[c] = fminf(l[c], f[c]); h[c] = fmaxf(h[c], f[c]); }
     }
     for (int c = 0; c < 3; ++c)
@@ -629,7 +635,7 @@ __global__ void __launch_bounds__(32 * kCostWarps) k_near_cost(NearArgs a, int B
     __syncthreads();
     const bool all = isinf(a.ext[t].x);
     const long long step = (a.nj + kCostSample - 1) / kCostSample, ns = (a.nj + step - 1) / step;
-    const float lim = a.r_cut * a.r_cut;
+    const float lim = a.tab.s_max - 2.0f;      // the cutoff, squared
     int n[kCostWarps] = {};
 #pragma unroll 4
     for (long long q = tid; q < ns; q += 32 * kCostWarps) {

@@ -529,7 +529,7 @@ cudaError_t launch_morton_sort(const double4 *xi, long long n, SortScratch &s, u
 // take the midpoint of the tile's bounding box as its FP64 centre.
 __global__ void k_tile_prep(const double4 *__restrict__ xi, const unsigned *__restrict__ perm,
                             long long n, int Bi, double4 *__restrict__ xt,
-                            double4 *__restrict__ ctr, float4 *__restrict__ ext)
+                            double4 *__restrict__ ctr, double4 *__restrict__ ext)
 {
     __shared__ double red[6][32];
     long long t = blockIdx.x;
@@ -565,17 +565,16 @@ __global__ void k_tile_prep(const double4 *__restrict__ xi, const unsigned *__re
         double c2 = 0.5 * (red[2][0] + red[5][0]);
         ctr[t] = make_double4(c0, c1, c2, 0.0);
         if (ext) {
-            // from the centre as stored, rounded up past the FP64 and FP32 roundings
-            auto half = [&](int c, double m) {
-                return odd ? INFINITY : (float)(fmax(red[3 + c][0] - m, m - red[c][0]) * (1.0 + 1e-6));
+            auto half = [&](int c, double m) {         // from the centre as stored
+                return odd ? INFINITY : fmax(red[3 + c][0] - m, m - red[c][0]);
             };
-            ext[t] = make_float4(half(0, c0), half(1, c1), half(2, c2), 0.0f);
+            ext[t] = make_double4(half(0, c0), half(1, c1), half(2, c2), 0.0);
         }
     }
 }
 
 cudaError_t launch_tile_prep(const double4 *xi, const unsigned *perm, long long n, int Bi,
-                             double4 *xi_tiled, double4 *ctr, cudaStream_t st, float4 *ext)
+                             double4 *xi_tiled, double4 *ctr, cudaStream_t st, double4 *ext)
 {
     long long nt = (n + Bi - 1) / Bi;
     if (nt <= 0) return cudaSuccess;
@@ -583,18 +582,18 @@ cudaError_t launch_tile_prep(const double4 *xi, const unsigned *perm, long long 
     return cudaGetLastError();
 }
 
-__global__ void k_pack_f32(const double4 *__restrict__ rec, long long n, float4 *__restrict__ out)
+__global__ void k_pack_f32(const double4 *__restrict__ rec, long long n, double sc, float4 *__restrict__ out)
 {
     const long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (k >= n) return;
     const double4 v = rec[k];
-    out[k] = make_float4((float)v.x, (float)v.y, (float)v.z, (float)v.w);
+    out[k] = make_float4((float)(v.x * sc), (float)(v.y * sc), (float)(v.z * sc), (float)v.w);
 }
 
-cudaError_t launch_pack_f32(const double4 *rec, long long n, float4 *out, cudaStream_t st)
+cudaError_t launch_pack_f32(const double4 *rec, long long n, double scale, float4 *out, cudaStream_t st)
 {
     if (n <= 0) return cudaSuccess;
-    k_pack_f32<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(rec, n, out);
+    k_pack_f32<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(rec, n, scale, out);
     return cudaGetLastError();
 }
 

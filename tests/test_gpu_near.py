@@ -147,3 +147,24 @@ def test_gradients(pg, orc, n, r_cut):
     assert rel(dx.cpu().numpy()[idx], ox) <= 1e-4
     assert rel(dm.cpu().numpy()[idx], om) <= 1e-4
     assert rel(dv.cpu().numpy(), ov) <= 1e-4
+
+
+# lengths scaled by a power of two scale every result exactly: at 2^-70 the
+# square of r_cut is an FP32 denormal, at 2^70 beyond FP32
+@pytest.mark.parametrize("k", [-70, 70])
+def test_unit_of_length(pg, orc, k):
+    torch = pytest.importorskip("torch")
+    from paper_1203_4037_gb300 import autograd as AG
+    n, r_cut, u = 20011, 0.1, 2.0 ** k
+    x, m = gen.plummer(n, 29)
+    w = torch.tensor(gen.unit_vectors(n, 30), device="cuda")
+    v, _, _ = table(orc, r_cut)
+
+    def grads(s):
+        xt, mt, vt = (torch.tensor(t, device="cuda", requires_grad=True) for t in (x * s, m, v))
+        a = AG.table_force(xt, mt, vt, r_cut * s, E, F)
+        return (t.cpu().numpy() for t in torch.autograd.grad(a, (xt, mt), w))
+
+    assert np.array_equal(run(pg, x * u, x * u, m, v, r_cut * u, True)[0], run(pg, x, x, m, v, r_cut, True)[0] * u)
+    (dx, dm), (dxu, dmu) = grads(1.0), grads(u)
+    assert np.array_equal(dxu, dx) and np.array_equal(dmu, dm * u)
