@@ -1463,7 +1463,7 @@ int near_args(pg_ctx *c, NearArgs &a, const double4 *xt, const double4 *jrec, lo
         (rc = ensure(c, c->part, ((size_t)ntiles + grid) * Bi * sizeof(double4))))
         return rc;
     a.tab = table_dev(c);
-    PG_CUDA(c, launch_pack_f32(jrec, nj, a.tab.scale, (float4 *)c->j_f32.p, c->stream));
+    PG_CUDA(c, launch_pack_f32(jrec, nj, (const double4 *)c->ctr.p, a.tab.scale, (float4 *)c->j_f32.p, c->stream));
     a.xi = xt;
     a.ctr = (const double4 *)c->ctr.p;
     a.ext = (const double4 *)c->t_ext.p;

@@ -311,7 +311,7 @@ struct NearArgs {
     const double4 *ext;    // half extents of each tile's box; infinite with a non-finite particle
     const double4 *jrec;   // j records (x, y, z, m)
     const double4 *jw;     // backward: loss weights in j order
-    const float4 *jf;      // j records in FP32, positions times tab.scale
+    const float4 *jf;      // j records in FP32, positions from ctr[0] times tab.scale
     long long ni, nj;
     int unit;              // j records per unit: kNearJ, or kNearJ / 2 or / 4 when that leaves few units
     int ntiles, nch;       // i-tiles; units per tile, ceil(nj / unit)
@@ -349,8 +349,9 @@ cudaError_t launch_near_plan(const NearArgs &a, int Bi, int run, float pair_cost
                              int *near, cudaStream_t st);
 // a step through nch units that spreads neighbours (coprime to nch)
 int near_stride(int nch);
-// records in FP32, positions times scale
-cudaError_t launch_pack_f32(const double4 *rec, long long n, double scale, float4 *out, cudaStream_t st);
+// records in FP32, positions from *org times scale
+cudaError_t launch_pack_f32(const double4 *rec, long long n, const double4 *org, double scale, float4 *out,
+                            cudaStream_t st);
 
 // df: double-float differencing (i-tiles that are not compact; packed
 // arithmetic whatever `packed` says)

@@ -39,7 +39,9 @@ static_assert(kNearJ % kNT == 0 && kIdx % 4 == 0, "whole rounds and whole words"
 
 // A tile's box as the test uses it, in units of the table's s (lengths times
 // sc; the cutoff is R = sqrt(s_max - 2)): FP32 squares in the caller's unit
-// would leave the range for an r_cut below 1e-19 or above 1e19. Its centre in
+// would leave the range for an r_cut below 1e-19 or above 1e19. Positions are
+// taken from tile 0's centre o: FP32 has no room for a cutoff 1e7 times
+// smaller than the distance to the caller's origin. Its centre in
 // FP32 and half extents grown past every rounding of the test: for a j in
 // range, |x_j| <= |c| + h + R, so its FP32 coordinate, the FP32 centre and
 // half extent, their difference and the growth are together within 6 2^-24 of
@@ -48,13 +50,13 @@ struct TileBox {
     float cx, cy, cz, hx, hy, hz, lim;
 };
 
-__device__ __forceinline__ TileBox tile_box(const double4 c, const double4 h, double sc, float R)
+__device__ __forceinline__ TileBox tile_box(const double4 c, const double4 h, const double4 o, double sc, float R)
 {
     constexpr float u = 3.6e-7f;   // just above 6 2^-24
     TileBox b;
-    b.cx = (float)(c.x * sc);
-    b.cy = (float)(c.y * sc);
-    b.cz = (float)(c.z * sc);
+    b.cx = (float)((c.x - o.x) * sc);
+    b.cy = (float)((c.y - o.y) * sc);
+    b.cz = (float)((c.z - o.z) * sc);
     const float hx = (float)(h.x * sc), hy = (float)(h.y * sc), hz = (float)(h.z * sc);
     b.hx = hx + u * (fabsf(b.cx) + hx + R);
     b.hy = hy + u * (fabsf(b.cy) + hy + R);
@@ -214,7 +216,7 @@ __device__ __forceinline__ bool near_stream(const NearArgs &a, const NearShared 
             }
             cur = t;
             held = 0;
-            box = tile_box(a.ctr[t], a.ext[t], a.tab.scale, sqrtf(a.tab.s_max - 2.0f));
+            box = tile_box(a.ctr[t], a.ext[t], a.ctr[0], a.tab.scale, sqrtf(a.tab.s_max - 2.0f));
             begin(t);
         }
         if (tid == 0) {
@@ -615,12 +617,13 @@ __global__ void __launch_bounds__(32 * kCostWarps) k_near_cost(NearArgs a, int B
     const long long t = blockIdx.x;
     const float inf = __int_as_float(0x7f800000);
     const double sc = a.tab.scale;
+    const double4 org = a.ctr[0];
     float l[3] = {inf, inf, inf}, h[3] = {-inf, -inf, -inf};
     for (int k = lane; k < run; k += 32) {
         const long long i = t * Bi + (long long)w * run + k;
         if (i >= a.ni) break;
         const double4 v = a.xi[i];
-        const float f[3] = {(float)(v.x * sc), (float)(v.y * sc), (float)(v.z * sc)};
+        const float f[3] = {(float)((v.x - org.x) * sc), (float)((v.y - org.y) * sc), (float)((v.z - org.z) * sc)};
         for (int c = 0; c < 3; ++c) { l[c] = fminf(l[c], f[c]); h[c] = fmaxf(h[c], f[c]); }
     }
     for (int c = 0; c < 3; ++c)

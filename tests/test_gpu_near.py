@@ -168,3 +168,14 @@ def test_unit_of_length(pg, orc, k):
     assert np.array_equal(run(pg, x * u, x * u, m, v, r_cut * u, True)[0], run(pg, x, x, m, v, r_cut, True)[0] * u)
     (dx, dm), (dxu, dmu) = grads(1.0), grads(u)
     assert np.array_equal(dxu, dx) and np.array_equal(dmu, dm * u)
+
+
+# a shift that every coordinate takes exactly changes no bit, also where
+# FP32 coordinates from the caller's origin would not tell the particles apart
+@pytest.mark.parametrize("shift", [2.0 ** 14, 2.0 ** 26])
+def test_far_from_the_origin(pg, orc, shift):
+    n, r_cut = 20011, 0.1
+    x, m = gen.plummer(n, 31)
+    x = np.round(x * 2.0 ** 20) / 2.0 ** 20
+    v, _, _ = table(orc, r_cut)
+    assert np.array_equal(run(pg, x + shift, x + shift, m, v, r_cut, True)[0], run(pg, x, x, m, v, r_cut, True)[0])
