@@ -1463,7 +1463,8 @@ int near_args(pg_ctx *c, NearArgs &a, const double4 *xt, const double4 *jrec, lo
         (rc = ensure(c, c->part, ((size_t)ntiles + grid) * Bi * sizeof(double4))))
         return rc;
     a.tab = table_dev(c);
-    PG_CUDA(c, launch_pack_f32(jrec, nj, (const double4 *)c->ctr.p, a.tab.scale, (float4 *)c->j_f32.p, c->stream));
+    PG_CUDA(c, launch_pack_f32(jrec, a.jw, nj, (const double4 *)c->ctr.p, a.tab.scale, (float4 *)c->j_f32.p,
+                               c->stream));
     a.xi = xt;
     a.ctr = (const double4 *)c->ctr.p;
     a.ext = (const double4 *)c->t_ext.p;
@@ -2843,14 +2844,14 @@ int pg_backward_dev(pg_ctx *c, const double *w, double *dx, double *dm, float *d
     if (cull) {
         const int nocc = near_backward_max_blocks_per_sm(c->ntab);
         const int ngrid = c->sms * (c->ctas_per_sm > 0 ? std::min(c->ctas_per_sm, nocc) : nocc);
+        na.wi = a.wv;
+        na.jw = a.jwv;
         if ((rc = near_args(c, na, a.xi, a.jx, n, n, Bi, Bi / 4, kNearBackCost, kNearBackTestCost, ngrid))) return rc;
         a.skip = na.near;
         nc.start = na.start;
         nc.near = na.near;
         nc.nch = na.nch;
         nc.grid = ngrid;
-        na.wi = a.wv;
-        na.jw = a.jwv;
         na.dv = a.dv;
         a.part = na.part;
     }

@@ -208,6 +208,12 @@ __device__ __forceinline__ double4 ldg_d4(const double4 *p)
     return r;
 }
 
+// a loss weight that is not finite in FP32 (or nearly so)
+__device__ __forceinline__ bool odd_weight(const double4 w)
+{
+    return !(fabsf((float)w.x) + fabsf((float)w.y) + fabsf((float)w.z) < 3.0e38f);
+}
+
 // Of a near-pair run: the CTAs that hold units of [u, v), asked for by all
 // threads of the block: b0 the last that starts at or before u, b1 past the
 // last that starts before v (CTAs without units in between). w: two words of

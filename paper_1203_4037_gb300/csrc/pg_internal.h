@@ -349,9 +349,10 @@ cudaError_t launch_near_plan(const NearArgs &a, int Bi, int run, float pair_cost
                              int *near, cudaStream_t st);
 // a step through nch units that spreads neighbours (coprime to nch)
 int near_stride(int nch);
-// records in FP32, positions from *org times scale
-cudaError_t launch_pack_f32(const double4 *rec, long long n, const double4 *org, double scale, float4 *out,
-                            cudaStream_t st);
+// records in FP32, positions from *org times scale; with w set, one whose loss
+// weight is not finite in FP32 gets a NaN for its mass (the tests then keep it)
+cudaError_t launch_pack_f32(const double4 *rec, const double4 *w, long long n, const double4 *org, double scale,
+                            float4 *out, cudaStream_t st);
 
 // df: double-float differencing (i-tiles that are not compact; packed
 // arithmetic whatever `packed` says)

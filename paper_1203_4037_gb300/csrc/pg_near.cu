@@ -127,16 +127,16 @@ struct WarpBox {
 };
 
 // The numbers of the n staged records (x, y, z, m given by at(e)) that this
-// warp keeps, in order, in idx; padded to whole groups of kPadIdx with `pad`.
-// Returns the padded count.
+// warp keeps (`all`: every one), in order, in idx; padded to whole groups of
+// kPadIdx with `pad`. Returns the padded count.
 template <typename At>
-__device__ __forceinline__ int warp_list(const WarpBox &b, int n, unsigned short *idx, int pad, At at)
+__device__ __forceinline__ int warp_list(const WarpBox &b, bool all, int n, unsigned short *idx, int pad, At at)
 {
     const int lane = threadIdx.x & 31;
     int k = 0;
     for (int e0 = 0; e0 < n; e0 += 32) {
         const int e = e0 + lane;
-        const bool kp = e < n && b.keep(at(e));
+        const bool kp = e < n && (all || b.keep(at(e)));
         const unsigned m = __ballot_sync(0xffffffffu, kp);
         if (kp) idx[k + __popc(m & ((1u << lane) - 1u))] = (unsigned short)e;
         k += __popc(m);
@@ -423,7 +423,7 @@ __global__ void __launch_bounds__(kNT, NearBlocks<NP>::value) k_near(NearArgs a)
 #pragma unroll 16
             for (int e = 0; e < kTJ; ++e) pair(e);
         } else {
-            const int nw = warp_list(wb, n, sm.idx, n, [&](int e) {
+            const int nw = warp_list(wb, false, n, sm.idx, n, [&](int e) {
                 const u64 *q = cvt + kW * e;
                 return make_float4(__uint_as_float((unsigned)q[0]), __uint_as_float((unsigned)q[1]),
                                    __uint_as_float((unsigned)q[2]), __uint_as_float((unsigned)q[3]));
@@ -519,8 +519,10 @@ __global__ void __launch_bounds__(kNT) k_near_backward(NearArgs a)
 
     auto eval = [&](const int *list, int n) {
         __syncthreads();               // the staging's last readers are done; the list is written
+        bool odd = false;              // a non-finite weight: its pairs are, near or far
         for (int k = tid; k < n; k += kNT) {
             const double4 v = ldg_d4(a.jrec + list[k]), ww = ldg_d4(a.jw + list[k]);
+            odd |= odd_weight(ww);
             cv[2 * k] = make_float4((float)((v.x - cx) * sc), (float)((v.y - cy) * sc), (float)((v.z - cz) * sc),
                                     (float)v.w);
             cv[2 * k + 1] = make_float4((float)ww.x, (float)ww.y, (float)ww.z, 0.0f);
@@ -529,8 +531,8 @@ __global__ void __launch_bounds__(kNT) k_near_backward(NearArgs a)
             cv[2 * n] = make_float4(1.0e4f, 1.0e4f, 1.0e4f, 0.0f);
             cv[2 * n + 1] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
         }
-        __syncthreads();
-        const int nw = warp_list(wb, n, sm.idx, n, [&](int e) { return cv[2 * e]; });
+        odd = __syncthreads_or(odd);
+        const int nw = warp_list(wb, odd, n, sm.idx, n, [&](int e) { return cv[2 * e]; });
         if (nw == 0) return;
         float g[KI][4];
 #pragma unroll

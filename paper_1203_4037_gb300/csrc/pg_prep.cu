@@ -582,20 +582,21 @@ cudaError_t launch_tile_prep(const double4 *xi, const unsigned *perm, long long 
     return cudaGetLastError();
 }
 
-__global__ void k_pack_f32(const double4 *__restrict__ rec, long long n, const double4 *__restrict__ org, double sc,
-                           float4 *__restrict__ out)
+__global__ void k_pack_f32(const double4 *__restrict__ rec, const double4 *__restrict__ w, long long n,
+                           const double4 *__restrict__ org, double sc, float4 *__restrict__ out)
 {
     const long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (k >= n) return;
     const double4 v = rec[k], o = *org;
-    out[k] = make_float4((float)((v.x - o.x) * sc), (float)((v.y - o.y) * sc), (float)((v.z - o.z) * sc), (float)v.w);
+    const float m = w && odd_weight(w[k]) ? __int_as_float(0x7fffffff) : (float)v.w;
+    out[k] = make_float4((float)((v.x - o.x) * sc), (float)((v.y - o.y) * sc), (float)((v.z - o.z) * sc), m);
 }
 
-cudaError_t launch_pack_f32(const double4 *rec, long long n, const double4 *org, double scale, float4 *out,
-                            cudaStream_t st)
+cudaError_t launch_pack_f32(const double4 *rec, const double4 *w, long long n, const double4 *org, double scale,
+                            float4 *out, cudaStream_t st)
 {
     if (n <= 0) return cudaSuccess;
-    k_pack_f32<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(rec, n, org, scale, out);
+    k_pack_f32<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(rec, w, n, org, scale, out);
     return cudaGetLastError();
 }
 

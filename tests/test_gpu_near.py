@@ -179,3 +179,21 @@ def test_far_from_the_origin(pg, orc, shift):
     x = np.round(x * 2.0 ** 20) / 2.0 ** 20
     v, _, _ = table(orc, r_cut)
     assert np.array_equal(run(pg, x + shift, x + shift, m, v, r_cut, True)[0], run(pg, x, x, m, v, r_cut, True)[0])
+
+
+# K u of a pair with a non-finite loss weight is non-finite near or far (0
+# times it), on both sides of the switch to sorted tiles (16384)
+@pytest.mark.parametrize("n", [16000, 16500])
+@pytest.mark.parametrize("bad", [np.nan, np.inf])
+def test_nonfinite_weight_reaches_every_gradient(pg, orc, n, bad):
+    torch = pytest.importorskip("torch")
+    from paper_1203_4037_gb300 import autograd as AG
+    x, m = gen.plummer(n, 43)
+    w = gen.unit_vectors(n, 44)
+    far = int(np.argmax(np.linalg.norm(x, axis=1)))
+    w[far, 1] = bad
+    v, _, _ = table(orc, 0.1)
+    xt, mt = (torch.tensor(t, device="cuda", requires_grad=True) for t in (x, m))
+    a = AG.table_force(xt, mt, torch.tensor(v, device="cuda"), 0.1, E, F)
+    dx, dm = torch.autograd.grad(a, (xt, mt), torch.tensor(w, device="cuda"))
+    assert not torch.isfinite(dx).any() and not torch.isfinite(dm).any()
