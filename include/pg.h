@@ -67,7 +67,7 @@ typedef struct pg_ctx pg_ctx;
 #define PG_PATH_NARROW 2  /* few i against many j: (i chunk, j chunk) items */
 
 /* how the all-pairs paths form pair differences (pg_set_differencing) */
-#define PG_DIFF_AUTO 0    /* double-float where i-tiles are not compact (the default) */
+#define PG_DIFF_AUTO 0    /* double-float or 48-bit fixed point where i-tiles are not compact (the default) */
 #define PG_DIFF_SINGLE 1  /* one FP32 offset per particle from an FP64 tile centre */
 #define PG_DIFF_DOUBLE 2  /* double-float on every all-pairs run */
 
@@ -425,8 +425,14 @@ int pg_tune(pg_ctx *ctx);
  * Morton-ordered (from 16384 on) and at least an eighth as many as the
  * j-particles, and double on every other tiled run (PG_TABLE included: the
  * shape's steep fall toward r_cut magnifies a difference's error) and on the
- * narrow path. pg_info's out[7] reports
- * what the last run used. Groups, tree lists and the cell list keep their
+ * narrow path. Where it would take double on a PG_NEWTON run of 48 or more i
+ * against 4096 or more j, of 2^24 pairs or more (2^28 on tiled runs), with
+ * the launch shape, split and path left to the library and eps > 0 from
+ * pg_set_eps, it forms d from 48-bit fixed-point positions in the j-set's
+ * cube instead (of half side R; the tensor cores take the differences, with
+ * an error of 2^-23 of |d| and 2^-47 R at most); the device takes double where
+ * the values do not fit that. pg_info's out[7] reports
+ * what the last run used (1 for the fixed point too). Groups, tree lists and the cell list keep their
  * own forms. PG_EINVAL for another mode. */
 int pg_set_differencing(pg_ctx *ctx, int mode);
 

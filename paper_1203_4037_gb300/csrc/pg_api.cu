@@ -1912,7 +1912,7 @@ int pack_j_for(pg_ctx *c, long long nj)
 bool use_tc(const pg_ctx *c)
 {
     if (c->mode != PG_NEWTON || use_ext(c) || c->np || c->split || c->ctas_per_sm || c->path != PG_PATH_AUTO ||
-        c->diff_mode == PG_DIFF_SINGLE || !c->packed)
+        c->diff_mode != PG_DIFF_AUTO || !c->packed)
         return false;
     const long long ni = c->ni, nj = nj_of(c);
     if (ni < 48 || nj < 4096 || ni * nj < (1LL << 24)) return false;

@@ -146,3 +146,20 @@ def test_no_signed_error(pg, orc, ni, nj):
     assert info["i_per_thread"] == 64
     _, po = orc.newton(xi, xj, mj.astype(np.float32).astype(np.float64), EPS)
     assert abs(np.mean(p / po - 1)) <= 1.5e-8
+
+
+def test_double_float_when_asked_for(pg):
+    # PG_DIFF_DOUBLE is double-float on the automatic path too: the forced narrow path's bits
+    xj, mj = gen.plummer(60000, 3)
+    xi = gen.plummer(300, 4)[0]
+    out = []
+    for path in (pg.PG_PATH_AUTO, pg.PG_PATH_NARROW):
+        with pg.Context(0) as c:
+            c.set_allpairs_path(path)
+            c.set_differencing(pg.PG_DIFF_DOUBLE)
+            c.set_eps(EPS)
+            c.set_j(xj, mj)
+            c.set_i(xi)
+            c.run()
+            out.append(c.get_force(300))
+    assert np.array_equal(out[0][0], out[1][0]) and np.array_equal(out[0][1], out[1][1])
