@@ -1904,7 +1904,7 @@ int pack_j_for(pg_ctx *c, long long nj)
 // The tensor-core path (pg_tc.cu): Newton runs of the default shape that
 // would difference in double-float, with enough pairs for its preparation and
 // the stand-in's empty launches. Whether this call's values fit its fixed
-// point (every i within the j-set's cube, eps within 2^-30 to 2^10 of its half
+// point (every i within the j-set's cube, eps within 2^-22 to 2^10 of its half
 // side) is known on the device only: the double-float path is enqueued behind it
 // and runs where they do not. From 48 i on: fewer leave most of a 32- or
 // 64-particle tile empty (2^20 j, kernel: 16 i 25 us, as the warp-mode

@@ -514,9 +514,11 @@ __global__ void k_tc_pack(const double4 *__restrict__ jrec, long long nj, long l
 }
 
 // The i-particles' digits, and whether this call can use them: every i within
-// the cube, and eps within the range where the digits' resolution
-// (R 2^-47, at most 2^-17 eps) and the FP32 range of the sums hold. The last
-// block writes the verdict.
+// the cube, and eps within 2^-22 to 2^10 R. Below, one step of the positions
+// (R 2^-47) is no longer small against FP32's rounding of a pair at eps (with
+// eps = 2^-30 R, i at 0.5 to 2 eps from a j have force errors of 3.5e-6 median
+// and 1.4e-5 at most; at 2^-22 R the steps are 1/4 ulp of eps); above, the
+// sums leave FP32's range. The last block writes the verdict.
 __global__ void __launch_bounds__(256) k_tc_prep(const double4 *__restrict__ xi, long long ni, long long npad,
                                                  float eps2, TcGeo *geo, unsigned char *__restrict__ idig,
                                                  unsigned *words, int *ok)
@@ -541,9 +543,9 @@ __global__ void __launch_bounds__(256) k_tc_prep(const double4 *__restrict__ xi,
     __threadfence();
     const bool far = __ldcg(words) != 0;
     // eps in units of the upper digits' last place, u = R 2^-23
-    const double e2 = ldexp((double)eps2, 2 * (23 - g.e)) * ((1.0 - kShort) * (1.0 - kShort));
-    const bool range = e2 >= 0x1p-14 && e2 <= 0x1p66;
-    geo->e2 = (float)e2;
+    const double e2 = ldexp((double)eps2, 2 * (23 - g.e));
+    const bool range = e2 >= 0x1p2 && e2 <= 0x1p66;
+    geo->e2 = (float)(e2 * ((1.0 - kShort) * (1.0 - kShort)));
     *ok = g.ok && !far && range;
     words[0] = words[1] = 0;
 }

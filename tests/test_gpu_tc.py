@@ -163,3 +163,23 @@ def test_double_float_when_asked_for(pg):
             c.run()
             out.append(c.get_force(300))
     assert np.array_equal(out[0][0], out[1][0]) and np.array_equal(out[0][1], out[1][1])
+
+
+def both(pg, xi, xj, mj, eps, **kw):
+    """The automatic path's (a, phi), and whether the tensor cores made them:
+    the stand-in's bits are those of the forced narrow path."""
+    a, p, _ = run(pg, xi, xj, mj, eps, **kw)
+    a2, p2, _ = run(pg, xi, xj, mj, eps, path=pg.PG_PATH_NARROW, **kw)
+    return a, p, not (np.array_equal(a, a2) and np.array_equal(p, p2))
+
+
+# one far j sets the step of all positions, R 2^-47: just inside the accepted
+# range (R = 4096, eps 2^22 times smaller), just outside, and far outside
+@pytest.mark.parametrize("far, fits", [(30.0, True), (6000.0, True), (8000.0, False), (1.6e6, False)])
+def test_close_pairs_beside_a_far_particle(pg, orc, far, fits):
+    xj, mj = gen.plummer(60000, 3)
+    xi = near_j(xj, 300, 9, EPS)
+    xj[11] = [far, 0.0, 0.0]
+    a, p, tc = both(pg, xi, xj, mj, EPS)
+    assert tc == fits
+    check(orc, a, p, xi, xj, mj, EPS)
