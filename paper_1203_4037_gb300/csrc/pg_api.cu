@@ -1905,7 +1905,7 @@ int pack_j_for(pg_ctx *c, long long nj)
 // would difference in double-float, with enough pairs for its preparation and
 // the stand-in's empty launches. Whether this call's values fit its fixed
 // point (every i within the j-set's cube, eps within 2^-22 to 2^10 of its half
-// side) is known on the device only: the double-float path is enqueued behind it
+// side, no mass too far below the largest) is known on the device only: the double-float path is enqueued behind it
 // and runs where they do not. From 48 i on: fewer leave most of a 32- or
 // 64-particle tile empty (2^20 j, kernel: 16 i 25 us, as the warp-mode
 // kernel's 25; 64 i 41 against 72; 1000 i 460 against 840).
@@ -1926,7 +1926,7 @@ int pack_tc(pg_ctx *c, long long nj)
 {
     if (c->tc_n == nj) return PG_OK;
     unsigned long long *words = (unsigned long long *)c->tc_geo.p;
-    PG_CUDA(c, launch_tc_pack((const double4 *)c->jrec.p, nj, words, (TcGeo *)(words + 10),
+    PG_CUDA(c, launch_tc_pack((const double4 *)c->jrec.p, nj, words, (TcGeo *)(words + kTcBoxWords + 2),
                               (unsigned char *)c->tc_dig.p, tc_mass(c, nj), c->stream));
     c->last_launches += 2;
     c->tc_n = nj;
@@ -1964,7 +1964,7 @@ int tc_room(pg_ctx *c)
     if (c->capturing)
         return c->tc_geo.cap && c->tc_dig.cap >= dig && c->part.cap >= part ? PG_OK : PG_ENOMEM;
     if (c->tc_geo.cap == 0) {
-        if ((rc = ensure(c, c->tc_geo, 10 * 8 + sizeof(TcGeo) + 16))) return rc;
+        if ((rc = ensure(c, c->tc_geo, (kTcBoxWords + 2) * 8 + sizeof(TcGeo)))) return rc;
         PG_CUDA(c, cudaMemsetAsync(c->tc_geo.p, 0, c->tc_geo.cap, c->stream));
     }
     if ((rc = ensure(c, c->tc_dig, dig))) return rc;
@@ -1976,14 +1976,16 @@ int enqueue_tc(pg_ctx *c, double *acc, double *pot)
     int rc;
     const long long ni = c->ni, nj = nj_of(c);
     const TcShape t = tc_shape(c);
-    unsigned long long *words = (unsigned long long *)c->tc_geo.p;   // 8: box, 1: the i flags, 1: the verdict
+    // the box's words, one for the i flags, one for the verdict, the geometry
+    unsigned long long *words = (unsigned long long *)c->tc_geo.p;
+    TcGeo *geo = (TcGeo *)(words + kTcBoxWords + 2);
     TcArgs a{};
     a.dig = (const unsigned char *)c->tc_dig.p;
     a.mass = tc_mass(c, nj);
     unsigned char *idig = (unsigned char *)c->part.p + t.part;
     a.idig = idig;
-    a.geo = (const TcGeo *)(words + 10);
-    int *ok = (int *)(words + 9);
+    a.geo = geo;
+    int *ok = (int *)(words + kTcBoxWords + 1);
     a.ok = ok;
     a.ni = ni;
     a.W = t.W;
@@ -1993,8 +1995,8 @@ int enqueue_tc(pg_ctx *c, double *acc, double *pot)
     a.status = (int *)c->status.p;
     if (c->capturing) c->graph_tc = true;
     else if ((rc = pack_tc(c, nj))) return rc;
-    PG_CUDA(c, launch_tc_prep((const double4 *)c->xi.p, ni, (float)(c->eps * c->eps), (TcGeo *)(words + 10),
-                              idig, (unsigned *)(words + 8), ok, c->stream));
+    PG_CUDA(c, launch_tc_prep((const double4 *)c->xi.p, ni, (float)(c->eps * c->eps), geo, idig,
+                              (unsigned *)(words + kTcBoxWords), ok, c->stream));
     if (c->timing) PG_CUDA(c, record_timing(c, c->tk0));
     PG_CUDA(c, launch_tc(a, t.grid, c->stream));
     const bool timing = c->timing;

@@ -271,6 +271,7 @@ struct TcGeo {             // set on the device from the j-set
     double cx, cy, cz;     // the cube's centre
     double scale;          // position -> fixed point, 2^47 / R
     double mscale;         // mass -> staged mass, 2^mexp
+    double mmin;           // smallest nonzero staged |mass| (0: none)
     int e, mexp;           // R = 2^e
     int ok;                // finite and in range
     float e2;              // eps^2 in the kernel's unit (R 2^-23), set by each call's preparation
@@ -290,7 +291,8 @@ int tc_bi(long long ni);                   // i-particles per tile
 size_t tc_dig_bytes(long long n);
 int tc_jtiles(long long nj);
 int tc_slots(long long ntiles, int njt, long long W, int grid);
-// words: 8 u64, zero before the first call and kept so
+// words: kTcBoxWords u64, zero before the first call and kept so
+constexpr int kTcBoxWords = 9;
 cudaError_t launch_tc_pack(const double4 *jrec, long long nj, unsigned long long *words, TcGeo *geo,
                            unsigned char *dig, float *mass, cudaStream_t st);
 // words: 2, zero before the first call and kept so; ok: the verdict

@@ -438,15 +438,16 @@ __device__ __forceinline__ double unord64(u64 u)
     return __longlong_as_double((long long)((u >> 63) ? (u & 0x7fffffffffffffffull) : ~u));
 }
 
-// The j-set's cube and largest mass; the last block to finish sets the
-// geometry and clears the words for the next call. words: 3 minima (stored
-// inverted, so that zero starts them all), 3 maxima, largest |m| (as bits,
-// all ones with a non-finite value), ticket.
+// The j-set's cube, largest and smallest nonzero mass; the last block to
+// finish sets the geometry and clears the words for the next call. words: 3
+// minima (stored inverted, so that zero starts them all), 3 maxima, largest
+// |m| (as bits, all ones with a non-finite value), smallest nonzero |m|
+// (inverted bits), ticket.
 __global__ void __launch_bounds__(256) k_tc_box(const double4 *__restrict__ jrec, long long nj, u64 *words,
                                                 TcGeo *geo)
 {
-    __shared__ u64 sh[7][8];
-    u64 v[7] = {0, 0, 0, 0, 0, 0, 0};
+    __shared__ u64 sh[8][8];
+    u64 v[8] = {0, 0, 0, 0, 0, 0, 0, 0};
     for (long long k = blockIdx.x * 256ll + threadIdx.x; k < nj; k += gridDim.x * 256ll) {
         const double4 r = jrec[k];
         const u64 o[3] = {ord64(r.x), ord64(r.y), ord64(r.z)};
@@ -456,30 +457,32 @@ __global__ void __launch_bounds__(256) k_tc_box(const double4 *__restrict__ jrec
             v[3 + d] = max(v[3 + d], o[d]);
         }
         const bool fin = isfinite(r.x) && isfinite(r.y) && isfinite(r.z) && isfinite(r.w);
-        v[6] = max(v[6], fin ? (u64)__double_as_longlong(fabs(r.w)) : ~0ull);
+        const u64 mb = (u64)__double_as_longlong(fabs(r.w));
+        v[6] = max(v[6], fin ? mb : ~0ull);
+        v[7] = max(v[7], mb ? ~mb : 0ull);
     }
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
 #pragma unroll
-    for (int q = 0; q < 7; ++q) {
+    for (int q = 0; q < 8; ++q) {
         for (int o = 16; o; o >>= 1) v[q] = max(v[q], __shfl_xor_sync(0xffffffffu, v[q], o));
         if (lane == 0) sh[q][w] = v[q];
     }
     __syncthreads();
-    if (threadIdx.x < 7) {
+    if (threadIdx.x < 8) {
         u64 m = 0;
         for (int q = 0; q < 8; ++q) m = max(m, sh[threadIdx.x][q]);
         atomicMax(words + threadIdx.x, m);
         __threadfence();
     }
     __syncthreads();
-    if (threadIdx.x != 0 || atomicAdd(words + 7, 1ull) != gridDim.x - 1) return;
+    if (threadIdx.x != 0 || atomicAdd(words + 8, 1ull) != gridDim.x - 1) return;
     __threadfence();
     double lo[3], hi[3];
     for (int d = 0; d < 3; ++d) {
         lo[d] = unord64(~__ldcg(words + d));
         hi[d] = unord64(__ldcg(words + 3 + d));
     }
-    const u64 mb = __ldcg(words + 6);
+    const u64 mb = __ldcg(words + 6), ms = __ldcg(words + 7);
     TcGeo g{};
     g.ok = 0;
     if (mb != ~0ull) {
@@ -494,10 +497,11 @@ __global__ void __launch_bounds__(256) k_tc_box(const double4 *__restrict__ jrec
         const int em = mb ? ilogb(__longlong_as_double((long long)mb)) : 0;
         g.mscale = ldexp(1.0, 20 - em);        // masses enter at most 2^21
         g.mexp = 20 - em;
+        g.mmin = ms ? __longlong_as_double((long long)~ms) * g.mscale : 0.0;
         g.ok = half < 1e300 && e > -900 && e < 900 && em > -900 && em < 900;
     }
     *geo = g;
-    for (int q = 0; q < 8; ++q) words[q] = 0;
+    for (int q = 0; q < kTcBoxWords; ++q) words[q] = 0;
 }
 
 // the j records' digits and scaled masses, padded with massless records
@@ -518,7 +522,9 @@ __global__ void k_tc_pack(const double4 *__restrict__ jrec, long long nj, long l
 // (R 2^-47) is no longer small against FP32's rounding of a pair at eps (with
 // eps = 2^-30 R, i at 0.5 to 2 eps from a j have force errors of 3.5e-6 median
 // and 1.4e-5 at most; at 2^-22 R the steps are 1/4 ulp of eps); above, the
-// sums leave FP32's range. The last block writes the verdict.
+// sums leave FP32's range. So do those of masses too far below the largest:
+// m / r^3 at the cube's diagonal is to stay above 2^-110 (2^-75 of the
+// largest mass at small eps). The last block writes the verdict.
 __global__ void __launch_bounds__(256) k_tc_prep(const double4 *__restrict__ xi, long long ni, long long npad,
                                                  float eps2, TcGeo *geo, unsigned char *__restrict__ idig,
                                                  unsigned *words, int *ok)
@@ -544,7 +550,8 @@ __global__ void __launch_bounds__(256) k_tc_prep(const double4 *__restrict__ xi,
     const bool far = __ldcg(words) != 0;
     // eps in units of the upper digits' last place, u = R 2^-23
     const double e2 = ldexp((double)eps2, 2 * (23 - g.e));
-    const bool range = e2 >= 0x1p2 && e2 <= 0x1p66;
+    const double rmax = rsqrt(3.0 * 0x1p48 + e2);
+    const bool range = e2 >= 0x1p2 && e2 <= 0x1p66 && (g.mmin == 0.0 || g.mmin * (rmax * rmax * rmax) >= 0x1p-110);
     geo->e2 = (float)(e2 * ((1.0 - kShort) * (1.0 - kShort)));
     *ok = g.ok && !far && range;
     words[0] = words[1] = 0;

@@ -183,3 +183,19 @@ def test_close_pairs_beside_a_far_particle(pg, orc, far, fits):
     a, p, tc = both(pg, xi, xj, mj, EPS)
     assert tc == fits
     check(orc, a, p, xi, xj, mj, EPS)
+
+
+# one body 2^k times as heavy as the others: their m / r^3, all of the force
+# on the heavy one, has to stay in FP32's range
+@pytest.mark.parametrize("k, fits", [(40, True), (110, False)])
+def test_one_heavy_body(pg, orc, k, fits):
+    x, m = gen.plummer(60000, 8)
+    m = np.full(60000, 2.0 ** -k)
+    m[5] = 1.0
+    a, p, tc = both(pg, x[:300], x, m, 0.01, self_=True)
+    assert tc == fits
+    # the heavy body's own potential is not compared: its own pair's m / eps is
+    # added and taken out in FP32 on every path (2e-3 off at 2^40, all of it from 2^60 on)
+    ao, po = orc.newton(x[:300], x, m, 0.01, skip=np.arange(300, dtype=np.int64))
+    assert_parity(rel_vec(a, ao), what="a")
+    assert_parity(np.delete(rel_scalar(p, po), 5), what="phi")
