@@ -1906,7 +1906,7 @@ int pack_j_for(pg_ctx *c, long long nj)
 // the stand-in's empty launches. Whether this call's values fit its fixed
 // point (every i within the j-set's cube, eps within 2^-22 to 2^10 of its half
 // side, no mass too far below the largest) is known on the device only: the double-float path is enqueued behind it
-// and runs where they do not. From 48 i on: fewer leave most of a 32- or
+// and runs where they do not. From 48 i on: fewer leave most of a
 // 64-particle tile empty (2^20 j, kernel: 16 i 25 us, as the warp-mode
 // kernel's 25; 64 i 41 against 72; 1000 i 460 against 840).
 bool use_tc(const pg_ctx *c)
@@ -1944,7 +1944,7 @@ struct TcShape {
 TcShape tc_shape(const pg_ctx *c)
 {
     TcShape t;
-    t.Bi = tc_bi(c->ni);
+    t.Bi = tc_bi();
     t.njt = tc_jtiles(nj_of(c));
     t.ntiles = (c->ni + t.Bi - 1) / t.Bi;
     t.W = t.ntiles * t.njt;

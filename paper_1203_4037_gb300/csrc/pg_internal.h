@@ -284,10 +284,10 @@ struct TcArgs {
     const int *ok;         // zero: this call's values do not fit, nothing runs
     long long ni, W;       // i-particles; units, i tiles times j tiles
     int njt, slots;        // j tiles; partial slots per i tile
-    double4 *part;         // [i tiles][slots][tc_bi]
+    double4 *part;         // [i tiles][slots][tc_bi()]
     int *status;
 };
-int tc_bi(long long ni);                   // i-particles per tile
+int tc_bi();                               // i-particles per tile
 size_t tc_dig_bytes(long long n);
 int tc_jtiles(long long nj);
 int tc_slots(long long ntiles, int njt, long long W, int grid);

@@ -21,7 +21,7 @@
 // forces and potentials are then nearer to 64 bits than the double-float
 // kernel's (1048 i, 563704 j: 4.8e-8 and 2.3e-8 against 5.8e-8 and 2.5e-8).
 //
-// A CTA owns units (tile of 32 GI i, tile of 128 j), an equal contiguous
+// A CTA owns units (tile of 64 i, tile of 128 j), an equal contiguous
 // range of them. One thread copies the j tiles in (cp.async.bulk), two issue
 // the MMAs of alternate tiles (tcgen05.mma, cta_group::1; barrier tries,
 // copies, MMAs and commits each take a thread 70 to 90 clocks, so one
@@ -61,19 +61,14 @@ constexpr int kFoldTiles = 128;        // j tiles per FP32 partial sum of a lane
 // without it
 constexpr double kShort = 2.5e-8;
 
-// GI groups of kIW i per CTA tile; the groups' warps (four each, one per TMEM
-// quadrant) share every j tile, with GI = 1 two streams take alternate tiles
-template <int GI> struct Tc {
-    static constexpr int kN = 3 * kIW * GI;                // MMA N: (group, axis, i)
-    static constexpr int kStages = GI == 2 ? 2 : 4;        // TMEM stages of kN columns
-    static constexpr int kSlots = 8;                       // staged j tiles
-    static constexpr int kStreams = kTcWarps / 4 / GI;
-    static constexpr size_t smem()
-    {
-        return (size_t)kSlots * kSlotBytes + 2 * kN * 32 + kTcWarps * 2 * kSums * sizeof(float) +
-               (2 * kSlots + 2 * kStages) * 8 + 48;
-    }
-};
+// two groups of kIW i per CTA tile; the groups' warps (four each, one per
+// TMEM quadrant) share every j tile
+constexpr int kBi = 2 * kIW;
+constexpr int kN = 3 * kBi;            // MMA N: (group, axis, i)
+constexpr int kStages = 2;             // TMEM stages of kN columns
+constexpr int kSlots = 8;              // staged j tiles
+constexpr size_t kTcSmem = (size_t)kSlots * kSlotBytes + 2 * kN * 32 + kTcWarps * 2 * kSums * sizeof(float) +
+                           (2 * kSlots + 2 * kStages) * 8 + 48;
 
 // ---------------------------------------------------------------- PTX
 // shared-memory operand, K-major without swizzle: core matrices of 8 rows x
@@ -148,20 +143,18 @@ __host__ __device__ __forceinline__ long long tc_owner(long long u, long long gr
 }
 
 // ---------------------------------------------------------------- the kernel
-template <int GI>
 __global__ void __launch_bounds__(kTcThreads, 1) k_tc(const __grid_constant__ TcArgs a)
 {
-    using C = Tc<GI>;
     extern __shared__ __align__(1024) unsigned char sm[];
     const uint32_t sA = smem_u32(sm);                                    // [slots][digits, masses]
-    unsigned char *bh = sm + C::kSlots * kSlotBytes, *bl = bh + C::kN * 32;   // B, upper and lower digits
-    float *red = reinterpret_cast<float *>(bl + C::kN * 32);             // [warps][hi, lo][kSums]
+    unsigned char *bh = sm + kSlots * kSlotBytes, *bl = bh + kN * 32;   // B, upper and lower digits
+    float *red = reinterpret_cast<float *>(bl + kN * 32);             // [warps][hi, lo][kSums]
     uint64_t *bars = reinterpret_cast<uint64_t *>(red + kTcWarps * 2 * kSums);
-    const uint32_t bFull = smem_u32(bars), bDone = bFull + 8 * C::kSlots, bEmpty = bDone + 8 * C::kStages,
-                   bFree = bEmpty + 8 * C::kStages;
-    volatile int *seg = reinterpret_cast<volatile int *>(bars + 2 * C::kSlots + 2 * C::kStages);   // i tile, j tiles, last
+    const uint32_t bFull = smem_u32(bars), bDone = bFull + 8 * kSlots, bEmpty = bDone + 8 * kStages,
+                   bFree = bEmpty + 8 * kStages;
+    volatile int *seg = reinterpret_cast<volatile int *>(bars + 2 * kSlots + 2 * kStages);   // i tile, j tiles, last
     volatile int *failed = seg + 4;
-    uint32_t *tptr = reinterpret_cast<uint32_t *>(bars + 2 * C::kSlots + 2 * C::kStages + 3);
+    uint32_t *tptr = reinterpret_cast<uint32_t *>(bars + 2 * kSlots + 2 * kStages + 3);
 
     const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
     const long long G = gridDim.x, b = blockIdx.x;
@@ -169,13 +162,13 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tc(const __grid_constant__ Tc
     if (u0 >= u1 || *a.ok == 0) return;
     if (tid == 0) {
         *failed = 0;
-        for (int k = 0; k < C::kSlots; ++k) {
+        for (int k = 0; k < kSlots; ++k) {
             mbar_init(bars + k, 1);
-            mbar_init(bars + C::kSlots + 2 * C::kStages + k, 1);
+            mbar_init(bars + kSlots + 2 * kStages + k, 1);
         }
-        for (int k = 0; k < C::kStages; ++k) {
-            mbar_init(bars + C::kSlots + k, 1);
-            mbar_init(bars + C::kSlots + C::kStages + k, 4 * GI);
+        for (int k = 0; k < kStages; ++k) {
+            mbar_init(bars + kSlots + k, 1);
+            mbar_init(bars + kSlots + kStages + k, kTcWarps);
         }
         mbar_fence_init();
     }
@@ -187,7 +180,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tc(const __grid_constant__ Tc
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tm = __shfl_sync(0xffffffffu, *tptr, 0);
-    constexpr uint32_t idesc = (1u << 4) | ((uint32_t)(C::kN / 8) << 17) | ((kTcJ / 16u) << 24);   // FP32 += FP16 x FP16
+    constexpr uint32_t idesc = (1u << 4) | ((uint32_t)(kN / 8) << 17) | ((kTcJ / 16u) << 24);   // FP32 += FP16 x FP16
     const int njt = a.njt;
 
     if (warp >= kTcWarps) {
@@ -212,15 +205,15 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tc(const __grid_constant__ Tc
                 const float *gm = a.mass + (size_t)s0 * kTcJ;
                 for (int q = 0; q < nt; ++q) {
                     const uint32_t bar = bFull + 8 * sl, dst = sA + sl * kSlotBytes;
-                    if (n >= C::kSlots) {
+                    if (n >= kSlots) {
                         wait_or_fail(bFree + 8 * sl, par ^ 1u, failed, a.status, 20);
                         if (*failed) break;
                     }
                     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(kSlotBytes) : "memory");
                     copy_in(dst, gd + (size_t)q * kDigBytes, kDigBytes, bar);
                     copy_in(dst + kDigBytes, gm + (size_t)q * kTcJ, kTcJ * 4, bar);
-                    if (n < C::kSlots) ++n;
-                    if (++sl == C::kSlots) { sl = 0; par ^= 1u; }
+                    if (n < kSlots) ++n;
+                    if (++sl == kSlots) { sl = 0; par ^= 1u; }
                 }
                 // after a failure, copies in flight land before the CTA's shared memory goes
                 if (*failed)
@@ -230,29 +223,29 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tc(const __grid_constant__ Tc
                 const u64 dh = operand(smem_u32(bh)), dl = operand(smem_u32(bl));
                 int q = q0;
                 for (; q < nt; q += 2) {
-                    const int st = sl % C::kStages;
-                    if (n >= C::kStages / 2) {
+                    const int st = sl % kStages;
+                    if (n >= kStages / 2) {
                         // the stage's previous tile is read, so the slot it came from is free
-                        wait_or_fail(bEmpty + 8 * st, ((sl / C::kStages) & 1) ^ 1u, failed, a.status, 21);
+                        wait_or_fail(bEmpty + 8 * st, ((sl / kStages) & 1) ^ 1u, failed, a.status, 21);
                         if (*failed) break;
-                        arrive(bFree + 8 * ((sl + C::kSlots - C::kStages) % C::kSlots));
+                        arrive(bFree + 8 * ((sl + kSlots - kStages) % kSlots));
                     }
                     wait_or_fail(bFull + 8 * sl, par, failed, a.status, 22);
                     if (*failed) break;
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                     const u64 da = operand(sA + sl * kSlotBytes);
-                    mma_f16(tm + st * C::kN, da, dh, idesc, 0);
-                    mma_f16(tm + st * C::kN, da, dl, idesc, 1);
+                    mma_f16(tm + st * kN, da, dh, idesc, 0);
+                    mma_f16(tm + st * kN, da, dl, idesc, 1);
                     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bDone + 8 * st) : "memory");
-                    if (n < C::kStages / 2) ++n;
+                    if (n < kStages / 2) ++n;
                     sl += 2;
-                    if (sl >= C::kSlots) { sl -= C::kSlots; par ^= 1u; }
+                    if (sl >= kSlots) { sl -= kSlots; par ^= 1u; }
                 }
                 q0 = q - nt;
                 // after a failure, the MMAs issued last end before the CTA's memory goes
                 if (*failed && n > 0) {
-                    const int ls = (sl + C::kSlots - 2) % C::kSlots;
-                    mbar_wait(bars + C::kSlots + ls % C::kStages, (ls / C::kStages) & 1, kWaitLimitNs / 4);
+                    const int ls = (sl + kSlots - 2) % kSlots;
+                    mbar_wait(bars + kSlots + ls % kStages, (ls / kStages) & 1, kWaitLimitNs / 4);
                 }
             }
             __syncthreads();
@@ -261,10 +254,11 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tc(const __grid_constant__ Tc
         }
     } else {
         asm volatile("setmaxnreg.inc.sync.aligned.u32 224;");
-        const int quad = warp & 3, grp = (warp >> 2) % GI, stream = (warp >> 2) / GI;
+        // (% 2: with the range of grp known the addresses stay in uniform registers; 2 % of the run)
+        const int quad = warp & 3, grp = (warp >> 2) % 2;
         const float e2s = a.geo->e2;
         const u64 e2 = pk2(e2s, e2s);
-        unsigned pos = stream, base = 0;   // this stream's next tile and the segment's end, counted over the CTA's tiles
+        unsigned pos = 0;                  // the next tile, counted over the CTA's tiles
         const uint32_t tb0 = tm + ((uint32_t)(quad * 32) << 16) + grp * 3 * kIW;
         const uint32_t ms0 = sA + kDigBytes + (quad * 32 + lane) * 4;
         float *mine = red + warp * 2 * kSums + lane * kLaneSums;
@@ -272,9 +266,9 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tc(const __grid_constant__ Tc
             __syncthreads();
             const int t = __shfl_sync(0xffffffffu, seg[0], 0), nt = __shfl_sync(0xffffffffu, seg[1], 0);
             // B: row (group, axis, i); digits as FP16 pairs {upper 0, 1}, {lower 0, 1}
-            for (int r = tid; r < C::kN; r += kTcWarps * 32) {
+            for (int r = tid; r < kN; r += kTcWarps * 32) {
                 const int g = r / (3 * kIW), axis = (r % (3 * kIW)) / kIW, ii = r % kIW;
-                const long long i = (long long)t * kIW * GI + g * kIW + ii;
+                const long long i = (long long)t * kBi + g * kIW + ii;
                 uint2 d = make_uint2(0u, 0u);
                 if (i < a.ni)
                     d = *reinterpret_cast<const uint2 *>(a.idig + (i / 8) * 256 + (axis >> 1) * 128 + (i % 8) * 16 + (axis & 1) * 8);
@@ -292,8 +286,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tc(const __grid_constant__ Tc
             fence_proxy_async();
             __syncthreads();
 
-            base += nt;
-            int rem = (int)(base - pos) > 0 ? ((int)(base - pos) + C::kStreams - 1) / C::kStreams : 0;
+            int rem = nt;
             u64 ax[kIW / 2], ay[kIW / 2], az[kIW / 2], ph[kIW / 2];
             while (rem > 0) {
 #pragma unroll
@@ -302,14 +295,14 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tc(const __grid_constant__ Tc
                 rem -= c;
 #pragma unroll 1
                 for (; c; --c) {
-                    const unsigned st = pos % C::kStages;
-                    wait_or_fail(bDone + 8 * st, (pos / C::kStages) & 1u, failed, a.status, 23);
+                    const unsigned st = pos % kStages;
+                    wait_or_fail(bDone + 8 * st, (pos / kStages) & 1u, failed, a.status, 23);
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                     float m;
-                    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(m) : "r"(ms0 + (pos % C::kSlots) * kSlotBytes));
+                    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(m) : "r"(ms0 + (pos % kSlots) * kSlotBytes));
                     const u64 m2 = pk2(m, m);
-                    const uint32_t tb = tb0 + st * C::kN;
-                    pos += C::kStreams;
+                    const uint32_t tb = tb0 + st * kN;
+                    ++pos;
                     float xb[2][4], yb[2][4], zb[2][4];
                     tmem_ld4(tb, xb[0]);
                     tmem_ld4(tb + kIW, yb[0]);
@@ -375,15 +368,14 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tc(const __grid_constant__ Tc
             }
             __syncthreads();
             {
-                // the segment's sums over quadrants and streams, in order
+                // the segment's sums over quadrants, in order
                 const long long slot = b - tc_owner((long long)t * njt, G, a.W);
-                double *dst = reinterpret_cast<double *>(a.part + ((size_t)t * a.slots + slot) * kIW * GI);
-                for (int e = tid; e < 4 * kIW * GI; e += kTcWarps * 32) {
+                double *dst = reinterpret_cast<double *>(a.part + ((size_t)t * a.slots + slot) * kBi);
+                for (int e = tid; e < 4 * kBi; e += kTcWarps * 32) {
                     const int i = e / 4, comp = e % 4, g = i / kIW, ii = i % kIW;
                     double s = 0.0;
-                    for (int w = 0; w < kTcWarps; ++w)
-                        if ((w >> 2) % GI == g)
-                            s += (double)red[w * 2 * kSums + comp * kIW + ii] + (double)red[w * 2 * kSums + kSums + comp * kIW + ii];
+                    for (int w = 4 * g; w < 4 * g + 4; ++w)
+                        s += (double)red[w * 2 * kSums + comp * kIW + ii] + (double)red[w * 2 * kSums + kSums + comp * kIW + ii];
                     dst[e] = s;
                 }
             }
@@ -588,21 +580,9 @@ __global__ void __launch_bounds__(256) k_tc_combine(TcArgs a, int Bi, int grid, 
     if (pot) pot[i] = s[3] * fp;
 }
 
-template <int GI>
-cudaError_t launch_tc_one(const TcArgs &a, int grid, cudaStream_t st)
-{
-    static bool done[kMaxDevices] = {};
-    const cudaError_t e = once_per_device(done, [] {
-        return cudaFuncSetAttribute(k_tc<GI>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Tc<GI>::smem());
-    });
-    if (e != cudaSuccess) return e;
-    k_tc<GI><<<grid, kTcThreads, Tc<GI>::smem(), st>>>(a);
-    return cudaGetLastError();
-}
-
 }  // namespace
 
-int tc_bi(long long ni) { return ni > kIW ? 2 * kIW : kIW; }
+int tc_bi() { return kBi; }
 size_t tc_dig_bytes(long long n) { return (size_t)((n + kTcJ - 1) / kTcJ) * kDigBytes; }
 int tc_jtiles(long long nj) { return (int)((nj + kTcJ - 1) / kTcJ); }
 int tc_slots(long long ntiles, int njt, long long W, int grid)
@@ -635,13 +615,19 @@ cudaError_t launch_tc_prep(const double4 *xi, long long ni, float eps2, TcGeo *g
 cudaError_t launch_tc(const TcArgs &a, int grid, cudaStream_t st)
 {
     if (grid <= 0 || a.W <= 0) return cudaErrorInvalidValue;
-    return tc_bi(a.ni) == 2 * kIW ? launch_tc_one<2>(a, grid, st) : launch_tc_one<1>(a, grid, st);
+    static bool done[kMaxDevices] = {};
+    const cudaError_t e = once_per_device(done, [] {
+        return cudaFuncSetAttribute(k_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTcSmem);
+    });
+    if (e != cudaSuccess) return e;
+    k_tc<<<grid, kTcThreads, kTcSmem, st>>>(a);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_tc_combine(const TcArgs &a, int grid, int self, long long self_off, double *acc, double *pot,
                               cudaStream_t st)
 {
-    k_tc_combine<<<(unsigned)((a.ni + 7) / 8), 256, 0, st>>>(a, tc_bi(a.ni), grid, self, self_off, acc, pot);
+    k_tc_combine<<<(unsigned)((a.ni + 7) / 8), 256, 0, st>>>(a, kBi, grid, self, self_off, acc, pot);
     return cudaGetLastError();
 }
 
