@@ -155,10 +155,13 @@ struct pg_ctx {
     long long jhl_n = -1;         // j records in g_jhl as double-float pairs (-1: stale)
     long long ihl_n = -1;         // i-particles in g_ihl as double-float pairs, caller order (-1: stale)
 
-    // Newton all pairs on the tensor cores: j digits and masses (of tc_n
-    // records, -1: stale), geometry and flag words
+    // Newton all pairs on the tensor cores: j digits and masses, geometry and
+    // flag words. The geometry is that of tc_box_n records (-1: stale) and the
+    // tc_gen-th taken; the digits are those of tc_n records where they fit with tc_eps
     DevBuf tc_dig, tc_geo;
-    long long tc_n = -1;
+    long long tc_n = -1, tc_box_n = -1, tc_gen = 0;
+    double tc_eps = -1.0;
+    TcSeen *tc_seen = nullptr;    // page-locked
     bool graph_tc = false;        // the captured run reads the j digits
     const int *skip = nullptr;    // set while the run's stand-in is enqueued: it runs where this word is zero
 
@@ -247,6 +250,19 @@ int ensure(pg_ctx *c, DevBuf &b, size_t bytes)
     }
     b.cap = want;
     return PG_OK;
+}
+
+// the j records of the tensor-core path, or the double-float records that its
+// stand-in packed, are no longer what its geometry says
+void tc_stale(pg_ctx *c) { c->tc_n = c->tc_box_n = -1; }
+
+// g_jhl grown: what it held is gone
+int ensure_jhl(pg_ctx *c, size_t bytes)
+{
+    if (bytes <= c->g_jhl.cap) return PG_OK;
+    c->jhl_n = -1;
+    tc_stale(c);
+    return ensure(c, c->g_jhl, bytes);
 }
 
 int ensure_pin(pg_ctx *c, PinBuf &b, size_t bytes);
@@ -520,6 +536,7 @@ void pg_destroy(pg_ctx *c)
                       &c->bw_wt, &c->bw_dv, &c->tickets, &c->t_ext, &c->j_f32, &c->t_cost, &c->t_dense, &c->t_start,
                       &c->tc_dig, &c->tc_geo};
     for (DevBuf *b : bufs) free_dev(*b);
+    if (c->tc_seen) cudaFreeHost(c->tc_seen);
     for (DevBuf &b : c->tb) free_dev(b);
     for (DevBuf *b : {&c->pm_rec, &c->pm_x, &c->pm_m, &c->pm_acc, &c->pm_pot}) free_dev(*b);
     pm_destroy(c->pm);
@@ -961,7 +978,7 @@ int pg_set_j(pg_ctx *c, long long adr, long long nj, const double *x, const doub
     PG_CUDA(c, launch_pack_j(dx, dx + 3 * nj, (double4 *)c->jrec.p + adr, nj, c->stream));
     c->nj_hw = std::max(c->nj_hw, adr + nj);
     c->jhl_n = -1;
-    c->tc_n = -1;
+    tc_stale(c);
     return PG_OK;
 }
 
@@ -977,7 +994,7 @@ int pg_set_j_rec_dev(pg_ctx *c, long long adr, long long nj, const double *rec)
                                cudaMemcpyDeviceToDevice, c->stream));
     c->nj_hw = std::max(c->nj_hw, adr + nj);
     c->jhl_n = -1;
-    c->tc_n = -1;
+    tc_stale(c);
     return PG_OK;
 }
 
@@ -992,7 +1009,7 @@ int pg_set_j_dev(pg_ctx *c, long long adr, long long nj, const double *x, const 
     PG_CUDA(c, launch_pack_j(x, m, (double4 *)c->jrec.p + adr, nj, c->stream));
     c->nj_hw = std::max(c->nj_hw, adr + nj);
     c->jhl_n = -1;
-    c->tc_n = -1;
+    tc_stale(c);
     return PG_OK;
 }
 
@@ -1397,7 +1414,7 @@ int enqueue_small(pg_ctx *c, const Plan &p, int nchunk, int jchunk, double *acc,
     const long long ntiles = (p.ni + small_bi() - 1) / small_bi();
     if ((rc = ensure(c, c->part, (size_t)ntiles * (nchunk / small_cluster()) * 8 * small_bi() * sizeof(float))) ||
         (rc = ensure(c, c->tickets, (size_t)ntiles * sizeof(unsigned))) ||
-        (rc = ensure(c, c->g_jhl, (size_t)p.nj * 32)) || (rc = ensure(c, c->g_ihl, (size_t)p.ni * 32)))
+        (rc = ensure_jhl(c, (size_t)p.nj * 32)) || (rc = ensure(c, c->g_ihl, (size_t)p.ni * 32)))
         return rc;
     if (c->tickets_zeroed < c->tickets.cap) {
         PG_CUDA(c, cudaMemsetAsync(c->tickets.p, 0, c->tickets.cap, c->stream));
@@ -1518,7 +1535,7 @@ int enqueue_allpairs(pg_ctx *c, const Plan &p, double *acc, double *pot)
     a.ctr = (const double4 *)c->ctr.p;
     a.jrec = (const double4 *)c->jrec.p;
     if (!table && !p.df) {   // the single-form Newton kernel stages double-float j records
-        if ((rc = ensure(c, c->g_jhl, (size_t)std::max<long long>(p.nj, 1) * 32)) ||
+        if ((rc = ensure_jhl(c, (size_t)std::max<long long>(p.nj, 1) * 32)) ||
             (rc = pack_j_hilo(c, p.nj)))
             return rc;
         a.jhl = (const float4 *)c->g_jhl.p;
@@ -1793,8 +1810,6 @@ bool use_narrow(const pg_ctx *c)
     return c->ni > 0 && c->ni <= 4096 && nj_of(c) >= 64 * c->ni;
 }
 
-int pack_j_for(pg_ctx *c, long long nj);   // below
-
 int enqueue_narrow(pg_ctx *c, double *acc, double *pot)
 {
     int rc;
@@ -1841,13 +1856,14 @@ int enqueue_narrow(pg_ctx *c, double *acc, double *pot)
     const long long nitems = (long long)nic * nch;
     if ((rc = ensure(c, c->g_ctr, (size_t)nic * sizeof(double4))) || (rc = ensure(c, c->g_queue, 16)) ||
         (rc = ensure(c, c->n_part, (size_t)nch * ni * sizeof(double4))) ||
-        (rc = ensure(c, c->g_jhl, (size_t)nj * 32)) || (rc = ensure(c, c->g_ihl, (size_t)ni * 32)))
+        (rc = ensure_jhl(c, (size_t)nj * 32)) || (rc = ensure(c, c->g_ihl, (size_t)ni * 32)))
         return rc;
     // chunk centres, double-float i records and zeroed work counters in one launch
     PG_CUDA(c, launch_narrow_prep((const double4 *)c->xi.p, ni, Bi, nic, (double4 *)c->g_ctr.p,
                                   (float4 *)c->g_ihl.p, (int *)c->g_queue.p, c->stream));
     c->ihl_n = ni;
-    if ((rc = pack_j_for(c, nj))) return rc;
+    // (a stand-in's are packed by the kernel that it stands in for)
+    if (!c->skip && (rc = pack_j_hilo(c, nj))) return rc;
     c->last_launches += 1;
     GroupArgs g = group_args(c);
     g.skip = c->skip;
@@ -1890,17 +1906,6 @@ int enqueue_narrow(pg_ctx *c, double *acc, double *pot)
     return PG_OK;
 }
 
-// the double-float j records of a run that may stand in for another: packed
-// on every run where that one cannot run (so never counted as packed)
-int pack_j_for(pg_ctx *c, long long nj)
-{
-    if (!c->skip) return pack_j_hilo(c, nj);
-    if (c->jhl_n == nj && !c->capturing) return PG_OK;
-    PG_CUDA(c, launch_pack_hilo((const double4 *)c->jrec.p, nj, (float4 *)c->g_jhl.p, c->stream, c->skip));
-    c->last_launches += 1;
-    return PG_OK;
-}
-
 // The tensor-core path (pg_tc.cu): Newton runs of the default shape that
 // would difference in double-float, with enough pairs for its preparation and
 // the stand-in's empty launches. Whether this call's values fit its fixed
@@ -1922,15 +1927,37 @@ bool use_tc(const pg_ctx *c)
 // tc_dig holds the j digits and, behind them, the staged masses
 float *tc_mass(const pg_ctx *c, long long nj) { return (float *)((char *)c->tc_dig.p + tc_dig_bytes(nj)); }
 
+TcGeo *tc_geometry(const pg_ctx *c)
+{
+    // the box's words, one for the i flags, one for the verdict, the geometry
+    return (TcGeo *)((unsigned long long *)c->tc_geo.p + kTcBoxWords + 2);
+}
+
 int pack_tc(pg_ctx *c, long long nj)
 {
-    if (c->tc_n == nj) return PG_OK;
-    unsigned long long *words = (unsigned long long *)c->tc_geo.p;
-    PG_CUDA(c, launch_tc_pack((const double4 *)c->jrec.p, nj, words, (TcGeo *)(words + kTcBoxWords + 2),
+    if (c->tc_n == nj && c->tc_eps == c->eps) return PG_OK;
+    if (c->tc_box_n != nj) {
+        PG_CUDA(c, launch_tc_box((const double4 *)c->jrec.p, nj, (unsigned long long *)c->tc_geo.p, tc_geometry(c),
+                                 c->tc_seen, ++c->tc_gen, c->stream));
+        c->tc_box_n = nj;
+        c->last_launches += 1;
+    }
+    PG_CUDA(c, launch_tc_pack((const double4 *)c->jrec.p, nj, (float)(c->eps * c->eps), tc_geometry(c),
                               (unsigned char *)c->tc_dig.p, tc_mass(c, nj), c->stream));
-    c->last_launches += 2;
+    c->last_launches += 1;
     c->tc_n = nj;
+    c->tc_eps = c->eps;
     return PG_OK;
+}
+
+// The present j-set is known not to fit with the present eps: the geometry
+// has come back to the host from an earlier call. The double-float path then
+// runs alone, with the results it has behind the device's verdict.
+bool tc_known_unfit(const pg_ctx *c)
+{
+    return c->tc_seen && c->tc_box_n == nj_of(c) &&
+           __atomic_load_n(&c->tc_seen->gen, __ATOMIC_ACQUIRE) == c->tc_gen &&
+           !tc_fits(c->tc_seen->ok, c->tc_seen->e, c->tc_seen->mmin, (float)(c->eps * c->eps));
 }
 
 // the path's memory: the geometry and flags (zeroed once), the j digits and
@@ -1962,12 +1989,20 @@ int tc_room(pg_ctx *c)
     const size_t part = t.part + tc_dig_bytes(c->ni);
     // a capture allocates nothing: it records the path the run before it took
     if (c->capturing)
-        return c->tc_geo.cap && c->tc_dig.cap >= dig && c->part.cap >= part ? PG_OK : PG_ENOMEM;
+        return c->tc_geo.cap && c->tc_dig.cap >= dig && c->part.cap >= part && c->g_jhl.cap >= (size_t)nj_of(c) * 32
+                   ? PG_OK : PG_ENOMEM;
     if (c->tc_geo.cap == 0) {
         if ((rc = ensure(c, c->tc_geo, (kTcBoxWords + 2) * 8 + sizeof(TcGeo)))) return rc;
         PG_CUDA(c, cudaMemsetAsync(c->tc_geo.p, 0, c->tc_geo.cap, c->stream));
+        if (cudaHostAlloc((void **)&c->tc_seen, sizeof(TcSeen), cudaHostAllocMapped) != cudaSuccess) {
+            (void)cudaGetLastError();
+            c->tc_seen = nullptr;       // then every call asks the device
+        } else {
+            *c->tc_seen = TcSeen{};
+        }
     }
-    if ((rc = ensure(c, c->tc_dig, dig))) return rc;
+    if (dig > c->tc_dig.cap) tc_stale(c);
+    if ((rc = ensure(c, c->tc_dig, dig)) || (rc = ensure_jhl(c, (size_t)nj_of(c) * 32))) return rc;
     return ensure(c, c->part, part);
 }
 
@@ -1976,9 +2011,8 @@ int enqueue_tc(pg_ctx *c, double *acc, double *pot)
     int rc;
     const long long ni = c->ni, nj = nj_of(c);
     const TcShape t = tc_shape(c);
-    // the box's words, one for the i flags, one for the verdict, the geometry
     unsigned long long *words = (unsigned long long *)c->tc_geo.p;
-    TcGeo *geo = (TcGeo *)(words + kTcBoxWords + 2);
+    TcGeo *geo = tc_geometry(c);
     TcArgs a{};
     a.dig = (const unsigned char *)c->tc_dig.p;
     a.mass = tc_mass(c, nj);
@@ -1987,7 +2021,10 @@ int enqueue_tc(pg_ctx *c, double *acc, double *pot)
     a.geo = geo;
     int *ok = (int *)(words + kTcBoxWords + 1);
     a.ok = ok;
+    a.jrec = (const double4 *)c->jrec.p;
+    a.jhl = c->jhl_n == nj && !c->capturing ? nullptr : (float4 *)c->g_jhl.p;
     a.ni = ni;
+    a.nj = nj;
     a.W = t.W;
     a.njt = t.njt;
     a.slots = t.slots;
@@ -2128,7 +2165,7 @@ int tree_node_bufs(pg_ctx *c, TreeScratch &t, long long n)
         (rc = tbuf(c, pg_ctx::TB_BIG, (P == 3 ? k : 1) * 4, t.big_list)) ||
         (rc = tbuf(c, pg_ctx::TB_NBIG, 4, t.nbig)) ||
         (rc = tbuf(c, pg_ctx::TB_NODEW, k * sizeof(TreeNodeW), t.nodew)) ||
-        (rc = ensure(c, c->g_jhl, (size_t)(n + P * k) * 32)))
+        (rc = ensure_jhl(c, (size_t)(n + P * k) * 32)))
         return rc;
     return PG_OK;
 }
@@ -2278,6 +2315,7 @@ int tree_call(pg_ctx *c, double *acc, double *pot, bool exact, bool *redo, int &
     PG_CUDA(c, launch_pack_hilo(t.jrec2, nj_room, (float4 *)c->g_jhl.p, c->side_stream));
     PG_CUDA(c, cudaEventRecord(c->tree_ev[2], c->side_stream));
     c->jhl_n = -1;      // the buffer now holds the tree's records
+    tc_stale(c);
     PG_CUDA(c, tree_stage_groups(n, c->tree_ncrit, t, c->sort, c->stream));
     if (exact) {
         ++reads;
@@ -2425,7 +2463,7 @@ int enqueue_groups(pg_ctx *c, double *acc, double *pot)
                                 c->ngroups, 0, 0, (double4 *)c->g_ctr.p, c->stream));
     // double-float copies of the j records and i positions for the FP32 differencing
     long long nj = nj_of(c);
-    if ((rc = ensure(c, c->g_jhl, (size_t)std::max<long long>(nj, 1) * 32)) ||
+    if ((rc = ensure_jhl(c, (size_t)std::max<long long>(nj, 1) * 32)) ||
         (rc = ensure(c, c->g_ihl, (size_t)std::max<long long>(c->ni, 1) * 32)))
         return rc;
     if ((rc = pack_j_hilo(c, nj))) return rc;
@@ -2566,7 +2604,8 @@ int enqueue_run(pg_ctx *c, double *acc, double *pot)
         c->last_launches += launches;
         return PG_OK;
     }
-    if (use_tc(c)) {
+    // (a capture records the path that the run before it asked the device for)
+    if (use_tc(c) && (c->capturing || !tc_known_unfit(c))) {
         Plan p;
         plan_allpairs(c, p);
         int nchunk = 0, jchunk = 0;
@@ -2575,7 +2614,7 @@ int enqueue_run(pg_ctx *c, double *acc, double *pot)
             const int rc = tc_room(c);
             if (rc == PG_OK) return enqueue_tc(c, acc, pot);
             if (rc != PG_ENOMEM) return rc;
-            c->tc_n = -1;
+            tc_stale(c);
         }
     }
     if (use_narrow(c)) return enqueue_narrow(c, acc, pot);
@@ -2647,6 +2686,7 @@ int run_into(pg_ctx *c, double *acc, double *pot)
         c->jhl_n = nj_of(c);
     }
     if (c->graph_tc) {
+        if (tc_known_unfit(c)) return enqueue_run(c, acc, pot);
         if ((rc = pack_tc(c, nj_of(c)))) return rc;
     }
     PG_CUDA(c, cudaGraphLaunch(c->gexec, c->stream));

@@ -208,6 +208,19 @@ __device__ __forceinline__ double4 ldg_d4(const double4 *p)
     return r;
 }
 
+// record i as a double-float pair: (hi, w) then (lo, w), lo = x - hi, w the
+// record's fourth value (the mass of a j record; eps^2 of an i record with
+// per-i softening, else 0)
+__device__ __forceinline__ void pack_hilo_one(const double4 *__restrict__ in, long long i,
+                                              float4 *__restrict__ out)
+{
+    double4 v = in[i];
+    float hx = (float)v.x, hy = (float)v.y, hz = (float)v.z;
+    out[2 * i] = make_float4(hx, hy, hz, (float)v.w);
+    out[2 * i + 1] = make_float4((float)(v.x - (double)hx), (float)(v.y - (double)hy),
+                                 (float)(v.z - (double)hz), (float)v.w);
+}
+
 // a loss weight that is not finite in FP32 (or nearly so)
 __device__ __forceinline__ bool odd_weight(const double4 w)
 {

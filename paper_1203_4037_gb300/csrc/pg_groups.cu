@@ -1313,31 +1313,17 @@ cudaError_t launch_group_partials_combine(const CombineArgs &c, int nchunks, cud
     return cudaGetLastError();
 }
 
-// double-float records: (hi, w) then (lo, w) per particle, lo = x - hi, w
-// the record's fourth value (the mass of a j record; eps^2 of an i record
-// with per-i softening, else 0)
-__device__ __forceinline__ void pack_hilo_one(const double4 *__restrict__ in, long long i,
-                                              float4 *__restrict__ out)
-{
-    double4 v = in[i];
-    float hx = (float)v.x, hy = (float)v.y, hz = (float)v.z;
-    out[2 * i] = make_float4(hx, hy, hz, (float)v.w);
-    out[2 * i + 1] = make_float4((float)(v.x - (double)hx), (float)(v.y - (double)hy),
-                                 (float)(v.z - (double)hz), (float)v.w);
-}
-
-__global__ void k_pack_hilo(const double4 *__restrict__ in, long long n, float4 *__restrict__ out,
-                            const int *__restrict__ skip)
+__global__ void k_pack_hilo(const double4 *__restrict__ in, long long n, float4 *__restrict__ out)
 {
     long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (i >= n || (skip && *skip)) return;
+    if (i >= n) return;
     pack_hilo_one(in, i, out);
 }
 
-cudaError_t launch_pack_hilo(const double4 *in, long long n, float4 *out, cudaStream_t st, const int *skip)
+cudaError_t launch_pack_hilo(const double4 *in, long long n, float4 *out, cudaStream_t st)
 {
     if (n <= 0) return cudaSuccess;
-    k_pack_hilo<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(in, n, out, skip);
+    k_pack_hilo<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(in, n, out);
     return cudaGetLastError();
 }
 

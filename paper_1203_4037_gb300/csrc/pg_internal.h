@@ -4,6 +4,7 @@
 #pragma once
 
 #include <cstddef>
+#include <cmath>
 #include <cstdint>
 #include <string>
 #include <cuda_runtime.h>
@@ -274,15 +275,43 @@ struct TcGeo {             // set on the device from the j-set
     double mmin;           // smallest nonzero staged |mass| (0: none)
     int e, mexp;           // R = 2^e
     int ok;                // finite and in range
-    float e2;              // eps^2 in the kernel's unit (R 2^-23), set by each call's preparation
+    // set by each call's preparation
+    float e2;              // eps^2 in the kernel's unit (R 2^-23)
+    int packed;            // the digits are written (they are not while eps does not fit)
+    int stood_in;          // a call on this j-set went to the double-float path,
+    int hl;                // and one before the present: its j records are packed
 };
+// the geometry as the host sees it, some time after the call that set it
+// (page-locked memory)
+struct TcSeen {
+    long long gen;         // which call's; written last
+    double mmin;
+    int e, ok;
+};
+// Whether a j-set and eps fit the fixed point. eps from 2^-22 to 2^10 R:
+// below, one step of the positions (R 2^-47) is no longer small against
+// FP32's rounding of a pair at eps (with eps = 2^-30 R, i at 0.5 to 2 eps from
+// a j have force errors of 3.5e-6 median and 1.4e-5 at most; at 2^-22 R the
+// steps are 1/4 ulp of eps); above, the sums leave FP32's range. So do those
+// of masses too far below the largest: m / r^3 at the cube's diagonal is to
+// stay above 2^-110 (2^-75 of the largest mass at small eps). The same
+// operations, rounded alike, on the device and on the host.
+__host__ __device__ inline bool tc_fits(int ok, int e, double mmin, float eps2)
+{
+    if (!ok) return false;
+    const double e2 = ldexp((double)eps2, 2 * (23 - e));     // eps in units of R 2^-23
+    const double r2 = 3.0 * 0x1p48 + e2;
+    return e2 >= 0x1p2 && e2 <= 0x1p66 && (mmin == 0.0 || mmin * mmin >= r2 * r2 * (r2 * 0x1p-220));
+}
 struct TcArgs {
     const unsigned char *dig;   // j digits, tiles of 128 records
     const float *mass;          // staged masses, padded with zeros
     const unsigned char *idig;  // i digits, the same layout
     const TcGeo *geo;
-    const int *ok;         // zero: this call's values do not fit, nothing runs
-    long long ni, W;       // i-particles; units, i tiles times j tiles
+    const int *ok;         // zero: this call's values do not fit, nothing runs but
+    const double4 *jrec;   // the packing of these nj records as the double-float
+    float4 *jhl;           // path's pairs, if it is not done yet (nullptr: it is)
+    long long ni, nj, W;   // i-particles; j; units, i tiles times j tiles
     int njt, slots;        // j tiles; partial slots per i tile
     double4 *part;         // [i tiles][slots][tc_bi()]
     int *status;
@@ -293,8 +322,11 @@ int tc_jtiles(long long nj);
 int tc_slots(long long ntiles, int njt, long long W, int grid);
 // words: kTcBoxWords u64, zero before the first call and kept so
 constexpr int kTcBoxWords = 9;
-cudaError_t launch_tc_pack(const double4 *jrec, long long nj, unsigned long long *words, TcGeo *geo,
-                           unsigned char *dig, float *mass, cudaStream_t st);
+cudaError_t launch_tc_box(const double4 *jrec, long long nj, unsigned long long *words, TcGeo *geo, TcSeen *seen,
+                          long long gen, cudaStream_t st);
+// the digits, if the j-set fits with this eps and they are not written yet
+cudaError_t launch_tc_pack(const double4 *jrec, long long nj, float eps2, const TcGeo *geo, unsigned char *dig,
+                           float *mass, cudaStream_t st);
 // words: 2, zero before the first call and kept so; ok: the verdict
 cudaError_t launch_tc_prep(const double4 *xi, long long ni, float eps2, TcGeo *geo, unsigned char *idig,
                            unsigned *words, int *ok, cudaStream_t st);
@@ -381,9 +413,7 @@ cudaError_t launch_groups(const GroupArgs &g, int grid, int np, bool table, bool
 cudaError_t launch_groups_finish(const GroupArgs &g, cudaStream_t st);
 // one device-side bounded wait that nothing ends (the timeout path's self-test)
 cudaError_t launch_wait_selftest(int *status, unsigned long long limit_ns, cudaStream_t st);
-// skip: a nonzero word there leaves the records as they are
-cudaError_t launch_pack_hilo(const double4 *in, long long n, float4 *out, cudaStream_t st,
-                             const int *skip = nullptr);
+cudaError_t launch_pack_hilo(const double4 *in, long long n, float4 *out, cudaStream_t st);
 // narrow path: chunk centres (chunks of `chunk` i, nic of them), double-float
 // i records and the two work counters zeroed, in one launch
 cudaError_t launch_narrow_prep(const double4 *xi, long long ni, long long chunk, long long nic,

@@ -159,7 +159,13 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tc(const __grid_constant__ Tc
     const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
     const long long G = gridDim.x, b = blockIdx.x;
     const long long u0 = b * a.W / G, u1 = (b + 1) * a.W / G;
-    if (u0 >= u1 || *a.ok == 0) return;
+    if (*a.ok == 0) {
+        if (a.jhl && !a.geo->hl)
+#pragma unroll 4
+            for (long long k = b * kTcThreads + tid; k < a.nj; k += G * kTcThreads) pack_hilo_one(a.jrec, k, a.jhl);
+        return;
+    }
+    if (u0 >= u1) return;
     if (tid == 0) {
         *failed = 0;
         for (int k = 0; k < kSlots; ++k) {
@@ -434,9 +440,9 @@ __device__ __forceinline__ double unord64(u64 u)
 // finish sets the geometry and clears the words for the next call. words: 3
 // minima (stored inverted, so that zero starts them all), 3 maxima, largest
 // |m| (as bits, all ones with a non-finite value), smallest nonzero |m|
-// (inverted bits), ticket.
+// (inverted bits), ticket. seen (may be null): the host's copy.
 __global__ void __launch_bounds__(256) k_tc_box(const double4 *__restrict__ jrec, long long nj, u64 *words,
-                                                TcGeo *geo)
+                                                TcGeo *geo, TcSeen *seen, long long gen)
 {
     __shared__ u64 sh[8][8];
     u64 v[8] = {0, 0, 0, 0, 0, 0, 0, 0};
@@ -494,29 +500,35 @@ __global__ void __launch_bounds__(256) k_tc_box(const double4 *__restrict__ jrec
     }
     *geo = g;
     for (int q = 0; q < kTcBoxWords; ++q) words[q] = 0;
+    if (seen) {
+        seen->mmin = g.mmin;
+        seen->e = g.e;
+        seen->ok = g.ok;
+        __threadfence_system();
+        *(volatile long long *)&seen->gen = gen;
+    }
 }
 
 // the j records' digits and scaled masses, padded with massless records
-__global__ void k_tc_pack(const double4 *__restrict__ jrec, long long nj, long long npad, const TcGeo *__restrict__ geo,
-                          unsigned char *__restrict__ dig, float *__restrict__ mass)
+__global__ void __launch_bounds__(256) k_tc_pack(const double4 *__restrict__ jrec, long long nj, long long npad,
+                                                 float eps2, const TcGeo *__restrict__ geo,
+                                                 unsigned char *__restrict__ dig, float *__restrict__ mass)
 {
-    const long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (k >= npad) return;
+    __shared__ int go;
     const TcGeo g = *geo;
-    double4 v = make_double4(g.cx, g.cy, g.cz, 0.0);
-    if (k < nj && g.ok) v = jrec[k];
-    write_digits(v, g, dig, k);
-    mass[k] = (float)(v.w * g.mscale);
+    if (threadIdx.x == 0) go = !g.packed && tc_fits(g.ok, g.e, g.mmin, eps2);
+    __syncthreads();
+    if (!go) return;
+    for (long long k = blockIdx.x * 256ll + threadIdx.x; k < npad; k += gridDim.x * 256ll) {
+        double4 v = make_double4(g.cx, g.cy, g.cz, 0.0);
+        if (k < nj) v = jrec[k];
+        write_digits(v, g, dig, k);
+        mass[k] = (float)(v.w * g.mscale);
+    }
 }
 
-// The i-particles' digits, and whether this call can use them: every i within
-// the cube, and eps within 2^-22 to 2^10 R. Below, one step of the positions
-// (R 2^-47) is no longer small against FP32's rounding of a pair at eps (with
-// eps = 2^-30 R, i at 0.5 to 2 eps from a j have force errors of 3.5e-6 median
-// and 1.4e-5 at most; at 2^-22 R the steps are 1/4 ulp of eps); above, the
-// sums leave FP32's range. So do those of masses too far below the largest:
-// m / r^3 at the cube's diagonal is to stay above 2^-110 (2^-75 of the
-// largest mass at small eps). The last block writes the verdict.
+// The i-particles' digits, and whether this call can use them: the j-set and
+// eps fit and every i lies within the cube. The last block writes the verdict.
 __global__ void __launch_bounds__(256) k_tc_prep(const double4 *__restrict__ xi, long long ni, long long npad,
                                                  float eps2, TcGeo *geo, unsigned char *__restrict__ idig,
                                                  unsigned *words, int *ok)
@@ -539,13 +551,13 @@ __global__ void __launch_bounds__(256) k_tc_prep(const double4 *__restrict__ xi,
     __threadfence();
     if (atomicAdd(words + 1, 1u) != gridDim.x - 1) return;
     __threadfence();
-    const bool far = __ldcg(words) != 0;
+    const bool far = __ldcg(words) != 0, fits = tc_fits(g.ok, g.e, g.mmin, eps2);
     // eps in units of the upper digits' last place, u = R 2^-23
-    const double e2 = ldexp((double)eps2, 2 * (23 - g.e));
-    const double rmax = rsqrt(3.0 * 0x1p48 + e2);
-    const bool range = e2 >= 0x1p2 && e2 <= 0x1p66 && (g.mmin == 0.0 || g.mmin * (rmax * rmax * rmax) >= 0x1p-110);
-    geo->e2 = (float)(e2 * ((1.0 - kShort) * (1.0 - kShort)));
-    *ok = g.ok && !far && range;
+    geo->e2 = (float)(ldexp((double)eps2, 2 * (23 - g.e)) * ((1.0 - kShort) * (1.0 - kShort)));
+    geo->packed = g.packed || fits;
+    geo->hl = g.stood_in;
+    geo->stood_in = g.stood_in || far || !fits;
+    *ok = fits && !far;
     words[0] = words[1] = 0;
 }
 
@@ -593,13 +605,21 @@ int tc_slots(long long ntiles, int njt, long long W, int grid)
     return s;
 }
 
-cudaError_t launch_tc_pack(const double4 *jrec, long long nj, unsigned long long *words, TcGeo *geo,
-                           unsigned char *dig, float *mass, cudaStream_t st)
+cudaError_t launch_tc_box(const double4 *jrec, long long nj, unsigned long long *words, TcGeo *geo, TcSeen *seen,
+                          long long gen, cudaStream_t st)
 {
     if (nj <= 0) return cudaErrorInvalidValue;
-    k_tc_box<<<(unsigned)std::min<long long>((nj + 255) / 256, 608), 256, 0, st>>>(jrec, nj, words, geo);
+    k_tc_box<<<(unsigned)std::min<long long>((nj + 255) / 256, 608), 256, 0, st>>>(jrec, nj, words, geo, seen, gen);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_tc_pack(const double4 *jrec, long long nj, float eps2, const TcGeo *geo, unsigned char *dig,
+                           float *mass, cudaStream_t st)
+{
+    if (nj <= 0) return cudaErrorInvalidValue;
     const long long npad = (long long)tc_jtiles(nj) * kTcJ;
-    k_tc_pack<<<(unsigned)((npad + 255) / 256), 256, 0, st>>>(jrec, nj, npad, geo, dig, mass);
+    k_tc_pack<<<(unsigned)std::min<long long>((npad + 255) / 256, 1216), 256, 0, st>>>(jrec, nj, npad, eps2, geo, dig,
+                                                                                        mass);
     return cudaGetLastError();
 }
 

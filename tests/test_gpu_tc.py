@@ -199,3 +199,76 @@ def test_one_heavy_body(pg, orc, k, fits):
     ao, po = orc.newton(x[:300], x, m, 0.01, skip=np.arange(300, dtype=np.int64))
     assert_parity(rel_vec(a, ao), what="a")
     assert_parity(np.delete(rel_scalar(p, po), 5), what="phi")
+
+
+@pytest.mark.parametrize("graph", [False, True])
+def test_a_set_that_does_not_fit_is_remembered(pg, orc, graph):
+    # once the host has seen the j-set's geometry, the double-float path runs
+    # alone, until the j or eps change
+    xj, mj = gen.plummer(60000, 3)
+    far = xj.copy()
+    far[11] = [1e9, 0.0, 0.0]
+    xi = gen.plummer(300, 4)[0]
+
+    def call(c, path):
+        c.set_allpairs_path(path)
+        c.run()
+        a, p = c.get_force(300)
+        return a, p, c.info()["launches"]
+
+    with pg.Context(0) as c:
+        c.set_graph(graph)
+        c.set_eps(EPS)
+        c.set_i(xi)
+        c.set_j(far, mj)
+        first = call(c, pg.PG_PATH_AUTO)
+        later = [call(c, pg.PG_PATH_AUTO) for _ in range(3)][-1]
+        c.set_graph(False)
+        narrow = [call(c, pg.PG_PATH_NARROW) for _ in range(2)][-1]
+        assert later[2] == narrow[2]
+        for a, p, _ in (first, later):
+            assert np.array_equal(a, narrow[0]) and np.array_equal(p, narrow[1])
+        # a j-set that fits takes the tensor cores again, and so does an eps that fits
+        c.set_graph(graph)
+        c.set_j(xj, mj)
+        a, p, n = call(c, pg.PG_PATH_AUTO)
+        check(orc, a, p, xi, xj, mj, EPS)
+        assert not np.array_equal(a, run(pg, xi, xj, mj, EPS, path=pg.PG_PATH_NARROW)[0])
+        c.set_eps(1e-9)
+        assert np.array_equal(call(c, pg.PG_PATH_AUTO)[0], run(pg, xi, xj, mj, 1e-9, path=pg.PG_PATH_NARROW)[0])
+        c.set_eps(EPS)
+        assert np.array_equal(call(c, pg.PG_PATH_AUTO)[0], a)
+
+
+def test_stand_in_after_other_paths(pg, orc):
+    # the stand-in's packed records are its own until another path writes the
+    # buffer (a tree) or it grows
+    xj, mj = gen.plummer(80000, 3)
+    xi = gen.plummer(300, 4)[0]
+    xi[7] = [500.0, -3.0, 2.0]
+    with pg.Context(0) as c:
+        c.set_eps(EPS)
+        c.set_j(xj, mj)
+        c.set_n(60000)
+
+        def stand_in(n):
+            c.set_n(n)
+            c.set_i(xi)
+            out = []
+            for _ in range(2):
+                c.run()
+                out.append(c.get_force(300))
+            ref = run(pg, xi, xj[:n], mj[:n], EPS, path=pg.PG_PATH_NARROW)
+            for a, p in out:
+                assert np.array_equal(a, ref[0]) and np.array_equal(p, ref[1])
+
+        stand_in(60000)
+        c.set_i(xj[:60000])
+        c.set_self(True)
+        c.set_tree(0.75, 256, 8)
+        c.run()
+        c.set_tree(-1.0, 256, 8)
+        c.set_self(False)
+        stand_in(60000)
+        stand_in(80000)
+        stand_in(60000)
