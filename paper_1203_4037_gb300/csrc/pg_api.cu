@@ -161,6 +161,7 @@ struct pg_ctx {
     DevBuf tc_dig, tc_geo;
     long long tc_n = -1, tc_box_n = -1, tc_gen = 0;
     double tc_eps = -1.0;
+    bool tc_hot = false;          // the last run was one for the tensor cores
     TcSeen *tc_seen = nullptr;    // page-locked
     bool graph_tc = false;        // the captured run reads the j digits
     const int *skip = nullptr;    // set while the run's stand-in is enqueued: it runs where this word is zero
@@ -255,6 +256,12 @@ int ensure(pg_ctx *c, DevBuf &b, size_t bytes)
 // the j records of the tensor-core path, or the double-float records that its
 // stand-in packed, are no longer what its geometry says
 void tc_stale(pg_ctx *c) { c->tc_n = c->tc_box_n = -1; }
+
+TcGeo *tc_geometry(const pg_ctx *c)
+{
+    // the box's words, one for the i flags, one for the verdict, the geometry
+    return (TcGeo *)((unsigned long long *)c->tc_geo.p + kTcBoxWords + 2);
+}
 
 // g_jhl grown: what it held is gone
 int ensure_jhl(pg_ctx *c, size_t bytes)
@@ -952,6 +959,23 @@ static int grow_j(pg_ctx *c, long long end)
     return PG_OK;
 }
 
+// j records adr .. adr + nj - 1 from device arrays. A whole j-set for a context
+// whose last run was one for the tensor cores: with their cube, in one pass.
+static int pack_j(pg_ctx *c, long long adr, long long nj, const double *x, const double *m)
+{
+    c->nj_hw = std::max(c->nj_hw, adr + nj);
+    c->jhl_n = -1;
+    tc_stale(c);
+    if (c->tc_hot && c->tc_geo.cap && adr == 0 && nj == nj_of(c)) {
+        PG_CUDA(c, launch_tc_pack_box(x, m, (double4 *)c->jrec.p, nj, (unsigned long long *)c->tc_geo.p, tc_geometry(c),
+                                      c->tc_seen, ++c->tc_gen, c->stream));
+        c->tc_box_n = nj;
+        return PG_OK;
+    }
+    PG_CUDA(c, launch_pack_j(x, m, (double4 *)c->jrec.p + adr, nj, c->stream));
+    return PG_OK;
+}
+
 int pg_set_j(pg_ctx *c, long long adr, long long nj, const double *x, const double *m)
 {
     if (!c) return PG_EINVAL;
@@ -975,11 +999,7 @@ int pg_set_j(pg_ctx *c, long long adr, long long nj, const double *x, const doub
         PG_CUDA(c, cudaEventRecord(c->pin_j.done, c->stream));
     }
     const double *dx = (const double *)c->stage.p;
-    PG_CUDA(c, launch_pack_j(dx, dx + 3 * nj, (double4 *)c->jrec.p + adr, nj, c->stream));
-    c->nj_hw = std::max(c->nj_hw, adr + nj);
-    c->jhl_n = -1;
-    tc_stale(c);
-    return PG_OK;
+    return pack_j(c, adr, nj, dx, dx + 3 * nj);
 }
 
 int pg_set_j_rec_dev(pg_ctx *c, long long adr, long long nj, const double *rec)
@@ -1006,11 +1026,7 @@ int pg_set_j_dev(pg_ctx *c, long long adr, long long nj, const double *x, const 
     if (nj == 0) return PG_OK;
     int rc;
     if ((rc = grow_j(c, adr + nj))) return rc;
-    PG_CUDA(c, launch_pack_j(x, m, (double4 *)c->jrec.p + adr, nj, c->stream));
-    c->nj_hw = std::max(c->nj_hw, adr + nj);
-    c->jhl_n = -1;
-    tc_stale(c);
-    return PG_OK;
+    return pack_j(c, adr, nj, x, m);
 }
 
 // the i records and their double-float pairs (written together by set_i)
@@ -1716,7 +1732,7 @@ GroupArgs group_args(pg_ctx *c)
 // df: double-float differencing (the narrow path's items); tj, nt: the
 // kernel's j-tile depth and threads per CTA (the caller's plain lists only)
 int launch_group_kernel(pg_ctx *c, const GroupArgs &g, bool cell, bool df = false, int tj = kGroupsTJ,
-                        int nt = kGroupsNT)
+                        int nt = kGroupsNT, bool queue_zeroed = false)
 {
     bool table = c->mode == PG_TABLE;
     int np = groups_np(c);
@@ -1740,7 +1756,7 @@ int launch_group_kernel(pg_ctx *c, const GroupArgs &g, bool cell, bool df = fals
     int grid = c->sms * per;
     GroupArgs gg = g;
     if (wper > 0) gg.queue_w = (int *)c->g_queue.p + 1;
-    PG_CUDA(c, cudaMemsetAsync(c->g_queue.p, 0, 2 * sizeof(int), c->stream));
+    if (!queue_zeroed) PG_CUDA(c, cudaMemsetAsync(c->g_queue.p, 0, 2 * sizeof(int), c->stream));
     if (c->timing) PG_CUDA(c, record_timing(c, c->tk0));
     PG_CUDA(c, launch_groups(gg, grid, np, table, cell, ext, df, tj, nt,
                              groups_smem(np, table, tab_units(c), df, tj, nt), c->stream));
@@ -1810,7 +1826,19 @@ bool use_narrow(const pg_ctx *c)
     return c->ni > 0 && c->ni <= 4096 && nj_of(c) >= 64 * c->ni;
 }
 
-int enqueue_narrow(pg_ctx *c, double *acc, double *pot)
+// a tensor-core run (below): its arguments and launches
+struct TcRun {
+    TcArgs a;
+    int grid;
+    unsigned char *idig;
+    unsigned *words;       // the i flags
+    int *ok;               // the verdict
+    bool timing;
+};
+int enqueue_tc_kernels(pg_ctx *c, const TcRun &r, const NarrowPrep &np);
+
+// tc: the run stands in for a tensor-core run, whose launches go with it
+int enqueue_narrow(pg_ctx *c, double *acc, double *pot, const TcRun *tc = nullptr)
 {
     int rc;
     const long long ni = c->ni, nj = nj_of(c);
@@ -1858,15 +1886,23 @@ int enqueue_narrow(pg_ctx *c, double *acc, double *pot)
         (rc = ensure(c, c->n_part, (size_t)nch * ni * sizeof(double4))) ||
         (rc = ensure_jhl(c, (size_t)nj * 32)) || (rc = ensure(c, c->g_ihl, (size_t)ni * 32)))
         return rc;
-    // chunk centres, double-float i records and zeroed work counters in one launch
-    PG_CUDA(c, launch_narrow_prep((const double4 *)c->xi.p, ni, Bi, nic, (double4 *)c->g_ctr.p,
-                                  (float4 *)c->g_ihl.p, (int *)c->g_queue.p, c->stream));
+    NarrowPrep prep;
+    prep.chunk = Bi;
+    prep.nic = nic;
+    prep.ctr = (double4 *)c->g_ctr.p;
+    prep.ihl = (float4 *)c->g_ihl.p;
+    prep.queue = (int *)c->g_queue.p;
     c->ihl_n = ni;
-    // (a stand-in's are packed by the kernel that it stands in for)
-    if (!c->skip && (rc = pack_j_hilo(c, nj))) return rc;
-    c->last_launches += 1;
+    if (tc) {
+        // (that kernel packs the stand-in's j records)
+        if ((rc = enqueue_tc_kernels(c, *tc, prep))) return rc;
+    } else {
+        PG_CUDA(c, launch_narrow_prep((const double4 *)c->xi.p, ni, prep, c->stream));
+        c->last_launches += 1;
+        if ((rc = pack_j_hilo(c, nj))) return rc;
+    }
     GroupArgs g = group_args(c);
-    g.skip = c->skip;
+    g.skip = tc ? tc->ok : nullptr;
     g.xi = (const double4 *)c->xi.p;
     g.jrec = (const double4 *)c->jrec.p;
     g.j_off = nullptr;
@@ -1887,7 +1923,8 @@ int enqueue_narrow(pg_ctx *c, double *acc, double *pot)
     g.part_stride = ni;
     g.acc = acc;
     g.pot = pot;
-    if ((rc = warp ? launch_group_warp_kernel(c, g, wper, df) : launch_group_kernel(c, g, false, df))) return rc;
+    if ((rc = warp ? launch_group_warp_kernel(c, g, wper, df)
+                   : launch_group_kernel(c, g, false, df, kGroupsTJ, kGroupsNT, true))) return rc;
     CombineArgs cb{};
     cb.part = (const double4 *)c->n_part.p;
     cb.jrec = (const double4 *)c->jrec.p;
@@ -1899,8 +1936,7 @@ int enqueue_narrow(pg_ctx *c, double *acc, double *pot)
     cb.accscale = g.accscale;
     cb.acc = acc;
     cb.pot = pot;
-    cb.skip = c->skip;
-    PG_CUDA(c, launch_group_partials_combine(cb, (int)nch, c->stream));
+    PG_CUDA(c, launch_group_partials_combine(cb, (int)nch, c->stream, tc ? &tc->a : nullptr, tc ? tc->grid : 0));
     c->last_launches += 1;
     c->last_slots = nch;
     return PG_OK;
@@ -1910,10 +1946,12 @@ int enqueue_narrow(pg_ctx *c, double *acc, double *pot)
 // would difference in double-float, with enough pairs for its preparation and
 // the stand-in's empty launches. Whether this call's values fit its fixed
 // point (every i within the j-set's cube, eps within 2^-22 to 2^10 of its half
-// side, no mass too far below the largest) is known on the device only: the double-float path is enqueued behind it
-// and runs where they do not. From 48 i on: fewer leave most of a
-// 64-particle tile empty (2^20 j, kernel: 16 i 25 us, as the warp-mode
-// kernel's 25; 64 i 41 against 72; 1000 i 460 against 840).
+// side, no mass too far below the largest) is known on the device: the
+// double-float path is enqueued behind it and runs where they do not. From 48
+// i on: fewer leave most of a 64-particle tile empty. From 2^24 pairs on also
+// with new j records in every call, the dearest (64 i on 2^18 j, a call: 57
+// us, 62 on the narrow path; 29 and 41 with the j kept; 1000 i on 2^20 j 546
+// and 892, 499 and 850).
 bool use_tc(const pg_ctx *c)
 {
     if (c->mode != PG_NEWTON || use_ext(c) || c->np || c->split || c->ctas_per_sm || c->path != PG_PATH_AUTO ||
@@ -1926,12 +1964,6 @@ bool use_tc(const pg_ctx *c)
 
 // tc_dig holds the j digits and, behind them, the staged masses
 float *tc_mass(const pg_ctx *c, long long nj) { return (float *)((char *)c->tc_dig.p + tc_dig_bytes(nj)); }
-
-TcGeo *tc_geometry(const pg_ctx *c)
-{
-    // the box's words, one for the i flags, one for the verdict, the geometry
-    return (TcGeo *)((unsigned long long *)c->tc_geo.p + kTcBoxWords + 2);
-}
 
 int pack_tc(pg_ctx *c, long long nj)
 {
@@ -1971,7 +2003,7 @@ struct TcShape {
 TcShape tc_shape(const pg_ctx *c)
 {
     TcShape t;
-    t.Bi = tc_bi();
+    t.Bi = kTcBi;
     t.njt = tc_jtiles(nj_of(c));
     t.ntiles = (c->ni + t.Bi - 1) / t.Bi;
     t.W = t.ntiles * t.njt;
@@ -2006,21 +2038,34 @@ int tc_room(pg_ctx *c)
     return ensure(c, c->part, part);
 }
 
+int enqueue_tc_kernels(pg_ctx *c, const TcRun &r, const NarrowPrep &np)
+{
+    PG_CUDA(c, launch_tc_prep((const double4 *)c->xi.p, r.a.ni, (float)(c->eps * c->eps), tc_geometry(c), r.idig,
+                              r.words, r.ok, np, c->stream));
+    if (r.timing) PG_CUDA(c, record_timing(c, c->tk0));
+    PG_CUDA(c, launch_tc(r.a, r.grid, c->stream));
+    c->last_launches += 2;
+    return PG_OK;
+}
+
 int enqueue_tc(pg_ctx *c, double *acc, double *pot)
 {
     int rc;
     const long long ni = c->ni, nj = nj_of(c);
     const TcShape t = tc_shape(c);
     unsigned long long *words = (unsigned long long *)c->tc_geo.p;
-    TcGeo *geo = tc_geometry(c);
-    TcArgs a{};
+    TcRun r{};
+    r.grid = t.grid;
+    r.idig = (unsigned char *)c->part.p + t.part;
+    r.words = (unsigned *)(words + kTcBoxWords);
+    r.ok = (int *)(words + kTcBoxWords + 1);
+    r.timing = c->timing;
+    TcArgs &a = r.a;
     a.dig = (const unsigned char *)c->tc_dig.p;
     a.mass = tc_mass(c, nj);
-    unsigned char *idig = (unsigned char *)c->part.p + t.part;
-    a.idig = idig;
-    a.geo = geo;
-    int *ok = (int *)(words + kTcBoxWords + 1);
-    a.ok = ok;
+    a.idig = r.idig;
+    a.geo = tc_geometry(c);
+    a.ok = r.ok;
     a.jrec = (const double4 *)c->jrec.p;
     a.jhl = c->jhl_n == nj && !c->capturing ? nullptr : (float4 *)c->g_jhl.p;
     a.ni = ni;
@@ -2032,28 +2077,23 @@ int enqueue_tc(pg_ctx *c, double *acc, double *pot)
     a.status = (int *)c->status.p;
     if (c->capturing) c->graph_tc = true;
     else if ((rc = pack_tc(c, nj))) return rc;
-    PG_CUDA(c, launch_tc_prep((const double4 *)c->xi.p, ni, (float)(c->eps * c->eps), geo, idig,
-                              (unsigned *)(words + kTcBoxWords), ok, c->stream));
-    if (c->timing) PG_CUDA(c, record_timing(c, c->tk0));
-    PG_CUDA(c, launch_tc(a, t.grid, c->stream));
-    const bool timing = c->timing;
-    PG_CUDA(c, launch_tc_combine(a, t.grid, c->self, c->self_off, acc, pot, c->stream));
-    c->last_launches += 3;
     // where the values do not fit: the double-float path
-    c->skip = ok;
     c->timing = false;
     if (use_narrow(c)) {
-        rc = enqueue_narrow(c, acc, pot);
-    } else {
+        rc = enqueue_narrow(c, acc, pot, &r);
+    } else if (!(rc = enqueue_tc_kernels(c, r, NarrowPrep()))) {
+        const cudaError_t e = launch_tc_combine(a, t.grid, c->self, c->self_off, acc, pot, c->stream);
+        c->last_launches += 1;
         Plan p;
         plan_allpairs(c, p);
-        rc = enqueue_allpairs(c, p, acc, pot);
+        c->skip = r.ok;
+        rc = e == cudaSuccess ? enqueue_allpairs(c, p, acc, pot) : cuda_fail(c, e, "launch_tc_combine");
+        c->skip = nullptr;
     }
-    c->skip = nullptr;
-    c->timing = timing;
+    c->timing = r.timing;
     if (rc) return rc;
-    if (timing) PG_CUDA(c, record_timing(c, c->tk1));
-    c->timed = timing;
+    if (c->timing) PG_CUDA(c, record_timing(c, c->tk1));
+    c->timed = c->timing;
     c->last_np = t.Bi / 2;
     c->last_df = true;
     c->last_split = 1;
@@ -2573,6 +2613,7 @@ int enqueue_run(pg_ctx *c, double *acc, double *pot)
     c->last_launches = 0;
     c->last_split = 0;
     c->last_tj = c->last_nt = 0;
+    c->tc_hot = false;
     // per-i softening lives in the i records' w (read by every path); a
     // captured graph writes it on every replay, as the records may be new
     if (c->have_epsi && (c->capturing || !c->epsi_applied)) {
@@ -2605,11 +2646,16 @@ int enqueue_run(pg_ctx *c, double *acc, double *pot)
         return PG_OK;
     }
     // (a capture records the path that the run before it asked the device for)
-    if (use_tc(c) && (c->capturing || !tc_known_unfit(c))) {
-        Plan p;
-        plan_allpairs(c, p);
-        int nchunk = 0, jchunk = 0;
-        if (use_narrow(c) || !use_small(c, p, nchunk, jchunk)) {
+    c->tc_hot = use_tc(c);
+    if (c->tc_hot && (c->capturing || !tc_known_unfit(c))) {
+        bool take = use_narrow(c);
+        if (!take) {
+            Plan p;
+            plan_allpairs(c, p);
+            int nchunk = 0, jchunk = 0;
+            take = !use_small(c, p, nchunk, jchunk);
+        }
+        if (take) {
             // without room for the digits the double-float path runs alone
             const int rc = tc_room(c);
             if (rc == PG_OK) return enqueue_tc(c, acc, pot);

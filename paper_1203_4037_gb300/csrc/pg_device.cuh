@@ -221,6 +221,100 @@ __device__ __forceinline__ void pack_hilo_one(const double4 *__restrict__ in, lo
                                  (float)(v.z - (double)hz), (float)v.w);
 }
 
+// ---------------------------------------------------------------- narrow path
+// FP64 centre of each group: midpoint of its i-particles' bounding box
+// group g holds i_off[g] .. i_off[g + 1], or without offsets the chunk
+// g chunk .. min((g + 1) chunk, ni)
+__device__ __forceinline__ void group_ctr_warp(const double4 *__restrict__ xi,
+                                               const long long *__restrict__ i_off, long long g,
+                                               long long chunk, long long ni, int lane,
+                                               double4 *__restrict__ ctr)
+{
+    const long long ib = i_off ? i_off[g] : g * chunk;
+    const long long ie = i_off ? i_off[g + 1] : min((g + 1) * chunk, ni);
+    double lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
+    for (long long i = ib + lane; i < ie; i += 32) {
+        double4 v = xi[i];
+        lo[0] = fmin(lo[0], v.x); lo[1] = fmin(lo[1], v.y); lo[2] = fmin(lo[2], v.z);
+        hi[0] = fmax(hi[0], v.x); hi[1] = fmax(hi[1], v.y); hi[2] = fmax(hi[2], v.z);
+    }
+    for (int c = 0; c < 3; ++c)
+        for (int o = 16; o; o >>= 1) {
+            lo[c] = fmin(lo[c], __shfl_xor_sync(0xffffffffu, lo[c], o));
+            hi[c] = fmax(hi[c], __shfl_xor_sync(0xffffffffu, hi[c], o));
+        }
+    if (lane == 0) {
+        bool empty = !(lo[0] <= hi[0]);
+        ctr[g] = empty ? make_double4(0, 0, 0, 0)
+                       : make_double4(0.5 * (lo[0] + hi[0]), 0.5 * (lo[1] + hi[1]),
+                                      0.5 * (lo[2] + hi[2]), 0.0);
+    }
+}
+
+// The narrow path's preparation, block blk of narrow_prep_blocks: one warp a
+// chunk centre in the first of them, then one thread an i record
+constexpr int kNarrowPrepThreads = 128;
+__host__ __device__ __forceinline__ long long narrow_prep_blocks(long long ni, const NarrowPrep &np)
+{
+    return (np.nic + kNarrowPrepThreads / 32 - 1) / (kNarrowPrepThreads / 32) +
+           (ni + kNarrowPrepThreads - 1) / kNarrowPrepThreads;
+}
+__device__ __forceinline__ void narrow_prep_block(const double4 *__restrict__ xi, long long ni, const NarrowPrep &np,
+                                                  long long blk)
+{
+    constexpr int kWarps = kNarrowPrepThreads / 32;
+    const long long cb = (np.nic + kWarps - 1) / kWarps;
+    if (blk == 0 && threadIdx.x < 2) np.queue[threadIdx.x] = 0;
+    if (blk < cb) {
+        const long long g = blk * kWarps + (threadIdx.x >> 5);
+        if (g < np.nic) group_ctr_warp(xi, nullptr, g, np.chunk, ni, threadIdx.x & 31, np.ctr);
+        return;
+    }
+    const long long i = (blk - cb) * kNarrowPrepThreads + threadIdx.x;
+    if (i < ni) pack_hilo_one(xi, i, np.ihl);
+}
+
+// ---------------------------------------------------------------- tensor cores
+// The differences come out short by this on average (the tensor cores round
+// them toward zero), so the unit they are read in is longer by it. From the
+// signed errors of forces (2 kTcShort) and potentials (kTcShort) against 64
+// bits, 12 sets of 112 to 2080 i against 3e5 to 1e6 j: +4.7e-8 and +2.6e-8
+// without it
+constexpr double kTcShort = 2.5e-8;
+
+__host__ __device__ __forceinline__ long long tc_owner(long long u, long long grid, long long W)
+{
+    return ((u + 1) * grid - 1) / W;
+}
+
+// i-particle i of a tensor-core run, by one warp: the partial sums of its tile
+// over the CTAs, the own pair's potential, the units
+__device__ __forceinline__ void tc_combine_one(const TcArgs &a, int grid, int self, long long self_off,
+                                               double *__restrict__ acc, double *__restrict__ pot, long long i)
+{
+    const int lane = threadIdx.x & 31;
+    const long long t = i / kTcBi, li = i % kTcBi;
+    const long long bf = tc_owner(t * a.njt, grid, a.W), bl = tc_owner((t + 1) * a.njt - 1, grid, a.W);
+    double s[4] = {0, 0, 0, 0};
+    for (long long k = lane; k <= bl - bf; k += 32) {
+        const double4 v = a.part[((size_t)t * a.slots + k) * kTcBi + li];
+        s[0] += v.x; s[1] += v.y; s[2] += v.z; s[3] += v.w;
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+        for (int o = 16; o; o >>= 1) s[q] += __shfl_xor_sync(0xffffffffu, s[q], o);
+    if (lane != 0) return;
+    const TcGeo &g = *a.geo;
+    // the own pair as the loop added it: d = 0 exactly
+    if (self) s[3] += (double)__fmul_rn(a.mass[i + self_off], rsq(g.e2));
+    const double fa = ldexp((1.0 - kTcShort) * (1.0 - kTcShort), 2 * (23 - g.e) - g.mexp),
+                 fp = ldexp(1.0 - kTcShort, 23 - g.e - g.mexp);
+    acc[3 * i] = s[0] * fa;
+    acc[3 * i + 1] = s[1] * fa;
+    acc[3 * i + 2] = s[2] * fa;
+    if (pot) pot[i] = s[3] * fp;
+}
+
 // a loss weight that is not finite in FP32 (or nearly so)
 __device__ __forceinline__ bool odd_weight(const double4 w)
 {

@@ -1273,10 +1273,14 @@ cudaError_t launch_groups_finish(const GroupArgs &g, cudaStream_t st)
 // thread).
 constexpr int kCombineThreads = 128;
 
+template <bool TC>
 __global__ void __launch_bounds__(kCombineThreads)
-k_group_partials_combine(CombineArgs c, int nchunks)
+k_group_partials_combine(CombineArgs c, int nchunks, TcArgs tc, int tc_grid)
 {
-    if (c.skip && *c.skip) return;
+    if (TC && *tc.ok) {
+        if (threadIdx.x < 32) tc_combine_one(tc, tc_grid, c.self, c.self_off, c.acc, c.pot, blockIdx.x);
+        return;
+    }
     __shared__ double4 wsum[kCombineThreads / 32];
     const long long i = blockIdx.x;
     const int t = threadIdx.x, lane = t & 31;
@@ -1306,10 +1310,12 @@ k_group_partials_combine(CombineArgs c, int nchunks)
     if (c.pot) c.pot[i] = c.newton || c.tabpot ? ph : 0.0;
 }
 
-cudaError_t launch_group_partials_combine(const CombineArgs &c, int nchunks, cudaStream_t st)
+cudaError_t launch_group_partials_combine(const CombineArgs &c, int nchunks, cudaStream_t st, const TcArgs *tc,
+                                          int tc_grid)
 {
     if (c.ni <= 0) return cudaSuccess;
-    k_group_partials_combine<<<(unsigned)c.ni, kCombineThreads, 0, st>>>(c, nchunks);
+    if (tc) k_group_partials_combine<true><<<(unsigned)c.ni, kCombineThreads, 0, st>>>(c, nchunks, *tc, tc_grid);
+    else k_group_partials_combine<false><<<(unsigned)c.ni, kCombineThreads, 0, st>>>(c, nchunks, TcArgs{}, 0);
     return cudaGetLastError();
 }
 
@@ -1328,35 +1334,6 @@ cudaError_t launch_pack_hilo(const double4 *in, long long n, float4 *out, cudaSt
 }
 
 // ------------------------------------------------------------------ prep
-// FP64 centre of each group: midpoint of its i-particles' bounding box
-// group g holds i_off[g] .. i_off[g + 1], or without offsets the chunk
-// g chunk .. min((g + 1) chunk, ni)
-__device__ __forceinline__ void group_ctr_warp(const double4 *__restrict__ xi,
-                                               const long long *__restrict__ i_off, long long g,
-                                               long long chunk, long long ni, int lane,
-                                               double4 *__restrict__ ctr)
-{
-    const long long ib = i_off ? i_off[g] : g * chunk;
-    const long long ie = i_off ? i_off[g + 1] : min((g + 1) * chunk, ni);
-    double lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
-    for (long long i = ib + lane; i < ie; i += 32) {
-        double4 v = xi[i];
-        lo[0] = fmin(lo[0], v.x); lo[1] = fmin(lo[1], v.y); lo[2] = fmin(lo[2], v.z);
-        hi[0] = fmax(hi[0], v.x); hi[1] = fmax(hi[1], v.y); hi[2] = fmax(hi[2], v.z);
-    }
-    for (int c = 0; c < 3; ++c)
-        for (int o = 16; o; o >>= 1) {
-            lo[c] = fmin(lo[c], __shfl_xor_sync(0xffffffffu, lo[c], o));
-            hi[c] = fmax(hi[c], __shfl_xor_sync(0xffffffffu, hi[c], o));
-        }
-    if (lane == 0) {
-        bool empty = !(lo[0] <= hi[0]);
-        ctr[g] = empty ? make_double4(0, 0, 0, 0)
-                       : make_double4(0.5 * (lo[0] + hi[0]), 0.5 * (lo[1] + hi[1]),
-                                      0.5 * (lo[2] + hi[2]), 0.0);
-    }
-}
-
 __global__ void k_group_ctr(const double4 *__restrict__ xi, const long long *__restrict__ i_off,
                             long long ngroups, const long long *__restrict__ ngroups_dev, long long chunk,
                             long long ni, double4 *__restrict__ ctr)
@@ -1366,31 +1343,16 @@ __global__ void k_group_ctr(const double4 *__restrict__ xi, const long long *__r
     group_ctr_warp(xi, i_off, g, chunk, ni, threadIdx.x & 31, ctr);
 }
 
-// The narrow path's preparation in one launch: the FP64 centre of each of
-// the nic i chunks (one warp each, blocks [0, cb)), the double-float i
-// records (blocks cb onwards, one thread each), and the two work counters
-// set to zero.
-__global__ void k_narrow_prep(const double4 *__restrict__ xi, long long ni, long long chunk, long long nic,
-                              long long cb, double4 *__restrict__ ctr, float4 *__restrict__ ihl,
-                              int *__restrict__ queue)
+__global__ void __launch_bounds__(kNarrowPrepThreads) k_narrow_prep(const double4 *__restrict__ xi, long long ni,
+                                                                    NarrowPrep np)
 {
-    if (blockIdx.x == 0 && threadIdx.x < 2) queue[threadIdx.x] = 0;
-    if (blockIdx.x < cb) {
-        const long long g = blockIdx.x * (long long)(blockDim.x >> 5) + (threadIdx.x >> 5);
-        if (g < nic) group_ctr_warp(xi, nullptr, g, chunk, ni, threadIdx.x & 31, ctr);
-        return;
-    }
-    const long long i = (blockIdx.x - cb) * (long long)blockDim.x + threadIdx.x;
-    if (i < ni) pack_hilo_one(xi, i, ihl);
+    narrow_prep_block(xi, ni, np, blockIdx.x);
 }
 
-cudaError_t launch_narrow_prep(const double4 *xi, long long ni, long long chunk, long long nic,
-                              double4 *ctr, float4 *ihl, int *queue, cudaStream_t st)
+cudaError_t launch_narrow_prep(const double4 *xi, long long ni, const NarrowPrep &np, cudaStream_t st)
 {
-    if (ni <= 0 || nic <= 0) return cudaErrorInvalidValue;
-    const long long cb = (nic + 3) / 4;                  // 4 warps of 128 threads
-    const long long pb = (ni + 127) / 128;
-    k_narrow_prep<<<(unsigned)(cb + pb), 128, 0, st>>>(xi, ni, chunk, nic, cb, ctr, ihl, queue);
+    if (ni <= 0 || np.nic <= 0) return cudaErrorInvalidValue;
+    k_narrow_prep<<<(unsigned)narrow_prep_blocks(ni, np), kNarrowPrepThreads, 0, st>>>(xi, ni, np);
     return cudaGetLastError();
 }
 

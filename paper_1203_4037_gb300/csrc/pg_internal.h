@@ -266,10 +266,20 @@ int pm_solve(PmState *s, const float *rho, const double4 *tgt, long long nt, dou
 // half extents of each tile's box (infinite with a non-finite particle)
 cudaError_t launch_tile_prep(const double4 *xi, const unsigned *perm, long long n, int Bi,
                              double4 *xi_tiled, double4 *ctr, cudaStream_t st, double4 *ext = nullptr);
+// The narrow path's preparation: the centres of nic chunks of `chunk` i each,
+// the double-float i records, two work counters zeroed
+struct NarrowPrep {
+    long long chunk = 0, nic = 0;
+    double4 *ctr = nullptr;
+    float4 *ihl = nullptr;
+    int *queue = nullptr;
+};
+
 // ---------------------------------------------------------------- tensor cores
 // Newton all pairs with the differences formed by tcgen05.mma (pg_tc.cu)
 struct TcGeo {             // set on the device from the j-set
     double cx, cy, cz;     // the cube's centre
+    double sx, sy, sz;     // and that times scale
     double scale;          // position -> fixed point, 2^47 / R
     double mscale;         // mass -> staged mass, 2^mexp
     double mmin;           // smallest nonzero staged |mass| (0: none)
@@ -313,10 +323,10 @@ struct TcArgs {
     float4 *jhl;           // path's pairs, if it is not done yet (nullptr: it is)
     long long ni, nj, W;   // i-particles; j; units, i tiles times j tiles
     int njt, slots;        // j tiles; partial slots per i tile
-    double4 *part;         // [i tiles][slots][tc_bi()]
+    double4 *part;         // [i tiles][slots][kTcBi]
     int *status;
 };
-int tc_bi();                               // i-particles per tile
+constexpr int kTcBi = 64;                  // i-particles per tile
 size_t tc_dig_bytes(long long n);
 int tc_jtiles(long long nj);
 int tc_slots(long long ntiles, int njt, long long W, int grid);
@@ -324,12 +334,16 @@ int tc_slots(long long ntiles, int njt, long long W, int grid);
 constexpr int kTcBoxWords = 9;
 cudaError_t launch_tc_box(const double4 *jrec, long long nj, unsigned long long *words, TcGeo *geo, TcSeen *seen,
                           long long gen, cudaStream_t st);
+// the same and launch_pack_j of the whole j-set in one pass
+cudaError_t launch_tc_pack_box(const double *x, const double *m, double4 *jrec, long long nj, unsigned long long *words,
+                               TcGeo *geo, TcSeen *seen, long long gen, cudaStream_t st);
 // the digits, if the j-set fits with this eps and they are not written yet
 cudaError_t launch_tc_pack(const double4 *jrec, long long nj, float eps2, const TcGeo *geo, unsigned char *dig,
                            float *mass, cudaStream_t st);
-// words: 2, zero before the first call and kept so; ok: the verdict
+// words: 2, zero before the first call and kept so; ok: the verdict; np: the
+// narrow path's preparation in the same launch (nic 0: none)
 cudaError_t launch_tc_prep(const double4 *xi, long long ni, float eps2, TcGeo *geo, unsigned char *idig,
-                           unsigned *words, int *ok, cudaStream_t st);
+                           unsigned *words, int *ok, const NarrowPrep &np, cudaStream_t st);
 cudaError_t launch_tc(const TcArgs &a, int grid, cudaStream_t st);
 cudaError_t launch_tc_combine(const TcArgs &a, int grid, int self, long long self_off, double *acc, double *pot,
                               cudaStream_t st);
@@ -414,10 +428,7 @@ cudaError_t launch_groups_finish(const GroupArgs &g, cudaStream_t st);
 // one device-side bounded wait that nothing ends (the timeout path's self-test)
 cudaError_t launch_wait_selftest(int *status, unsigned long long limit_ns, cudaStream_t st);
 cudaError_t launch_pack_hilo(const double4 *in, long long n, float4 *out, cudaStream_t st);
-// narrow path: chunk centres (chunks of `chunk` i, nic of them), double-float
-// i records and the two work counters zeroed, in one launch
-cudaError_t launch_narrow_prep(const double4 *xi, long long ni, long long chunk, long long nic,
-                              double4 *ctr, float4 *ihl, int *queue, cudaStream_t st);
+cudaError_t launch_narrow_prep(const double4 *xi, long long ni, const NarrowPrep &np, cudaStream_t st);
 // the batched kernel's j-tile depth and threads per CTA by default, and
 // whether (tj, nt) is compiled (every path: the default; plain Newton lists:
 // also 256 x 128, 1024 x 256 and 512 x 256)
@@ -600,7 +611,9 @@ cudaError_t tree_stage_records(int Bi, TreeScratch &t, SortScratch &sort, cudaSt
 
 // narrow all-pairs: part[k ni + i] for j chunks k = 0 .. nchunks - 1 (the
 // tile fields of c are unused)
-cudaError_t launch_group_partials_combine(const CombineArgs &c, int nchunks, cudaStream_t st);
+// tc: a run that the tensor-core kernel did (on tc_grid CTAs) if its verdict is nonzero
+cudaError_t launch_group_partials_combine(const CombineArgs &c, int nchunks, cudaStream_t st,
+                                          const TcArgs *tc = nullptr, int tc_grid = 0);
 cudaError_t launch_cell_build(const double4 *jrec, long long n, double box, int nc, int Bi,
                               double scale, CellScratch &s, SortScratch &sort, cudaStream_t st);
 cudaError_t launch_excl_scan(unsigned *a, long long n, unsigned *sums, cudaStream_t st);

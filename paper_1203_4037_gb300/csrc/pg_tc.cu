@@ -17,7 +17,7 @@
 // a second adds the lower 24 bits' difference, rounded by the tensor core at
 // the last place of the result: d carries one rounding relative to |d|,
 // however far the i-particles are spread (measured: mean -3.2e-8, at most
-// 1.5e-7 relative, against 64 bits). The sums take that mean back (kShort):
+// 1.5e-7 relative, against 64 bits). The sums take that mean back (kTcShort):
 // forces and potentials are then nearer to 64 bits than the double-float
 // kernel's (1048 i, 563704 j: 4.8e-8 and 2.3e-8 against 5.8e-8 and 2.5e-8).
 //
@@ -54,16 +54,11 @@ constexpr int kDigBytes = kTcJ * 32;   // digits of a j tile
 constexpr int kSlotBytes = kDigBytes + kTcJ * 4;   // and its masses
 constexpr int kSums = 4 * kIW, kLaneSums = kSums / 32;
 constexpr int kFoldTiles = 128;        // j tiles per FP32 partial sum of a lane
-// The differences come out short by this on average (the tensor cores round
-// them toward zero), so the unit they are read in is longer by it. From the
-// signed errors of forces (2 kShort) and potentials (kShort) against 64
-// bits, 12 sets of 112 to 2080 i against 3e5 to 1e6 j: +4.7e-8 and +2.6e-8
-// without it
-constexpr double kShort = 2.5e-8;
 
 // two groups of kIW i per CTA tile; the groups' warps (four each, one per
 // TMEM quadrant) share every j tile
-constexpr int kBi = 2 * kIW;
+constexpr int kBi = kTcBi;
+static_assert(kTcBi == 2 * kIW, "two groups");
 constexpr int kN = 3 * kBi;            // MMA N: (group, axis, i)
 constexpr int kStages = 2;             // TMEM stages of kN columns
 constexpr int kSlots = 8;              // staged j tiles
@@ -135,11 +130,6 @@ __device__ __forceinline__ void copy_in(uint32_t dst, const void *src, unsigned 
 {
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                  ::"r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
-}
-
-__host__ __device__ __forceinline__ long long tc_owner(long long u, long long grid, long long W)
-{
-    return ((u + 1) * grid - 1) / W;
 }
 
 // ---------------------------------------------------------------- the kernel
@@ -399,9 +389,14 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tc(const __grid_constant__ Tc
 // ---------------------------------------------------------------- digits
 // a coordinate's four digits as FP16, lower digit 1 scaled by 2^-11 (its
 // place value 2^-24 is below FP16's normal range)
-__device__ __forceinline__ void digits(double x, double c, double scale, __half *h)
+// (x scale is exact, a power of two, so y is (x - c) scale, rounded once, with
+// cs = c scale; adding 1.5 2^52 rounds it to an integer, the low bits of the
+// sum. The packing of 2^20 records takes 21 us; a subtraction, a product and
+// a conversion to 64-bit integers a coordinate took 25.)
+__device__ __forceinline__ void digits(double x, double cs, double scale, __half *h)
 {
-    const long long X = __double2ll_rn((x - c) * scale);
+    const double y = fma(x, scale, -cs);
+    const long long X = __double_as_longlong(y + 0x1.8p52) - __double_as_longlong(0x1.8p52);
     const long long hi = (X + (1ll << 23)) >> 24, lo = X - (hi << 24);
     const int h0 = (int)((hi + 2048) >> 12), h1 = (int)(hi - ((long long)h0 << 12));
     const int l0 = (int)((lo + 2048) >> 12), l1 = (int)(lo - ((long long)l0 << 12));
@@ -414,9 +409,9 @@ __device__ __forceinline__ void digits(double x, double c, double scale, __half 
 __device__ __forceinline__ void write_digits(const double4 v, const TcGeo &g, unsigned char *dig, long long k)
 {
     __align__(16) __half h[16];
-    digits(v.x, g.cx, g.scale, h);
-    digits(v.y, g.cy, g.scale, h + 4);
-    digits(v.z, g.cz, g.scale, h + 8);
+    digits(v.x, g.sx, g.scale, h);
+    digits(v.y, g.sy, g.scale, h + 4);
+    digits(v.z, g.sz, g.scale, h + 8);
     h[12] = __float2half_rn(4096.0f);
     h[13] = __float2half_rn(1.0f);
     h[14] = __float2half_rn(1.0f / 4096.0f);
@@ -431,6 +426,8 @@ __device__ __forceinline__ u64 ord64(double v)
     const u64 b = (u64)__double_as_longlong(v);
     return (b >> 63) ? ~b : (b | 0x8000000000000000ull);
 }
+// (on the integer pipe: a comparison in FP64 takes a warp 16 clocks of the SM)
+__device__ __forceinline__ bool finite64(double v) { return (__double2hiint(v) & 0x7ff00000) != 0x7ff00000; }
 __device__ __forceinline__ double unord64(u64 u)
 {
     return __longlong_as_double((long long)((u >> 63) ? (u & 0x7fffffffffffffffull) : ~u));
@@ -440,24 +437,44 @@ __device__ __forceinline__ double unord64(u64 u)
 // finish sets the geometry and clears the words for the next call. words: 3
 // minima (stored inverted, so that zero starts them all), 3 maxima, largest
 // |m| (as bits, all ones with a non-finite value), smallest nonzero |m|
-// (inverted bits), ticket. seen (may be null): the host's copy.
-__global__ void __launch_bounds__(256) k_tc_box(const double4 *__restrict__ jrec, long long nj, u64 *words,
-                                                TcGeo *geo, TcSeen *seen, long long gen)
+// (inverted bits), ticket. seen (may be null): the host's copy. PACK: from
+// the caller's arrays, with the records written as k_pack_j writes them.
+// Bound: the latency of the records; kBoxRec of them in flight a thread, at
+// most kBoxBlocks blocks at the words. 2^20 from the caller's arrays: 18 us,
+// k_pack_j alone 11 (tests of isfinite, comparisons in FP64, made it 33).
+constexpr int kBoxRec = 2;
+constexpr long long kBoxBlocks = 608;
+template <bool PACK>
+__global__ void __launch_bounds__(256) k_tc_box(const double *__restrict__ x, const double *__restrict__ m,
+                                                double4 *__restrict__ jrec, long long nj, u64 *words, TcGeo *geo,
+                                                TcSeen *seen, long long gen)
 {
     __shared__ u64 sh[8][8];
     u64 v[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    for (long long k = blockIdx.x * 256ll + threadIdx.x; k < nj; k += gridDim.x * 256ll) {
-        const double4 r = jrec[k];
-        const u64 o[3] = {ord64(r.x), ord64(r.y), ord64(r.z)};
+    const long long stride = gridDim.x * 256ll;
+    for (long long k0 = blockIdx.x * 256ll + threadIdx.x; k0 < nj; k0 += kBoxRec * stride) {
+        double4 rec[kBoxRec];
 #pragma unroll
-        for (int d = 0; d < 3; ++d) {
-            v[d] = max(v[d], ~o[d]);
-            v[3 + d] = max(v[3 + d], o[d]);
+        for (int q = 0; q < kBoxRec; ++q) {
+            const long long k = k0 + q * stride;
+            if (k < nj) rec[q] = PACK ? make_double4(x[3 * k], x[3 * k + 1], x[3 * k + 2], m[k]) : jrec[k];
         }
-        const bool fin = isfinite(r.x) && isfinite(r.y) && isfinite(r.z) && isfinite(r.w);
-        const u64 mb = (u64)__double_as_longlong(fabs(r.w));
-        v[6] = max(v[6], fin ? mb : ~0ull);
-        v[7] = max(v[7], mb ? ~mb : 0ull);
+#pragma unroll
+        for (int q = 0; q < kBoxRec; ++q) {
+            const long long k = k0 + q * stride;
+            if (k >= nj) break;
+            const double4 r = rec[q];
+            if (PACK) jrec[k] = r;
+            const u64 o[3] = {ord64(r.x), ord64(r.y), ord64(r.z)};
+#pragma unroll
+            for (int d = 0; d < 3; ++d) {
+                v[d] = max(v[d], ~o[d]);
+                v[3 + d] = max(v[3 + d], o[d]);
+            }
+            const u64 mb = (u64)__double_as_longlong(r.w) & ~(1ull << 63);
+            v[6] = max(v[6], finite64(r.x) && finite64(r.y) && finite64(r.z) && finite64(r.w) ? mb : ~0ull);
+            v[7] = max(v[7], mb ? ~mb : 0ull);
+        }
     }
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
 #pragma unroll
@@ -469,7 +486,7 @@ __global__ void __launch_bounds__(256) k_tc_box(const double4 *__restrict__ jrec
     if (threadIdx.x < 8) {
         u64 m = 0;
         for (int q = 0; q < 8; ++q) m = max(m, sh[threadIdx.x][q]);
-        atomicMax(words + threadIdx.x, m);
+        if (m > __ldcg(words + threadIdx.x)) atomicMax(words + threadIdx.x, m);
         __threadfence();
     }
     __syncthreads();
@@ -492,11 +509,15 @@ __global__ void __launch_bounds__(256) k_tc_box(const double4 *__restrict__ jrec
         int e = half > 0.0 ? ilogb(1.25 * half) + 1 : 0;
         g.e = e;
         g.scale = ldexp(1.0, 47 - e);
+        g.sx = g.cx * g.scale;
+        g.sy = g.cy * g.scale;
+        g.sz = g.cz * g.scale;
         const int em = mb ? ilogb(__longlong_as_double((long long)mb)) : 0;
         g.mscale = ldexp(1.0, 20 - em);        // masses enter at most 2^21
         g.mexp = 20 - em;
         g.mmin = ms ? __longlong_as_double((long long)~ms) * g.mscale : 0.0;
-        g.ok = half < 1e300 && e > -900 && e < 900 && em > -900 && em < 900;
+        g.ok = half < 1e300 && e > -900 && e < 900 && em > -900 && em < 900 &&
+               fabs(g.sx) < 1e300 && fabs(g.sy) < 1e300 && fabs(g.sz) < 1e300;
     }
     *geo = g;
     for (int q = 0; q < kTcBoxWords; ++q) words[q] = 0;
@@ -529,31 +550,36 @@ __global__ void __launch_bounds__(256) k_tc_pack(const double4 *__restrict__ jre
 
 // The i-particles' digits, and whether this call can use them: the j-set and
 // eps fit and every i lies within the cube. The last block writes the verdict.
-__global__ void __launch_bounds__(256) k_tc_prep(const double4 *__restrict__ xi, long long ni, long long npad,
-                                                 float eps2, TcGeo *geo, unsigned char *__restrict__ idig,
-                                                 unsigned *words, int *ok)
+// The first tb blocks; those behind them prepare the narrow path.
+constexpr int kPrepThreads = kTcJ;
+static_assert(kPrepThreads == kNarrowPrepThreads, "one launch");
+__global__ void __launch_bounds__(kPrepThreads) k_tc_prep(const double4 *__restrict__ xi, long long ni, int tb,
+                                                          float eps2, TcGeo *geo, unsigned char *__restrict__ idig,
+                                                          unsigned *words, int *ok, NarrowPrep np)
 {
-    const long long k = blockIdx.x * 256ll + threadIdx.x;
+    if (blockIdx.x >= tb) {
+        narrow_prep_block(xi, ni, np, blockIdx.x - tb);
+        return;
+    }
+    const long long k = blockIdx.x * (long long)kPrepThreads + threadIdx.x;    // of whole tiles of kTcJ
     const TcGeo g = *geo;
     bool bad = false;
-    if (k < npad) {
-        double4 v = make_double4(g.cx, g.cy, g.cz, 0.0);
-        if (k < ni && g.ok) {
-            const double4 r = xi[k];
-            const double lim = ldexp(1.0, g.e) * (1.0 - 0x1p-20);
-            bad = !(fabs(r.x - g.cx) < lim && fabs(r.y - g.cy) < lim && fabs(r.z - g.cz) < lim);
-            if (!bad) v = r;
-        }
-        write_digits(v, g, idig, k);
+    double4 v = make_double4(g.cx, g.cy, g.cz, 0.0);
+    if (k < ni && g.ok) {
+        const double4 r = xi[k];
+        const double lim = ldexp(1.0, g.e) * (1.0 - 0x1p-20);
+        bad = !(fabs(r.x - g.cx) < lim && fabs(r.y - g.cy) < lim && fabs(r.z - g.cz) < lim);
+        if (!bad) v = r;
     }
+    write_digits(v, g, idig, k);
     if (__syncthreads_or(bad) && threadIdx.x == 0) atomicOr(words, 1u);
     if (threadIdx.x != 0) return;
     __threadfence();
-    if (atomicAdd(words + 1, 1u) != gridDim.x - 1) return;
+    if (atomicAdd(words + 1, 1u) != tb - 1) return;
     __threadfence();
     const bool far = __ldcg(words) != 0, fits = tc_fits(g.ok, g.e, g.mmin, eps2);
     // eps in units of the upper digits' last place, u = R 2^-23
-    geo->e2 = (float)(ldexp((double)eps2, 2 * (23 - g.e)) * ((1.0 - kShort) * (1.0 - kShort)));
+    geo->e2 = (float)(ldexp((double)eps2, 2 * (23 - g.e)) * ((1.0 - kTcShort) * (1.0 - kTcShort)));
     geo->packed = g.packed || fits;
     geo->hl = g.stood_in;
     geo->stood_in = g.stood_in || far || !fits;
@@ -561,40 +587,16 @@ __global__ void __launch_bounds__(256) k_tc_prep(const double4 *__restrict__ xi,
     words[0] = words[1] = 0;
 }
 
-// one warp per i: the partial sums of its tile over the CTAs, the own pair's
-// potential, the units
-__global__ void __launch_bounds__(256) k_tc_combine(TcArgs a, int Bi, int grid, int self, long long self_off,
+__global__ void __launch_bounds__(256) k_tc_combine(TcArgs a, int grid, int self, long long self_off,
                                                     double *__restrict__ acc, double *__restrict__ pot)
 {
     if (*a.ok == 0) return;
     const long long i = blockIdx.x * 8ll + (threadIdx.x >> 5);
-    const int lane = threadIdx.x & 31;
-    if (i >= a.ni) return;
-    const long long t = i / Bi, li = i % Bi;
-    const long long bf = tc_owner(t * a.njt, grid, a.W), bl = tc_owner((t + 1) * a.njt - 1, grid, a.W);
-    double s[4] = {0, 0, 0, 0};
-    for (long long k = lane; k <= bl - bf; k += 32) {
-        const double4 v = a.part[((size_t)t * a.slots + k) * Bi + li];
-        s[0] += v.x; s[1] += v.y; s[2] += v.z; s[3] += v.w;
-    }
-#pragma unroll
-    for (int q = 0; q < 4; ++q)
-        for (int o = 16; o; o >>= 1) s[q] += __shfl_xor_sync(0xffffffffu, s[q], o);
-    if (lane != 0) return;
-    const TcGeo &g = *a.geo;
-    // the own pair as the loop added it: d = 0 exactly
-    if (self) s[3] += (double)__fmul_rn(a.mass[i + self_off], rsq(g.e2));
-    const double fa = ldexp((1.0 - kShort) * (1.0 - kShort), 2 * (23 - g.e) - g.mexp),
-                 fp = ldexp(1.0 - kShort, 23 - g.e - g.mexp);
-    acc[3 * i] = s[0] * fa;
-    acc[3 * i + 1] = s[1] * fa;
-    acc[3 * i + 2] = s[2] * fa;
-    if (pot) pot[i] = s[3] * fp;
+    if (i < a.ni) tc_combine_one(a, grid, self, self_off, acc, pot, i);
 }
 
 }  // namespace
 
-int tc_bi() { return kBi; }
 size_t tc_dig_bytes(long long n) { return (size_t)((n + kTcJ - 1) / kTcJ) * kDigBytes; }
 int tc_jtiles(long long nj) { return (int)((nj + kTcJ - 1) / kTcJ); }
 int tc_slots(long long ntiles, int njt, long long W, int grid)
@@ -605,11 +607,25 @@ int tc_slots(long long ntiles, int njt, long long W, int grid)
     return s;
 }
 
+static unsigned box_blocks(long long nj)
+{
+    return (unsigned)std::min<long long>((nj + 256 * kBoxRec - 1) / (256 * kBoxRec), kBoxBlocks);
+}
+
 cudaError_t launch_tc_box(const double4 *jrec, long long nj, unsigned long long *words, TcGeo *geo, TcSeen *seen,
                           long long gen, cudaStream_t st)
 {
     if (nj <= 0) return cudaErrorInvalidValue;
-    k_tc_box<<<(unsigned)std::min<long long>((nj + 255) / 256, 608), 256, 0, st>>>(jrec, nj, words, geo, seen, gen);
+    k_tc_box<false><<<box_blocks(nj), 256, 0, st>>>(nullptr, nullptr, const_cast<double4 *>(jrec), nj, words, geo, seen,
+                                                    gen);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_tc_pack_box(const double *x, const double *m, double4 *jrec, long long nj, unsigned long long *words,
+                               TcGeo *geo, TcSeen *seen, long long gen, cudaStream_t st)
+{
+    if (nj <= 0) return cudaErrorInvalidValue;
+    k_tc_box<true><<<box_blocks(nj), 256, 0, st>>>(x, m, jrec, nj, words, geo, seen, gen);
     return cudaGetLastError();
 }
 
@@ -624,11 +640,12 @@ cudaError_t launch_tc_pack(const double4 *jrec, long long nj, float eps2, const 
 }
 
 cudaError_t launch_tc_prep(const double4 *xi, long long ni, float eps2, TcGeo *geo, unsigned char *idig,
-                           unsigned *words, int *ok, cudaStream_t st)
+                           unsigned *words, int *ok, const NarrowPrep &np, cudaStream_t st)
 {
     if (ni <= 0) return cudaErrorInvalidValue;
-    const long long npad = (ni + kTcJ - 1) / kTcJ * kTcJ;
-    k_tc_prep<<<(unsigned)((npad + 255) / 256), 256, 0, st>>>(xi, ni, npad, eps2, geo, idig, words, ok);
+    const int tb = tc_jtiles(ni);
+    const long long nb = tb + (np.nic > 0 ? narrow_prep_blocks(ni, np) : 0);
+    k_tc_prep<<<(unsigned)nb, kPrepThreads, 0, st>>>(xi, ni, tb, eps2, geo, idig, words, ok, np);
     return cudaGetLastError();
 }
 
@@ -647,7 +664,7 @@ cudaError_t launch_tc(const TcArgs &a, int grid, cudaStream_t st)
 cudaError_t launch_tc_combine(const TcArgs &a, int grid, int self, long long self_off, double *acc, double *pot,
                               cudaStream_t st)
 {
-    k_tc_combine<<<(unsigned)((a.ni + 7) / 8), 256, 0, st>>>(a, kBi, grid, self, self_off, acc, pot);
+    k_tc_combine<<<(unsigned)((a.ni + 7) / 8), 256, 0, st>>>(a, grid, self, self_off, acc, pot);
     return cudaGetLastError();
 }
 

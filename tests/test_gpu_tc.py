@@ -272,3 +272,22 @@ def test_stand_in_after_other_paths(pg, orc):
         stand_in(60000)
         stand_in(80000)
         stand_in(60000)
+
+
+@pytest.mark.parametrize("ni", [64, 300])
+def test_new_j_records_cost_two_launches_more(pg, ni):
+    # a run on new records: their digits and the tensor cores' kernel beside the narrow path's launches
+    xj, mj = gen.plummer(349526, 3)
+    xi = gen.plummer(ni, 4)[0]
+    n = []
+    for path in (pg.PG_PATH_AUTO, pg.PG_PATH_NARROW):
+        with pg.Context(0) as c:
+            c.set_allpairs_path(path)
+            c.set_eps(EPS)
+            for _ in range(2):
+                c.set_j(xj, mj)
+                c.set_i(xi)
+                c.run()
+                a, p = c.get_force(ni)
+            n.append(c.info()["launches"])
+    assert n[0] <= n[1] + 2
