@@ -454,7 +454,9 @@ int pg_set_split(pg_ctx *ctx, int items_per_warp);
 /* Path of the all-pairs force loop (no groups, no periodic box); both give
  * the same sums up to FP32 rounding order. PG_PATH_TILED gives every CTA a
  * tile of i-particles in registers and a share of the j records, combining
- * the shares in FP64. PG_PATH_NARROW serves the individual time step regime
+ * the shares in FP64; in PG_TABLE mode with 16384 or more i-particles (their
+ * tiles are then compact) a tile takes only the j-particles within r_cut of
+ * its box, unless those are most of them. PG_PATH_NARROW serves the individual time step regime
  * (Section 5: a step evaluates only the particles due for an update, often
  * tens to hundreds against all N): the i-set is cut into chunks and the j
  * records into chunks of equal length, every (i chunk, j chunk) pair is one
@@ -481,13 +483,17 @@ int pg_set_timing(pg_ctx *ctx, int on);
  * waits for that kernel's end event). */
 int pg_kernel_time(pg_ctx *ctx, double *ms);
 
-/* Counters: out[0] pair evaluations enqueued by the last run, out[1] kernel
- * launches of the last run, out[2] i per thread, out[3] grid size of the
+/* Counters: out[0] pair evaluations enqueued by the last run (tabulated runs
+ * on Morton-ordered i, which leave out pairs beyond the cutoff: ni nj all
+ * the same), out[1] kernel
+ * launches of the last run, out[2] i per thread (48-bit fixed-point runs, see
+ * pg_set_differencing: the 64 i of a CTA's tile; their numbers are those of
+ * the enqueued run also where the device then takes double), out[3] grid size of the
  * force kernel, out[4] partial slots per tile, out[5] 1 if the pair arithmetic
  * is packed FP32x2, out[6] items per warp of a narrow run (0 for other paths),
  * out[7] 1 if the pair differences were formed in double-float (FP32 offset
  * plus its FP32 residual: the narrow path, and tiled runs whose i-tiles are
- * not compact), 0 if from one FP32 offset per particle, out[8] and out[9]
+ * not compact) or fixed point, 0 if from one FP32 offset per particle, out[8] and out[9]
  * the j-tile depth and threads per CTA of the batched kernel (0 when the run
  * did not use it).
  * Returns how many were written (at most 10). */

@@ -2096,10 +2096,11 @@ int enqueue_tc(pg_ctx *c, double *acc, double *pot)
     c->timed = c->timing;
     c->last_np = t.Bi / 2;
     c->last_df = true;
-    c->last_split = 1;
+    c->last_split = 0;
+    c->last_tj = c->last_nt = 0;
     c->last_pairs = ni * nj;
     c->last_grid = t.grid;
-    c->last_slots = std::max(t.slots, 2);
+    c->last_slots = t.slots;
     return PG_OK;
 }
 

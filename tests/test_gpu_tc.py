@@ -291,3 +291,19 @@ def test_new_j_records_cost_two_launches_more(pg, ni):
                 a, p = c.get_force(ni)
             n.append(c.info()["launches"])
     assert n[0] <= n[1] + 2
+
+
+def test_info_of_a_run(pg):
+    xj, mj = gen.plummer(60000, 3)
+    _, _, info = run(pg, gen.plummer(300, 4)[0], xj, mj, EPS)
+    # neither narrow items nor the batched kernel
+    assert info["split"] == 0 and info["j_tile"] == 0 and info["block_threads"] == 0
+    # the CTAs that share a tile of 64 i, in equal ranges of the (i tile, tile of 128 j) units
+    njt = -(-60000 // 128)
+    W = 5 * njt
+
+    def owner(u):
+        return ((u + 1) * info["grid"] - 1) // W
+
+    assert info["slots"] == max(owner((t + 1) * njt - 1) - owner(t * njt) + 1 for t in range(5))
+    assert info["pairs"] == 300 * 60000
