@@ -1482,6 +1482,26 @@ int near_unit(int ntiles, long long nj, int grid)
     return unit;
 }
 
+// The memory of a near-pair run beside the all-pairs run's. PG_ENOMEM: there is
+// no room, and the all-pairs kernel runs alone (c->part may then be gone). A
+// capture allocates nothing: it records what the run before it did.
+int near_room(pg_ctx *c, int ntiles, long long nj, int Bi, int grid)
+{
+    const struct {
+        DevBuf *b;
+        size_t bytes;
+    } need[] = {{&c->j_f32, (size_t)nj * sizeof(float4)},
+                {&c->t_cost, (size_t)ntiles * (sizeof(unsigned long long) + sizeof(unsigned))},
+                {&c->t_dense, (size_t)ntiles},
+                {&c->t_start, (size_t)(grid + 2) * sizeof(long long)},
+                {&c->part, ((size_t)ntiles + grid) * Bi * sizeof(double4)}};
+    for (const auto &n : need) {
+        const int rc = !c->capturing ? ensure(c, *n.b, n.bytes) : n.b->cap >= n.bytes ? PG_OK : PG_ENOMEM;
+        if (rc) return rc;
+    }
+    return PG_OK;
+}
+
 // the table's near-pair runs (pg_near.cu): the FP32 j records, the tiles'
 // extents (in t_ext already) and the split of the units by cost
 int near_args(pg_ctx *c, NearArgs &a, const double4 *xt, const double4 *jrec, long long ni, long long nj, int Bi,
@@ -1490,11 +1510,6 @@ int near_args(pg_ctx *c, NearArgs &a, const double4 *xt, const double4 *jrec, lo
     int rc;
     const int ntiles = (int)((ni + Bi - 1) / Bi);
     a.unit = near_unit(ntiles, nj, grid);
-    if ((rc = ensure(c, c->j_f32, (size_t)nj * sizeof(float4))) ||
-        (rc = ensure(c, c->t_cost, (size_t)ntiles * (sizeof(unsigned long long) + sizeof(unsigned)))) || (rc = ensure(c, c->t_dense, ntiles)) ||
-        (rc = ensure(c, c->t_start, (size_t)(grid + 2) * sizeof(long long))) ||
-        (rc = ensure(c, c->part, ((size_t)ntiles + grid) * Bi * sizeof(double4))))
-        return rc;
     a.tab = table_dev(c);
     PG_CUDA(c, launch_pack_f32(jrec, a.jw, nj, (const double4 *)c->ctr.p, a.tab.scale, (float4 *)c->j_f32.p,
                                c->stream));
@@ -1535,13 +1550,17 @@ int enqueue_allpairs(pg_ctx *c, const Plan &p, double *acc, double *pot)
     }
     if (p.ni == 0) return PG_OK;
     const bool ext = use_ext(c);
-    const bool near = cull && p.nj > 0;
+    bool near = cull && p.nj > 0;
     NearArgs na{};
     int ngrid = 0;
-    if ((rc = ensure(c, c->part, (size_t)p.ntiles * p.slots * p.Bi * sizeof(double4)))) return rc;
     if (near) {
         const int occ = near_max_blocks_per_sm(p.np, tab_units(c), ext, p.df);
         ngrid = c->sms * (c->ctas_per_sm > 0 ? std::min(c->ctas_per_sm, occ) : occ);
+        if ((rc = near_room(c, p.ntiles, p.nj, p.Bi, ngrid)) && rc != PG_ENOMEM) return rc;
+        near = rc == PG_OK;
+    }
+    if ((rc = ensure(c, c->part, (size_t)p.ntiles * p.slots * p.Bi * sizeof(double4)))) return rc;
+    if (near) {
         if ((rc = near_args(c, na, (const double4 *)c->xt.p, (const double4 *)c->jrec.p, p.ni, p.nj, p.Bi, 64 * p.np,
                             kNearPairCost * p.np, kNearTestCost, ngrid)))
             return rc;
@@ -2875,6 +2894,15 @@ int pg_backward_dev(pg_ctx *c, const double *w, double *dx, double *dm, float *d
         long long bl = stream_k_first((t + 1) * njsub - 1, grid, W);
         slots = std::max<int>(slots, (int)(bl - bf + 1));
     }
+    // a table on sorted tiles evaluates the near pairs
+    bool cull = table && n >= 16384;
+    int ngrid = 0;
+    if (cull) {
+        const int nocc = near_backward_max_blocks_per_sm(c->ntab);
+        ngrid = c->sms * (c->ctas_per_sm > 0 ? std::min(c->ctas_per_sm, nocc) : nocc);
+        if ((rc = near_room(c, ntiles, n, Bi, ngrid)) && rc != PG_ENOMEM) return rc;
+        cull = rc == PG_OK;
+    }
     if ((rc = ensure(c, c->xt, n * sizeof(double4))) || (rc = ensure(c, c->ctr, ntiles * sizeof(double4))) ||
         (rc = ensure(c, c->bw_wj, n * sizeof(double4))) || (rc = ensure(c, c->bw_wt, n * sizeof(double4))) ||
         (rc = ensure(c, c->part, (size_t)ntiles * slots * Bi * sizeof(double4))) ||
@@ -2902,7 +2930,6 @@ int pg_backward_dev(pg_ctx *c, const double *w, double *dx, double *dm, float *d
         c->last_launches += 3 + 1 + 4;
     }
     c->i_dirty = true;      // the tile buffers now hold the backward's order
-    const bool cull = table && n >= 16384;
     if (cull && (rc = ensure(c, c->t_ext, ntiles * sizeof(double4)))) return rc;
     PG_CUDA(c, launch_tile_prep((const double4 *)c->jrec.p, c->perm, n, Bi, (double4 *)c->xt.p,
                                 (double4 *)c->ctr.p, c->stream, cull ? (double4 *)c->t_ext.p : nullptr));
@@ -2931,8 +2958,6 @@ int pg_backward_dev(pg_ctx *c, const double *w, double *dx, double *dm, float *d
     NearArgs na{};
     NearCombine nc;
     if (cull) {
-        const int nocc = near_backward_max_blocks_per_sm(c->ntab);
-        const int ngrid = c->sms * (c->ctas_per_sm > 0 ? std::min(c->ctas_per_sm, nocc) : nocc);
         na.wi = a.wv;
         na.jw = a.jwv;
         if ((rc = near_args(c, na, a.xi, a.jx, n, n, Bi, Bi / 4, kNearBackCost, kNearBackTestCost, ngrid))) return rc;

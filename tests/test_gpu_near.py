@@ -197,3 +197,29 @@ def test_nonfinite_weight_reaches_every_gradient(pg, orc, n, bad):
     a = AG.table_force(xt, mt, torch.tensor(v, device="cuda"), 0.1, E, F)
     dx, dm = torch.autograd.grad(a, (xt, mt), torch.tensor(w, device="cuda"))
     assert not torch.isfinite(dx).any() and not torch.isfinite(dm).any()
+
+
+def test_without_room_for_the_near_records(pg, orc):
+    # the FP32 j records (64 MiB) cannot be had: the all-pairs kernel runs alone
+    torch = pytest.importorskip("torch")
+    n, nj, r_cut = 16384, 1 << 22, 0.1
+    x, _ = gen.plummer(n, 51)
+    xj, mj = gen.plummer(nj, 52)
+    v, _, _ = table(orc, r_cut)
+    want = run(pg, x, xj, mj, v, r_cut, False)[0]
+    with pg.Context(0) as c:
+        c.set_mode(pg.PG_TABLE)
+        c.set_table_values(v, r_cut, E, F)
+        c.set_allpairs_path(pg.PG_PATH_TILED)
+        c.set_j(xj, mj)
+        c.set_i(x)
+        torch.cuda.empty_cache()
+        keep = torch.empty(torch.cuda.mem_get_info()[0] - (48 << 20), dtype=torch.uint8, device="cuda")
+        try:
+            c.run()
+            got = c.get_force(n)[0]
+        finally:
+            del keep
+            torch.cuda.empty_cache()
+    err = np.linalg.norm(got - want, axis=1)
+    assert np.max(err) <= 1e-5 * np.max(np.linalg.norm(want, axis=1))
