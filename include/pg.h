@@ -430,7 +430,7 @@ int pg_tune(pg_ctx *ctx);
  * the launch shape, split and path left to the library and eps > 0 from
  * pg_set_eps, it forms d from 48-bit fixed-point positions in the j-set's
  * cube instead (of half side R; the tensor cores take the differences, with
- * an error of 2^-23 of |d| and 2^-47 R at most); the device takes double where
+ * an error of at most 1.5e-7 |d|, and 2^-47 R from the positions); the device takes double where
  * the values do not fit that. pg_info's out[7] reports
  * what the last run used (1 for the fixed point too). Groups, tree lists and the cell list keep their
  * own forms. PG_EINVAL for another mode. */

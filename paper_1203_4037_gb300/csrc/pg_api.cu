@@ -479,6 +479,8 @@ int read_status(pg_ctx *c)
 }
 
 int prep_sort(pg_ctx *c, long long n);   // below, with the tree
+int sort_room(pg_ctx *c, long long n);
+int bbox_room(pg_ctx *c);
 int pack_j_hilo(pg_ctx *c, long long nj); // below, with the groups
 
 }  // namespace
@@ -1371,20 +1373,7 @@ int enqueue_tiles(pg_ctx *c, const Plan &p)
     bool do_sort = tiles_sorted(c, n);
     c->perm = nullptr;
     if (do_sort && n > 1) {
-        size_t hn = sort_hist_entries(n);
-        size_t nb = (hn + 4095) / 4096 + 1;
-        if ((rc = ensure(c, c->skeys0, n * 4)) || (rc = ensure(c, c->skeys1, n * 4)) ||
-            (rc = ensure(c, c->svals0, n * 4)) || (rc = ensure(c, c->svals1, n * 4)) ||
-            (rc = ensure(c, c->shist, hn * 4)) || (rc = ensure(c, c->ssums, nb * 4)) ||
-            (rc = ensure(c, c->sbbox, 6 * 8)))
-            return rc;
-        c->sort.keys[0] = (unsigned *)c->skeys0.p;
-        c->sort.keys[1] = (unsigned *)c->skeys1.p;
-        c->sort.vals[0] = (unsigned *)c->svals0.p;
-        c->sort.vals[1] = (unsigned *)c->svals1.p;
-        c->sort.hist = (unsigned *)c->shist.p;
-        c->sort.sums = (unsigned *)c->ssums.p;
-        c->sort.bbox = (unsigned long long *)c->sbbox.p;
+        if ((rc = sort_room(c, n)) || (rc = bbox_room(c))) return rc;
         PG_CUDA(c, launch_morton_sort((const double4 *)c->xi.p, n, c->sort, &c->perm, c->stream));
         c->last_launches += 3 + 1 + 4;
     }
@@ -1687,12 +1676,12 @@ int upload_group_items(pg_ctx *c)
     std::vector<GroupItem> items;
     std::vector<long long> cost;
     // A CTA takes an item at a time, so the longest item bounds the run: a
-    // group above half a CTA's share of the pairs (three CTAs an SM) is cut
-    // into chunks of Bi / 2, Bi / 4, ... i-particles, at least 64 (each chunk
-    // stages the j-list anew). Whole, 4000 groups of 16 to 512 i and 1024 to
-    // 16384 j took 2.37 ms with the SMs busy 77 % of it. Cut at 1, 1/2, 1/4
-    // and 1/8 of the share: 2.34, 2.04, 2.13, 2.21 ms; 1500 such groups 1.10,
-    // 0.84, 0.83 at 1, 1/2, 1/3; 500 groups 0.45 (0.61 in chunks of 128 or more).
+    // group above half a CTA's share of the pairs is cut into chunks of Bi / 2,
+    // Bi / 4, ... i-particles, at least 64 (each chunk stages the j-list anew).
+    // The share is that of three CTAs an SM, whatever shape runs. Cut at 1,
+    // 1/2, 1/4 and 1/8 of it, 4000 groups of 16 to 512 i and 1024 to 16384 j
+    // take 2.34, 2.04, 2.13, 2.21 ms (whole 2.37); 1500 such groups 1.10, 0.84,
+    // 0.83 at 1, 1/2, 1/3; 500 groups 0.45 (0.61 in chunks of 128 or more).
     double total = 0;
     for (long long g = 0; g < c->ngroups; ++g)
         total += (double)(c->h_ioff[g + 1] - c->h_ioff[g]) * (double)(c->h_joff[g + 1] - c->h_joff[g]);
@@ -2189,20 +2178,34 @@ int read_dev(pg_ctx *c, void *dst, const void *src, size_t bytes)
 }
 
 // the radix sort's scratch for n keys, in c->sort
-int prep_sort(pg_ctx *c, long long n)
+int sort_room(pg_ctx *c, long long n)
 {
-    const size_t hn = sort_hist_entries(n);
-    const size_t nb = (std::max<size_t>(hn, (size_t)n + 1) + 4095) / 4096 + 1;
     int rc;
     if ((rc = ensure(c, c->skeys0, n * 4)) || (rc = ensure(c, c->skeys1, n * 4)) ||
         (rc = ensure(c, c->svals0, n * 4)) || (rc = ensure(c, c->svals1, n * 4)) ||
-        (rc = ensure(c, c->shist, hn * 4)) || (rc = ensure(c, c->ssums, nb * 4)))
+        (rc = ensure(c, c->shist, sort_hist_entries(n) * 4)))
         return rc;
     c->sort.keys[0] = (unsigned *)c->skeys0.p;
     c->sort.keys[1] = (unsigned *)c->skeys1.p;
     c->sort.vals[0] = (unsigned *)c->svals0.p;
     c->sort.vals[1] = (unsigned *)c->svals1.p;
     c->sort.hist = (unsigned *)c->shist.p;
+    return PG_OK;
+}
+
+// the bounding box that Morton keys are taken in
+int bbox_room(pg_ctx *c)
+{
+    const int rc = ensure(c, c->sbbox, 6 * 8);
+    c->sort.bbox = (unsigned long long *)c->sbbox.p;
+    return rc;
+}
+
+// the sort's scratch and that of scans of up to n + 1 counts
+int prep_sort(pg_ctx *c, long long n)
+{
+    int rc;
+    if ((rc = sort_room(c, n)) || (rc = ensure(c, c->ssums, ((n + 1 + 4095) / 4096 + 1) * 4))) return rc;
     c->sort.sums = (unsigned *)c->ssums.p;
     return PG_OK;
 }
@@ -2561,8 +2564,7 @@ int enqueue_cells(pg_ctx *c, double *acc, double *pot)
     long long item_cap = ncell + n / Bi + 1;
     long long sn = std::max(n, item_cap);
     CellScratch &s = c->cells;
-    size_t hn = sort_hist_entries(sn);
-    size_t nb = (std::max<size_t>(hn, ncell + 1) + 4095) / 4096 + 1;
+    const size_t nb = (size_t)(ncell + 1 + 4095) / 4096 + 1;
     if ((rc = ensure(c, c->c_wrapped, n * 32)) || (rc = ensure(c, c->c_xs, n * 32)) ||
         (rc = ensure(c, c->c_xo, n * 16)) ||
         (rc = ensure(c, c->c_perm, n * 4)) || (rc = ensure(c, c->c_start, (ncell + 1) * 4)) ||
@@ -2571,9 +2573,7 @@ int enqueue_cells(pg_ctx *c, double *acc, double *pot)
         (rc = ensure(c, c->c_items_raw, item_cap * sizeof(GroupItem))) ||
         (rc = ensure(c, c->c_items, item_cap * sizeof(GroupItem))) ||
         (rc = ensure(c, c->c_pairs, 16)) ||
-        (rc = ensure(c, c->skeys0, sn * 4)) || (rc = ensure(c, c->skeys1, sn * 4)) ||
-        (rc = ensure(c, c->svals0, sn * 4)) || (rc = ensure(c, c->svals1, sn * 4)) ||
-        (rc = ensure(c, c->shist, hn * 4)) || (rc = ensure(c, c->ssums, nb * 4)) ||
+        (rc = sort_room(c, sn)) || (rc = ensure(c, c->ssums, nb * 4)) ||
         (rc = ensure(c, c->g_queue, 16)))
         return rc;
     if (n >= (1LL << 31)) return fail(c, PG_EINVAL, "too many particles for the cell path");
@@ -2590,11 +2590,6 @@ int enqueue_cells(pg_ctx *c, double *acc, double *pot)
     s.item_cap = item_cap;
     s.pairs = (unsigned long long *)c->c_pairs.p;
     s.ncta = (unsigned *)((char *)c->c_pairs.p + 8);
-    c->sort.keys[0] = (unsigned *)c->skeys0.p;
-    c->sort.keys[1] = (unsigned *)c->skeys1.p;
-    c->sort.vals[0] = (unsigned *)c->svals0.p;
-    c->sort.vals[1] = (unsigned *)c->svals1.p;
-    c->sort.hist = (unsigned *)c->shist.p;
     c->sort.sums = (unsigned *)c->ssums.p;
     PG_CUDA(c, launch_cell_build((const double4 *)c->jrec.p, n, c->box, nc, Bi, c->scale, s,
                                  c->sort, c->stream));
@@ -2912,20 +2907,7 @@ int pg_backward_dev(pg_ctx *c, const double *w, double *dx, double *dm, float *d
     // tile order: the Morton order of the particles when it pays
     c->perm = nullptr;
     if (n >= 16384) {
-        size_t hn = sort_hist_entries(n);
-        size_t nb = (hn + 4095) / 4096 + 1;
-        if ((rc = ensure(c, c->skeys0, n * 4)) || (rc = ensure(c, c->skeys1, n * 4)) ||
-            (rc = ensure(c, c->svals0, n * 4)) || (rc = ensure(c, c->svals1, n * 4)) ||
-            (rc = ensure(c, c->shist, hn * 4)) || (rc = ensure(c, c->ssums, nb * 4)) ||
-            (rc = ensure(c, c->sbbox, 6 * 8)))
-            return rc;
-        c->sort.keys[0] = (unsigned *)c->skeys0.p;
-        c->sort.keys[1] = (unsigned *)c->skeys1.p;
-        c->sort.vals[0] = (unsigned *)c->svals0.p;
-        c->sort.vals[1] = (unsigned *)c->svals1.p;
-        c->sort.hist = (unsigned *)c->shist.p;
-        c->sort.sums = (unsigned *)c->ssums.p;
-        c->sort.bbox = (unsigned long long *)c->sbbox.p;
+        if ((rc = sort_room(c, n)) || (rc = bbox_room(c))) return rc;
         PG_CUDA(c, launch_morton_sort((const double4 *)c->jrec.p, n, c->sort, &c->perm, c->stream));
         c->last_launches += 3 + 1 + 4;
     }

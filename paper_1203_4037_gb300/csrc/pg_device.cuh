@@ -197,7 +197,6 @@ __device__ __forceinline__ void bulk_g2s(void *dst, const void *src, unsigned by
         ::"r"(smem_u32(dst)), "l"(src), "r"(bytes), "r"(smem_u32(bar)) : "memory");
 }
 
-// ---------------------------------------------------------------- planned splits
 // ---------------------------------------------------------------- misc
 __device__ __forceinline__ double4 ldg_d4(const double4 *p)
 {
@@ -275,11 +274,11 @@ __device__ __forceinline__ void narrow_prep_block(const double4 *__restrict__ xi
 }
 
 // ---------------------------------------------------------------- tensor cores
-// The differences come out short by this on average (the tensor cores round
-// them toward zero), so the unit they are read in is longer by it. From the
-// signed errors of forces (2 kTcShort) and potentials (kTcShort) against 64
-// bits, 12 sets of 112 to 2080 i against 3e5 to 1e6 j: +4.7e-8 and +2.6e-8
-// without it
+// The differences come out short (the tensor cores round them toward zero),
+// so the unit they are read in is longer by this. Fitted to the signed errors
+// of forces (2 kTcShort) and potentials (kTcShort) against 64 bits, 12 sets
+// of 112 to 2080 i against 3e5 to 1e6 j: +4.7e-8 and +2.6e-8 without it. (The
+// differences themselves, all weighted alike, are 3.2e-8 short.)
 constexpr double kTcShort = 2.5e-8;
 
 __host__ __device__ __forceinline__ long long tc_owner(long long u, long long grid, long long W)
@@ -315,6 +314,7 @@ __device__ __forceinline__ void tc_combine_one(const TcArgs &a, int grid, int se
     if (pot) pot[i] = s[3] * fp;
 }
 
+// ---------------------------------------------------------------- near pairs
 // a loss weight that is not finite in FP32 (or nearly so)
 __device__ __forceinline__ bool odd_weight(const double4 w)
 {

@@ -1347,11 +1347,10 @@ cudaError_t tree_stage_moments(long long n, TreeScratch &t, cudaStream_t st)
     // the level) go to the one-block kernel. A node is about 50 FP64
     // operations, with second moments about 200, and one SM issues two a
     // clock: the line lies where a level's work on one SM takes as long as a
-    // launch of its own (about 10 us). With 2048 for both, the one-block
-    // kernel of a 300007-particle quadrupole tree took 185 us. The other
-    // coarse levels run in blocks of 64 nodes for the same reason: 2000 nodes
-    // in blocks of 256 leave the work to eight SMs (26 us a level; now 14).
-    // The call: 1678 -> 1555 us; 2^20 monopoles 2317 -> 2289 us.
+    // launch of its own, about 10 us (a line of 2048 nodes leaves the one-block
+    // kernel 185 us on 300007 particles with second moments, this one 50).
+    // The other levels run in blocks of 64 nodes, so that 2000 nodes fill 31
+    // SMs: 14 us a level, in blocks of 256 on eight SMs 26.
     const long long top = t.npseudo == 3 ? 128 : 512;
     int L0 = -1;
     while (L0 + 1 < kLevels - 1 && t.hint_runs[L0 + 1] <= top) ++L0;
