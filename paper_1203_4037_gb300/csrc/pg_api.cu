@@ -5,6 +5,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -162,7 +163,7 @@ struct pg_ctx {
     long long tc_n = -1, tc_box_n = -1, tc_gen = 0;
     double tc_eps = -1.0;
     bool tc_hot = false;          // the last run was one for the tensor cores
-    TcSeen *tc_seen = nullptr;    // page-locked
+    TcSeen *tc_seen = nullptr;    // page-locked, a slot of the process's page
     bool graph_tc = false;        // the captured run reads the j digits
     const int *skip = nullptr;    // set while the run's stand-in is enqueued: it runs where this word is zero
 
@@ -253,6 +254,46 @@ int ensure(pg_ctx *c, DevBuf &b, size_t bytes)
     return PG_OK;
 }
 
+// Page-locked words for the geometries that come back to the host: one page,
+// taken by the process's first tensor-core run (70 us) and kept until it
+// exits, a slot a context. A context that finds no slot asks the device on
+// every call.
+constexpr int kSeenSlots = 64;
+struct SeenPage {
+    std::mutex lock;
+    TcSeen *p = nullptr;
+    bool tried = false;
+    bool used[kSeenSlots] = {};
+} g_seen;
+
+TcSeen *take_seen()
+{
+    std::lock_guard<std::mutex> l(g_seen.lock);
+    if (!g_seen.tried) {
+        g_seen.tried = true;
+        if (cudaHostAlloc((void **)&g_seen.p, kSeenSlots * sizeof(TcSeen), cudaHostAllocPortable | cudaHostAllocMapped) !=
+            cudaSuccess) {
+            (void)cudaGetLastError();
+            g_seen.p = nullptr;
+        }
+    }
+    for (int k = 0; g_seen.p && k < kSeenSlots; ++k)
+        if (!g_seen.used[k]) {
+            g_seen.used[k] = true;
+            g_seen.p[k] = TcSeen{};
+            return g_seen.p + k;
+        }
+    return nullptr;
+}
+
+// after the context's last kernel
+void give_seen(TcSeen *s)
+{
+    if (!s) return;
+    std::lock_guard<std::mutex> l(g_seen.lock);
+    g_seen.used[s - g_seen.p] = false;
+}
+
 // the j records of the tensor-core path, or the double-float records that its
 // stand-in packed, are no longer what its geometry says
 void tc_stale(pg_ctx *c) { c->tc_n = c->tc_box_n = -1; }
@@ -267,8 +308,10 @@ TcGeo *tc_geometry(const pg_ctx *c)
 int ensure_jhl(pg_ctx *c, size_t bytes)
 {
     if (bytes <= c->g_jhl.cap) return PG_OK;
-    c->jhl_n = -1;
-    tc_stale(c);
+    if (c->g_jhl.cap) {
+        c->jhl_n = -1;
+        tc_stale(c);
+    }
     return ensure(c, c->g_jhl, bytes);
 }
 
@@ -545,7 +588,7 @@ void pg_destroy(pg_ctx *c)
                       &c->bw_wt, &c->bw_dv, &c->tickets, &c->t_ext, &c->j_f32, &c->t_cost, &c->t_dense, &c->t_start,
                       &c->tc_dig, &c->tc_geo};
     for (DevBuf *b : bufs) free_dev(*b);
-    if (c->tc_seen) cudaFreeHost(c->tc_seen);
+    give_seen(c->tc_seen);
     for (DevBuf &b : c->tb) free_dev(b);
     for (DevBuf *b : {&c->pm_rec, &c->pm_x, &c->pm_m, &c->pm_acc, &c->pm_pot}) free_dev(*b);
     pm_destroy(c->pm);
@@ -1841,12 +1884,15 @@ struct TcRun {
     unsigned char *idig;
     unsigned *words;       // the i flags
     int *ok;               // the verdict
+    size_t part;           // bytes of partial sums in c->part; the i digits lie behind them
     bool timing;
+    bool jhl_later;        // g_jhl is not there yet
 };
-int enqueue_tc_kernels(pg_ctx *c, const TcRun &r, const NarrowPrep &np);
+int enqueue_tc_kernels(pg_ctx *c, TcRun &r, const NarrowPrep &np);
+int tc_first_jhl(pg_ctx *c, const TcRun &r);
 
 // tc: the run stands in for a tensor-core run, whose launches go with it
-int enqueue_narrow(pg_ctx *c, double *acc, double *pot, const TcRun *tc = nullptr)
+int enqueue_narrow(pg_ctx *c, double *acc, double *pot, TcRun *tc = nullptr)
 {
     int rc;
     const long long ni = c->ni, nj = nj_of(c);
@@ -1891,9 +1937,12 @@ int enqueue_narrow(pg_ctx *c, double *acc, double *pot, const TcRun *tc = nullpt
         return fail(c, PG_EINVAL, "too many narrow items");
     const long long nitems = (long long)nic * nch;
     if ((rc = ensure(c, c->g_ctr, (size_t)nic * sizeof(double4))) || (rc = ensure(c, c->g_queue, 16)) ||
-        (rc = ensure(c, c->n_part, (size_t)nch * ni * sizeof(double4))) ||
-        (rc = ensure_jhl(c, (size_t)nj * 32)) || (rc = ensure(c, c->g_ihl, (size_t)ni * 32)))
+        (rc = ensure(c, c->g_ihl, (size_t)ni * 32)))
         return rc;
+    auto room = [&] {
+        const int e = ensure(c, c->n_part, (size_t)nch * ni * sizeof(double4));
+        return e ? e : ensure_jhl(c, (size_t)nj * 32);
+    };
     NarrowPrep prep;
     prep.chunk = Bi;
     prep.nic = nic;
@@ -1903,8 +1952,9 @@ int enqueue_narrow(pg_ctx *c, double *acc, double *pot, const TcRun *tc = nullpt
     c->ihl_n = ni;
     if (tc) {
         // (that kernel packs the stand-in's j records)
-        if ((rc = enqueue_tc_kernels(c, *tc, prep))) return rc;
+        if ((rc = enqueue_tc_kernels(c, *tc, prep)) || (rc = room()) || (rc = tc_first_jhl(c, *tc))) return rc;
     } else {
+        if ((rc = room())) return rc;
         PG_CUDA(c, launch_narrow_prep((const double4 *)c->xi.p, ni, prep, c->stream));
         c->last_launches += 1;
         if ((rc = pack_j_hilo(c, nj))) return rc;
@@ -2021,38 +2071,53 @@ TcShape tc_shape(const pg_ctx *c)
     return t;
 }
 
+// The run's memory (a capture allocates nothing, and records the path that the
+// run before it took). PG_ENOMEM: there is no room, and the double-float path
+// runs alone. Its buffers, which it needs either way, come behind the launch of
+// the tensor-core kernel, so that a first run allocates them while that runs.
 int tc_room(pg_ctx *c)
 {
     int rc;
     const TcShape t = tc_shape(c);
-    const size_t dig = tc_dig_bytes(nj_of(c)) + (size_t)t.njt * 128 * sizeof(float);
+    const long long nj = nj_of(c);
+    const size_t dig = tc_dig_bytes(nj) + (size_t)t.njt * 128 * sizeof(float);
     const size_t part = t.part + tc_dig_bytes(c->ni);
-    // a capture allocates nothing: it records the path the run before it took
-    if (c->capturing)
-        return c->tc_geo.cap && c->tc_dig.cap >= dig && c->part.cap >= part && c->g_jhl.cap >= (size_t)nj_of(c) * 32
-                   ? PG_OK : PG_ENOMEM;
+    if (c->capturing) {
+        c->graph_tc = c->tc_geo.cap && c->tc_dig.cap >= dig && c->part.cap >= part;
+        return c->graph_tc ? PG_OK : PG_ENOMEM;
+    }
     if (c->tc_geo.cap == 0) {
         if ((rc = ensure(c, c->tc_geo, (kTcBoxWords + 2) * 8 + sizeof(TcGeo)))) return rc;
         PG_CUDA(c, cudaMemsetAsync(c->tc_geo.p, 0, c->tc_geo.cap, c->stream));
-        if (cudaHostAlloc((void **)&c->tc_seen, sizeof(TcSeen), cudaHostAllocMapped) != cudaSuccess) {
-            (void)cudaGetLastError();
-            c->tc_seen = nullptr;       // then every call asks the device
-        } else {
-            *c->tc_seen = TcSeen{};
-        }
+        if (!c->tc_seen) c->tc_seen = take_seen();
     }
     if (dig > c->tc_dig.cap) tc_stale(c);
-    if ((rc = ensure(c, c->tc_dig, dig)) || (rc = ensure_jhl(c, (size_t)nj_of(c) * 32))) return rc;
-    return ensure(c, c->part, part);
+    if ((rc = ensure(c, c->tc_dig, dig)) || (rc = ensure(c, c->part, part)) ||
+        (c->g_jhl.cap && (rc = ensure_jhl(c, (size_t)nj * 32))))
+        return rc;
+    return pack_tc(c, nj);
 }
 
-int enqueue_tc_kernels(pg_ctx *c, const TcRun &r, const NarrowPrep &np)
+int enqueue_tc_kernels(pg_ctx *c, TcRun &r, const NarrowPrep &np)
 {
+    r.jhl_later = c->g_jhl.cap == 0;
+    r.a.jhl = r.jhl_later || (c->jhl_n == r.a.nj && !c->capturing) ? nullptr : (float4 *)c->g_jhl.p;
+    r.a.part = (double4 *)c->part.p;
+    r.a.idig = r.idig = (unsigned char *)c->part.p + r.part;
     PG_CUDA(c, launch_tc_prep((const double4 *)c->xi.p, r.a.ni, (float)(c->eps * c->eps), tc_geometry(c), r.idig,
                               r.words, r.ok, np, c->stream));
     if (r.timing) PG_CUDA(c, record_timing(c, c->tk0));
     PG_CUDA(c, launch_tc(r.a, r.grid, c->stream));
     c->last_launches += 2;
+    return PG_OK;
+}
+
+// the stand-in's j records where their buffer came behind the kernel that packs them
+int tc_first_jhl(pg_ctx *c, const TcRun &r)
+{
+    if (!r.jhl_later) return PG_OK;
+    PG_CUDA(c, launch_pack_hilo(r.a.jrec, r.a.nj, (float4 *)c->g_jhl.p, c->stream, r.ok));
+    c->last_launches += 1;
     return PG_OK;
 }
 
@@ -2064,27 +2129,22 @@ int enqueue_tc(pg_ctx *c, double *acc, double *pot)
     unsigned long long *words = (unsigned long long *)c->tc_geo.p;
     TcRun r{};
     r.grid = t.grid;
-    r.idig = (unsigned char *)c->part.p + t.part;
+    r.part = t.part;
     r.words = (unsigned *)(words + kTcBoxWords);
     r.ok = (int *)(words + kTcBoxWords + 1);
     r.timing = c->timing;
     TcArgs &a = r.a;
     a.dig = (const unsigned char *)c->tc_dig.p;
     a.mass = tc_mass(c, nj);
-    a.idig = r.idig;
     a.geo = tc_geometry(c);
     a.ok = r.ok;
     a.jrec = (const double4 *)c->jrec.p;
-    a.jhl = c->jhl_n == nj && !c->capturing ? nullptr : (float4 *)c->g_jhl.p;
     a.ni = ni;
     a.nj = nj;
     a.W = t.W;
     a.njt = t.njt;
     a.slots = t.slots;
-    a.part = (double4 *)c->part.p;
     a.status = (int *)c->status.p;
-    if (c->capturing) c->graph_tc = true;
-    else if ((rc = pack_tc(c, nj))) return rc;
     // where the values do not fit: the double-float path
     c->timing = false;
     if (use_narrow(c)) {
@@ -2094,8 +2154,10 @@ int enqueue_tc(pg_ctx *c, double *acc, double *pot)
         c->last_launches += 1;
         Plan p;
         plan_allpairs(c, p);
+        rc = e == cudaSuccess ? ensure_jhl(c, (size_t)nj * 32) : cuda_fail(c, e, "launch_tc_combine");
+        if (!rc) rc = tc_first_jhl(c, r);
         c->skip = r.ok;
-        rc = e == cudaSuccess ? enqueue_allpairs(c, p, acc, pot) : cuda_fail(c, e, "launch_tc_combine");
+        if (!rc) rc = enqueue_allpairs(c, p, acc, pot);
         c->skip = nullptr;
     }
     c->timing = r.timing;

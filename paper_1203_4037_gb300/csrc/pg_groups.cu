@@ -1319,17 +1319,18 @@ cudaError_t launch_group_partials_combine(const CombineArgs &c, int nchunks, cud
     return cudaGetLastError();
 }
 
-__global__ void k_pack_hilo(const double4 *__restrict__ in, long long n, float4 *__restrict__ out)
+__global__ void k_pack_hilo(const double4 *__restrict__ in, long long n, float4 *__restrict__ out,
+                            const int *__restrict__ skip)
 {
     long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (i >= n) return;
+    if (i >= n || (skip && *skip)) return;
     pack_hilo_one(in, i, out);
 }
 
-cudaError_t launch_pack_hilo(const double4 *in, long long n, float4 *out, cudaStream_t st)
+cudaError_t launch_pack_hilo(const double4 *in, long long n, float4 *out, cudaStream_t st, const int *skip)
 {
     if (n <= 0) return cudaSuccess;
-    k_pack_hilo<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(in, n, out);
+    k_pack_hilo<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(in, n, out, skip);
     return cudaGetLastError();
 }
 

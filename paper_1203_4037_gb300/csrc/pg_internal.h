@@ -427,7 +427,9 @@ cudaError_t launch_groups(const GroupArgs &g, int grid, int np, bool table, bool
 cudaError_t launch_groups_finish(const GroupArgs &g, cudaStream_t st);
 // one device-side bounded wait that nothing ends (the timeout path's self-test)
 cudaError_t launch_wait_selftest(int *status, unsigned long long limit_ns, cudaStream_t st);
-cudaError_t launch_pack_hilo(const double4 *in, long long n, float4 *out, cudaStream_t st);
+// skip: a nonzero word there leaves the records as they are
+cudaError_t launch_pack_hilo(const double4 *in, long long n, float4 *out, cudaStream_t st,
+                             const int *skip = nullptr);
 cudaError_t launch_narrow_prep(const double4 *xi, long long ni, const NarrowPrep &np, cudaStream_t st);
 // the batched kernel's j-tile depth and threads per CTA by default, and
 // whether (tj, nt) is compiled (every path: the default; plain Newton lists:

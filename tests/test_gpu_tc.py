@@ -307,3 +307,27 @@ def test_info_of_a_run(pg):
 
     assert info["slots"] == max(owner((t + 1) * njt - 1) - owner(t * njt) + 1 for t in range(5))
     assert info["pairs"] == 300 * 60000
+
+
+def test_more_contexts_than_words_for_their_geometry(pg):
+    # 64 contexts of a process can see their geometry; the others ask the
+    # device on every call, and closed contexts give their words back
+    xj, mj = gen.plummer(32769, 3)
+    far = xj.copy()
+    far[11] = [1e9, 0.0, 0.0]
+    xi = gen.plummer(512, 4)[0]
+    ref = [run(pg, xi, y, mj, EPS, path=pg.PG_PATH_NARROW) for y in (xj, far)]
+    for _ in range(2):
+        cs = [pg.Context(0) for _ in range(66)]
+        for k, c in enumerate(cs):
+            c.set_eps(EPS)
+            c.set_j(far if k % 2 else xj, mj)
+            c.set_i(xi)
+        for _ in range(2):
+            for k, c in enumerate(cs):
+                c.run()
+                a, p = c.get_force(512)
+                same = np.array_equal(a, ref[k % 2][0]) and np.array_equal(p, ref[k % 2][1])
+                assert same == bool(k % 2)
+        for c in cs:
+            c.close()
