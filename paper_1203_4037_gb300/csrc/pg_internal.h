@@ -304,7 +304,7 @@ struct TcSeen {
 // a j have force errors of 3.5e-6 median and 1.4e-5 at most; at 2^-22 R the
 // steps are 1/4 ulp of eps); above, the sums leave FP32's range. So do those
 // of masses too far below the largest: m / r^3 at the cube's diagonal is to
-// stay above 2^-110 (2^-75 of the largest mass at small eps). The same
+// stay above 2^-110 (2^-56 of the largest mass at small eps). The same
 // operations, rounded alike, on the device and on the host.
 __host__ __device__ inline bool tc_fits(int ok, int e, double mmin, float eps2)
 {

@@ -17,12 +17,14 @@
 //
 // Bound: the tests, about 12 instructions per (i-tile, j), and the latency
 // of a unit (copy, two barriers, list) and of a batch (gather, conversion,
-// barrier); the pair terms are a few per cent of n^2. Measured (kernel, Plummer
-// spheres, r_cut = 0.1 scale lengths, against the all-pairs kernels): forward
-// 2.72 -> 0.36 ms at 65536, 43.1 -> 2.7 ms at 262144; backward 5.96 -> 0.60 ms
-// and 94 -> 4.4 ms. With equal unit counts instead of the split by cost the
-// forward kernel took 0.56 ms (an earlier form), converting records in place
-// instead of from a list about 8000 clocks per 256 j.
+// barrier); the pair terms are a few per cent of n^2. Measured (kernels, one
+// Plummer sphere of 65536, r_cut = 0.1 scale lengths, against the all-pairs
+// kernels): forward 2.72 -> 0.36 ms, backward 5.96 -> 0.67 ms; how well the
+// sampled costs split the units depends on the set (262144, six spheres:
+// forward 2.0 to 3.7 ms, all pairs 43 ms). With equal unit counts instead of
+// the split by cost the forward kernel took 0.56 ms (an earlier form),
+// converting records in place instead of from a list about 8000 clocks per
+// 256 j.
 #include <type_traits>
 
 #include "pg_device.cuh"
