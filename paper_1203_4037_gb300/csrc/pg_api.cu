@@ -2239,10 +2239,13 @@ int read_dev(pg_ctx *c, void *dst, const void *src, size_t bytes)
     return PG_OK;
 }
 
-// the radix sort's scratch for n keys, in c->sort
+// The radix sort's scratch for n keys, in c->sort. The tile order of an earlier
+// run lies in it (c->perm), so every sort makes the next tiled run order its
+// i-particles anew.
 int sort_room(pg_ctx *c, long long n)
 {
     int rc;
+    c->i_dirty = true;
     if ((rc = ensure(c, c->skeys0, n * 4)) || (rc = ensure(c, c->skeys1, n * 4)) ||
         (rc = ensure(c, c->svals0, n * 4)) || (rc = ensure(c, c->svals1, n * 4)) ||
         (rc = ensure(c, c->shist, sort_hist_entries(n) * 4)))

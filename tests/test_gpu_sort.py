@@ -81,3 +81,33 @@ def test_more_cells_than_particles(pg, orc):
 def test_order_without_waiting(pg, n):
     with pg.Context(0) as c:
         c.selftest_sort(n)
+
+
+@pytest.mark.parametrize("other", ["tree", "mesh", "selftest"])
+def test_tiles_after_another_sort(pg, other):
+    # a tiled run keeps its order between calls in the sort's buffers; other
+    # sorts of the context (also larger ones, which move the buffers) use them
+    x, m = gen.plummer(20011, 77)
+    with pg.Context(0) as c:
+        c.set_eps(0.01)
+        c.set_self(True)
+        c.set_j(x, m)
+        c.set_i(x)
+        c.run()
+        a, p = c.get_force(len(x))
+        if other == "tree":
+            c.set_tree(0.75, 256, 8)
+            c.run()
+            c.set_tree(-1.0, 256, 8)
+        elif other == "mesh":
+            y, w = gen.clustered_box(100003, 5)
+            c.set_periodic(1.0)
+            c.set_pm(64, pg.PG_SPLIT_GAUSS, 1 / 64)
+            c.pm_forces(y, w)
+            c.set_pm(0, pg.PG_SPLIT_GAUSS, 1.0)
+            c.set_periodic(0.0)
+        else:
+            c.selftest_sort(1 << 20)
+        c.run()
+        a2, p2 = c.get_force(len(x))
+    assert np.array_equal(a, a2) and np.array_equal(p, p2)
